@@ -169,6 +169,13 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
   return r;
 }
 
+// 1 / d by the hardware reciprocal
+__device__ __forceinline__ float rcp_approx(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return r;
+}
+
 // The per-lattice constants collide_pair multiplies by, each broadcast to
 // both lanes of an F2; negations and doublings are folded in (exact in
 // FP32, so every source of them gives the same bits).
@@ -228,12 +235,13 @@ __device__ __forceinline__ void collide_pair(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2
   const F2 IS = P(PC_IS);
   const F2 rho_phys = SCALED ? rho_p * IS : rho_p;
   // -rho'/rho per lane by the hardware reciprocal (the sign folded into
-  // the numerator, which is exact)
+  // the numerator, which is exact): rho' * rcp(rho) without __fdividef's
+  // handling of denominators above 2^126, the same bits below
   const F2 den = P(PC_R0) + rho_phys;
   float rl, rh, dl, dh;
   f2split(rho_phys, rl, rh);
   f2split(den, dl, dh);
-  const F2 nc = f2(__fdividef(-rl, dl), __fdividef(-rh, dh));
+  const F2 nc = f2(-rl * rcp_approx(dl), -rh * rcp_approx(dh));
   F2 jxx = jx_p * jx_p, jyy = jy_p * jy_p, jxy = jx_p * jy_p;
   if (SCALED) {
     jxx = jxx * IS;
@@ -268,6 +276,129 @@ __device__ __forceinline__ void collide_pair(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2
   const F2 TWO = f2s(2.0f), NTWO = f2s(-2.0f);
   const F2 a = fma2(TWO, r4, r3);  // axis velocities: -r3 - 2 r4
   const F2 b = fma2(TWO, r3, r4);  // diagonals: 2 r3 + r4
+  f0 = fma2(f2s(-4.0f), r4 - r3, f0);
+  const F2 ax = a - r7, ay = a + r7;
+  f1 = f1 + fma2(TWO, r5, ax);
+  f3 = f3 + fma2(NTWO, r5, ax);
+  f2_ = f2_ + fma2(TWO, r6, ay);
+  f4 = f4 + fma2(NTWO, r6, ay);
+  const F2 bp = b + r5, bm = b - r5;
+  f5 = f5 - ((bp + r6) + r8);
+  f6 = f6 - ((bm + r6) - r8);
+  f7 = f7 - ((bm - r6) + r8);
+  f8 = f8 - ((bp - r6) - r8);
+}
+
+// The FP32 constants of collide_pair_hl: the high parts with their low parts
+// (collide_dev's PRECISE form), each broadcast to both lanes of a pair,
+// doublings and negations folded in (exact).
+enum HlConst {
+  HL_R0, HL_2JX, HL_2JY, HL_JX, HL_JY,               // rho0, 2 j0, j0
+  HL_NQ0H, HL_NQ0L, HL_ND0H, HL_ND0L, HL_NX0H, HL_NX0L,  // -|j0|^2, ...
+  HL_I2H, HL_I2L,                                    // 1 / rho0^2
+  HL_K3H, HL_K3L, HL_K4H, HL_K4L, HL_NK5H, HL_NK5L,  // rates / D
+  HL_NK6H, HL_NK6L, HL_K7H, HL_K7L, HL_K8H, HL_K8L,
+  HL_COUNT
+};
+
+__host__ __device__ __forceinline__ float hl_const(const DevParams &P, int c) {
+  switch (c) {
+    case HL_R0: return P.rho0;
+    case HL_2JX: return 2.0f * P.jx0;
+    case HL_2JY: return 2.0f * P.jy0;
+    case HL_JX: return P.jx0;
+    case HL_JY: return P.jy0;
+    case HL_NQ0H: return -P.q0h;
+    case HL_NQ0L: return -P.q0l;
+    case HL_ND0H: return -P.d0h;
+    case HL_ND0L: return -P.d0l;
+    case HL_NX0H: return -P.x0h;
+    case HL_NX0L: return -P.x0l;
+    case HL_I2H: return P.i2h;
+    case HL_I2L: return P.i2l;
+    case HL_K3H: return P.k3;
+    case HL_K3L: return P.l3;
+    case HL_K4H: return P.k4;
+    case HL_K4L: return P.l4;
+    case HL_NK5H: return -P.k5;
+    case HL_NK5L: return -P.l5;
+    case HL_NK6H: return -P.k6;
+    case HL_NK6L: return -P.l6;
+    case HL_K7H: return P.k7;
+    case HL_K7L: return P.l7;
+    case HL_K8H: return P.k8;
+    default: return P.l8;
+  }
+}
+
+// the broadcast pairs, as a kernel parameter or in shared memory
+struct HlPairs {
+  float2 c[HL_COUNT];
+  __device__ __forceinline__ F2 operator()(HlConst k) const { return f2(c[k].x, c[k].y); }
+};
+
+inline HlPairs hl_pairs(const DevParams &P) {
+  HlPairs H;
+  for (int k = 0; k < HL_COUNT; ++k) H.c[k].x = H.c[k].y = hl_const(P, k);
+  return H;
+}
+
+// a * (h + l), as mul_hl<true>
+__device__ __forceinline__ F2 mul_hl2(F2 a, F2 h, F2 l) { return fma2(a, h, a * l); }
+
+// collide_dev<true, false> (FP32 storage) for two nodes, one per lane: the
+// same operations in the same order, so each lane's result equals the scalar
+// form's bit for bit (its one product that the compiler contracts, the
+// -3 dJ of n3, is an explicit multiply-add here; products by powers of two
+// are exact either way).
+__device__ __forceinline__ void collide_pair_hl(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2 &f4, F2 &f5,
+                                                F2 &f6, F2 &f7, F2 &f8, const HlPairs &P) {
+  const F2 s13 = f1 + f3, s24 = f2_ + f4;
+  const F2 d13 = f1 - f3, d24 = f2_ - f4;
+  const F2 s57 = f5 + f7, s68 = f6 + f8;
+  const F2 d57 = f5 - f7, d68 = f6 - f8;
+  const F2 axis = s13 + s24;
+  const F2 diag = s57 + s68;
+  const F2 dxd = d57 - d68;
+  const F2 dyd = d57 + d68;
+  const F2 rho_p = (f0 + axis) + diag;
+  const F2 jx_p = d13 + dxd;
+  const F2 jy_p = d24 + dyd;
+
+  // -rho'/rho per lane (the sign folded into the numerator, exact)
+  const F2 R0 = P(HL_R0);
+  const F2 den = R0 + rho_p;
+  float rl, rh, dl, dh;
+  f2split(rho_p, rl, rh);
+  f2split(den, dl, dh);
+  const F2 nc = f2(-rl * rcp_approx(dl), -rh * rcp_approx(dh));
+  const F2 tx = fma2(P(HL_2JX), jx_p, jx_p * jx_p);
+  const F2 ty = fma2(P(HL_2JY), jy_p, jy_p * jy_p);
+  const F2 txy = fma2(P(HL_JX), jy_p, fma2(jx_p, P(HL_JY), jx_p * jy_p));
+  const F2 I2H = P(HL_I2H), I2L = P(HL_I2L);
+  const F2 nj = mul_hl2(fma2(R0, tx + ty, mul_hl2(rho_p, P(HL_NQ0H), P(HL_NQ0L))), I2H, I2L);
+  const F2 np = mul_hl2(fma2(R0, tx - ty, mul_hl2(rho_p, P(HL_ND0H), P(HL_ND0L))), I2H, I2L);
+  const F2 nx = mul_hl2(fma2(R0, txy, mul_hl2(rho_p, P(HL_NX0H), P(HL_NX0L))), I2H, I2L);
+  const F2 djsq = fma2(nj, nc, nj);
+  const F2 dpxx = fma2(np, nc, np);
+  const F2 dpxy = fma2(nx, nc, nx);
+
+  const F2 TWO = f2s(2.0f), NTWO = f2s(-2.0f);
+  const F2 n3 = fma2(f2s(-3.0f), djsq, fma2(f2s(4.0f), diag, fma2(NTWO, f0, axis)));
+  const F2 n4 = fma2(f2s(3.0f), djsq, f2s(3.0f) * (f0 - axis));
+  const F2 m5 = fma2(NTWO, dxd, d13);  // -n5, -n6: their rates come negated
+  const F2 m6 = fma2(NTWO, dyd, d24);
+  const F2 n7 = (s13 - s24) - dpxx;
+  const F2 n8 = (s57 - s68) - dpxy;
+  const F2 r3 = mul_hl2(n3, P(HL_K3H), P(HL_K3L));
+  const F2 r4 = mul_hl2(n4, P(HL_K4H), P(HL_K4L));
+  const F2 r5 = mul_hl2(m5, P(HL_NK5H), P(HL_NK5L));
+  const F2 r6 = mul_hl2(m6, P(HL_NK6H), P(HL_NK6L));
+  const F2 r7 = mul_hl2(n7, P(HL_K7H), P(HL_K7L));
+  const F2 r8 = mul_hl2(n8, P(HL_K8H), P(HL_K8L));
+
+  const F2 a = fma2(TWO, r4, r3);
+  const F2 b = fma2(TWO, r3, r4);
   f0 = fma2(f2s(-4.0f), r4 - r3, f0);
   const F2 ax = a - r7, ay = a + r7;
   f1 = f1 + fma2(TWO, r5, ax);

@@ -19,6 +19,7 @@
 
 #include "bounds.cuh"
 #include "lbm_internal.h"
+#include "plan.h"
 #include "runtime.h"
 
 namespace lbm {
@@ -233,28 +234,51 @@ static cudaError_t launch_one(lbm_ctx *h, int from, cudaStream_t st) {
   return launch_step_dev(h->L, src, dst, st, h->block, h->L.variant);
 }
 
-// capture `steps` (even) launches starting from buffer 0 into a graph
-static int capture_graph(lbm_ctx *h, int steps) {
-  free_graph(h);
+// one launch of `steps` steps (next_steps) from buffer `from` into the other
+static cudaError_t launch_some(lbm_ctx *h, int from, int steps, cudaStream_t st,
+                               const float *forced = nullptr) {
+  const void *src = h->L.buf[from];
+  void *dst = h->L.buf[from ^ 1];
+  if (h->L.plan == PLAN_TILE)
+    return launch_tile(h->L, src, dst, st, steps, forced, h->sx, h->sy);
+  return steps > 1 ? launch_rows(h->L, src, dst, st, steps) : launch_one(h, from, st);
+}
+
+// Captured launches: an even number (so a replay leaves the buffer parity),
+// about 64 steps
+static int graph_launches(const lbm_ctx *h) {
+  const int per = h->L.plan == PLAN_TILE ? h->L.tile.steps : (h->L.plan == PLAN_ROWS ? kRowSteps : 1);
+  return std::max(2, (64 / per + 1) & ~1);
+}
+
+// capture graph_launches(h) launches starting from buffer 0 into a graph;
+// forced: with the point source's table (PLAN_TILE)
+static int capture_graph(lbm_ctx *h, cudaGraphExec_t *out, int *steps, bool forced) {
   cudaStream_t cs;
   CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+  int done = 0;
   if (e == cudaSuccess) {
-    for (int k = 0; k < steps && e == cudaSuccess; ++k) e = launch_one(h, k & 1, cs);
+    const int launches = graph_launches(h);
+    for (int k = 0; k < launches && e == cudaSuccess; ++k) {
+      const int n = next_steps(h->L, 1 << 20);
+      e = launch_some(h, k & 1, n, cs, forced ? h->src_tab32 + 9 * done : nullptr);
+      done += n;
+    }
     cudaError_t e2 = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = e2;
   }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&h->graph, g, 0);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
   if (g) cudaGraphDestroy(g);
   cudaStreamDestroy(cs);
   if (e != cudaSuccess) {
-    h->graph = nullptr;
+    *out = nullptr;
     set_error(std::string("graph capture: ") + cudaGetErrorString(e));
     cudaGetLastError();
     return LBM_ECUDA;
   }
-  h->graph_steps = steps;
+  *steps = done;
   return LBM_OK;
 }
 
@@ -601,6 +625,7 @@ int create_lattice(int nx, int ny, const double S[9], double rho0, const double 
   h->L.variant = default_variant(storage_dtype);
   h->L.esize = esize;
   h->L.cur = 0;
+  if (!halo) plan_lattice(h->L, sm_count());
   // Lallemand-Luo order (rho, e, eps, jx, qx, jy, qy, pxx, pxy) -> paper
   // order (rho, jx, jy, e, eps, qx, qy, pxx, pxy)
   const int ll_of_paper[9] = {0, 3, 5, 1, 2, 4, 6, 7, 8};
@@ -727,6 +752,61 @@ void advance_one(lbm_handle h) {
 }
 }  // namespace lbm
 
+// Forced steps in tiles: the stored populations of the source node for each
+// step of a replay are computed here as the forcing kernel computes them
+// (k_force_node: FP64 difference to the base, rounded to storage), uploaded
+// and read by the tile kernel in place of what the node pulls.
+static int step_forced_tile(lbm_ctx *h, long n) {
+  constexpr int kMax = 64 + 2 * kMaxTileSteps;
+  if (!h->src_tab32) {
+    h->src_tab32 = (float *)dev_alloc(sizeof(float) * 9 * kMax);
+    if (!h->src_tab32) {
+      set_error("out of device memory for the source table");
+      return LBM_ENOMEM;
+    }
+  }
+  if (h->src_graph && (h->src_gx != h->sx || h->src_gy != h->sy)) {
+    cudaGraphExecDestroy(h->src_graph);
+    h->src_graph = nullptr;
+  }
+  const double PI = 3.14159265358979323846;
+  while (n > 0) {
+    if (!h->src_graph && h->L.cur == 0 && n >= 64) {
+      int rc = capture_graph(h, &h->src_graph, &h->src_steps, true);
+      if (rc != LBM_OK) return rc;
+      h->src_gx = h->sx;
+      h->src_gy = h->sy;
+    }
+    const bool replay = h->src_graph && h->L.cur == 0 && n >= h->src_steps;
+    const int k = replay ? h->src_steps : next_steps(h->L, n);
+    float tab[9 * kMax];
+    for (int q = 0; q < k; ++q) {
+      double fs[9];
+      const double rho_t = h->rho0 + h->s_amp * sin(2.0 * PI * (double)(h->t + q) / h->s_period);
+      host_feq_j(rho_t, 0.0, 0.0, fs);
+      for (int i = 0; i < 9; ++i) {
+        const double d = fs[i] - h->f0[i];
+        float v = (float)d;
+        if (h->L.dtype == LBM_F16DEV) v = __half2float(__float2half_rn((float)(d * h->qscale)));
+        else if (h->L.dtype == LBM_BF16DEV) v = __bfloat162float(__float2bfloat16_rn((float)d));
+        tab[9 * q + i] = v;
+      }
+    }
+    // pageable source: the copy is staged before the call returns
+    CK(cudaMemcpyAsync(h->src_tab32, tab, sizeof(float) * 9 * k, cudaMemcpyHostToDevice,
+                       h->stream));
+    if (replay) {
+      CK(cudaGraphLaunch(h->src_graph, h->stream));
+    } else {
+      CK(launch_some(h, h->L.cur, k, h->stream, h->src_tab32));
+      h->L.cur ^= 1;
+    }
+    n -= k;
+    h->t += k;
+  }
+  return LBM_OK;
+}
+
 extern "C" {
 
 int lbm_create(int nx, int ny, const double S[9], double rho0, const double u0[2],
@@ -740,6 +820,7 @@ int lbm_destroy(lbm_handle h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   free_graph(h);
   dev_free(h->src_tab);
+  dev_free(h->src_tab32);
   dev_free(h->alloc[0]);
   dev_free(h->alloc[1]);
   dev_free(h->partials);
@@ -813,10 +894,12 @@ int lbm_step(lbm_handle h, long n) {
   REQUIRE(!h->slab || n <= 1, "a slab takes one step between halo exchanges");
   REQUIRE(h->batch == nullptr, "lattice is a batch member; step the batch");
   DevGuard g(h->device);
-  if (n > 0) {
+  // the launch variants belong to the single-step kernel
+  if (n > 0 && (h->L.plan == PLAN_SINGLE || n == 1 || (h->src_on && h->L.plan == PLAN_ROWS))) {
     int rc = maybe_autotune(h);
     if (rc != LBM_OK) return rc;
   }
+  if (h->src_on && h->L.plan == PLAN_TILE) return step_forced_tile(h, n);
   if (h->src_on) {
     // The forcing changes every step.  Runs of kSrcGraph steps from buffer 0
     // replay a captured graph after the host uploads that run's forcing
@@ -852,21 +935,23 @@ int lbm_step(lbm_handle h, long n) {
     }
     return LBM_OK;
   }
-  const int G = 64;  // steps per captured graph (even)
   while (n > 0) {
+    const int G = h->graph ? h->graph_steps : 64;
     if (h->L.cur == 0 && n >= G) {
-      if (!h->graph || h->graph_steps != G) {
-        int rc = capture_graph(h, G);
+      if (!h->graph) {
+        int rc = capture_graph(h, &h->graph, &h->graph_steps, false);
         if (rc != LBM_OK) return rc;
+        continue;
       }
       CK(cudaGraphLaunch(h->graph, h->stream));
       n -= G;
       h->t += G;
     } else {
-      CK(launch_one(h, h->L.cur, h->stream));
+      const int k = next_steps(h->L, n);
+      CK(launch_some(h, h->L.cur, k, h->stream));
       h->L.cur ^= 1;
-      n -= 1;
-      h->t += 1;
+      n -= k;
+      h->t += k;
     }
   }
   return LBM_OK;

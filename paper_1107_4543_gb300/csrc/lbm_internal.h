@@ -37,9 +37,34 @@ struct DevGuard {
   DevGuard &operator=(const DevGuard &) = delete;
 };
 
+// Work split of the kernels that advance several steps per launch
+// (step_multi.cuh; chosen in plan.h).
+// k_step_rows: strips of `width` chunks, tasks of `rows` rows of one strip
+struct RowsGeom {
+  int strips, width, rows;
+};
+// k_step_tile: tiles of bx x by nodes, at most `steps` steps per launch
+struct TileGeom {
+  int bx, by, ntx, nty, steps;
+};
+constexpr int kRowSteps = 3;       // steps per k_step_rows launch (2 for a remainder)
+constexpr int kTileCols = 64;      // columns of a tile with its halo: 32 lanes of 2 nodes
+constexpr int kTileThreads = 512;
+constexpr int kMaxTileSteps = 8;
+constexpr int kMaxSmem = 227 * 1024;  // shared memory of one block on sm_103
+__host__ __device__ constexpr int tile_halo_x(int steps) { return (steps + 1) & ~1; }
+// both step buffers of one tile
+inline size_t tile_bytes(int by, int steps, int esize) {
+  return (size_t)2 * 9 * (by + 2 * steps) * kTileCols * esize;
+}
+enum StepPlan { PLAN_SINGLE, PLAN_ROWS, PLAN_TILE };
+
 // Everything a step launch needs about one lattice.
 struct Lattice {
   Geom g;
+  StepPlan plan = PLAN_SINGLE;
+  RowsGeom rows = {};
+  TileGeom tile = {};
   int dtype;
   int V;             // nodes per vector (vec_nodes)
   int variant;       // launch variant of the step kernel (tuner)
@@ -193,6 +218,39 @@ inline cudaError_t launch_batch_resident(int dtype, const BatchEntry *ents, cons
   }
 }
 
+// step_multi.cuh: kRowSteps or 2 steps, and 1 .. L.tile.steps steps
+cudaError_t launch_rows_f32(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps);
+cudaError_t launch_rows_f16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps);
+cudaError_t launch_rows_bf16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                             int steps);
+cudaError_t launch_tile_f32(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps, const float *forced, int sx, int sy);
+cudaError_t launch_tile_f16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps, const float *forced, int sx, int sy);
+cudaError_t launch_tile_bf16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                             int steps, const float *forced, int sx, int sy);
+inline cudaError_t launch_rows(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                               int steps) {
+  switch (L.dtype) {
+    case LBM_F32DEV: return launch_rows_f32(L, src, dst, st, steps);
+    case LBM_F16DEV: return launch_rows_f16(L, src, dst, st, steps);
+    case LBM_BF16DEV: return launch_rows_bf16(L, src, dst, st, steps);
+    default: return cudaErrorInvalidValue;
+  }
+}
+// forced (may be null): the stored populations of node (sx, sy) before each
+// step's collision, 9 FP32 values per step in stored units (device memory)
+inline cudaError_t launch_tile(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                               int steps, const float *forced = nullptr, int sx = 0, int sy = 0) {
+  switch (L.dtype) {
+    case LBM_F32DEV: return launch_tile_f32(L, src, dst, st, steps, forced, sx, sy);
+    case LBM_F16DEV: return launch_tile_f16(L, src, dst, st, steps, forced, sx, sy);
+    case LBM_BF16DEV: return launch_tile_bf16(L, src, dst, st, steps, forced, sx, sy);
+    default: return cudaErrorInvalidValue;
+  }
+}
 // Nodes per vector of a storage type (host side of d2q9_pull.cuh's Elem).
 inline int vec_nodes(int dtype) {
   return dtype == LBM_F64 || dtype == LBM_F64DEV ? 2

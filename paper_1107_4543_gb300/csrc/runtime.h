@@ -42,6 +42,8 @@ struct lbm_ctx {
   // forced steps in graphs: kSrcGraph x (forced node from src_tab[k], step)
   cudaGraphExec_t src_graph = nullptr;
   double *src_tab = nullptr;  // 9 populations per captured step
+  float *src_tab32 = nullptr; // the same in stored units (tiles)
+  int src_steps = 0;          // steps of src_graph (tiles)
   int src_gx = -1, src_gy = -1;  // source node the graph was captured for
 };
 

@@ -1,6 +1,7 @@
 // Step kernels for one storage type (__nv_bfloat16); see step_impl.cuh.
 #define LBM_TABLE_PAIRS  // this unit holds its type's constant table
 #include "step_impl.cuh"
+#include "step_multi.cuh"
 
 namespace lbm {
 
@@ -23,6 +24,16 @@ cudaError_t launch_batch_resident_bf16(const BatchEntry *ents, const int *idx, i
                                       int nents, size_t smem, int parity, long steps,
                                       const int *limits, cudaStream_t st) {
   return launch_resident_t<__nv_bfloat16>(ents, idx, nres, nents, smem, parity, steps, limits, st);
+}
+
+cudaError_t launch_rows_bf16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps) {
+  return launch_rows_t<__nv_bfloat16>(L, src, dst, st, steps);
+}
+
+cudaError_t launch_tile_bf16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps, const float *forced, int sx, int sy) {
+  return launch_tile_t<__nv_bfloat16>(L, src, dst, st, steps, forced, sx, sy);
 }
 
 unsigned bounds_word_step_bf16(bool reset) { return bounds::read_word(reset); }

@@ -1,6 +1,7 @@
 // Step kernels for one storage type (float); see step_impl.cuh.
 #define LBM_TABLE_DEV  // this unit holds its type's constant table
 #include "step_impl.cuh"
+#include "step_multi.cuh"
 
 namespace lbm {
 
@@ -23,6 +24,16 @@ cudaError_t launch_batch_resident_f32(const BatchEntry *ents, const int *idx, in
                                       int nents, size_t smem, int parity, long steps,
                                       const int *limits, cudaStream_t st) {
   return launch_resident_t<float>(ents, idx, nres, nents, smem, parity, steps, limits, st);
+}
+
+cudaError_t launch_rows_f32(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps) {
+  return launch_rows_t<float>(L, src, dst, st, steps);
+}
+
+cudaError_t launch_tile_f32(const Lattice &L, const void *src, void *dst, cudaStream_t st,
+                            int steps, const float *forced, int sx, int sy) {
+  return launch_tile_t<float>(L, src, dst, st, steps, forced, sx, sy);
 }
 
 unsigned bounds_word_step_f32(bool reset) { return bounds::read_word(reset); }

@@ -1,0 +1,103 @@
+"""GPU checks of the kernels that advance several steps per launch
+(csrc/step_multi.cuh) against the single-step kernel: the same arithmetic
+with the same storage rounding between steps, so populations are equal bit
+for bit, at sizes where tiles, strips and the periodic wrap can go wrong."""
+import numpy as np
+import pytest
+
+import lbm_inputs as inp
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1107_4543_gb300 import build, lbm
+
+    build.build()
+    lbm.load()
+    return lbm
+
+
+RATES = inp.s_ll(inp.rates("OPT"))
+
+
+def noisy(nx, ny, seed):
+    """Random populations: every direction of every node differs."""
+    return inp.random_populations(nx, ny, seed, amp=1e-3)
+
+
+# one row, one column, around a pair, a chunk, a tile (44 .. 60 columns) and
+# several tiles; the storage type's single-step kernel runs in one slab
+TILE_SIZES = [(2, 2), (3, 2), (5, 3), (8, 2), (9, 7), (44, 5), (45, 40), (59, 8), (64, 64),
+              (65, 97), (101, 101), (131, 23), (512, 16), (300, 290)]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("nx,ny", TILE_SIZES)
+def test_tiles_equal_single_steps(L, nx, ny, dtype):
+    f = noisy(nx, ny, 3)
+    for steps in (1, 5, 67, 131):
+        h = L.lbm_create(nx, ny, RATES, 1.0, (0.05, -0.02), L.DTYPES[dtype])
+        s = L.lbm_slabs_create(nx, ny, RATES, 1.0, (0.05, -0.02), L.DTYPES[dtype], 1)
+        try:
+            L.lbm_set_populations(h, f)
+            L.lbm_slabs_set_populations(s, f)
+            L.lbm_step(h, steps)
+            L.lbm_slabs_step(s, steps)
+            assert np.array_equal(L.lbm_get_populations(h), L.lbm_slabs_get_populations(s, ny, nx))
+        finally:
+            L.lbm_destroy(h)
+            L.lbm_slabs_destroy(s)
+
+
+# rows of the least lattices the rows kernel takes: shorter than a chunk, one
+# and two strips, a partial last chunk of every kind, two rows
+ROW_SIZES = [("f32", nx, ny) for nx, ny in [(2, 700001), (3, 420001), (5, 260001), (9, 150001), (10, 130001),
+                                            (11, 120001), (109, 12001), (119, 10601),
+                                            (121, 10501), (242, 5203), (1203, 1101), (700001, 2),
+                                            (420003, 3)]]
+ROW_SIZES += [(d, nx, ny) for d in ("f16", "bf16")
+              for nx, ny in [(17, 190001), (22, 140001), (219, 14001), (239, 12601), (241, 12501), (1500001, 2), (4097, 737)]]
+
+
+@pytest.mark.parametrize("dtype,nx,ny", ROW_SIZES)
+def test_rows_equal_single_steps(L, dtype, nx, ny):
+    f = noisy(nx, ny, 5)
+    h = L.lbm_create(nx, ny, RATES, 1.0, (0.05, -0.02), L.DTYPES[dtype])
+    g = L.lbm_create(nx, ny, RATES, 1.0, (0.05, -0.02), L.DTYPES[dtype])
+    try:
+        for x in (h, g):
+            L.lbm_set_variant(x, 2)
+            L.lbm_set_populations(x, f)
+        for steps in (3, 7, 2, 4):
+            L.lbm_step(h, steps)
+            for _ in range(steps):
+                L.lbm_step(g, 1)  # the single-step kernel
+        a = L.lbm_get_populations(h)
+        assert np.array_equal(a, L.lbm_get_populations(g))
+    finally:
+        L.lbm_destroy(h)
+        L.lbm_destroy(g)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "bf16"])
+def test_forced_tiles_follow_the_single_forced_steps(L, dtype):
+    """A point source inside the tiles' halos: runs of many steps equal runs
+    of one step at a time, across replays and remainders."""
+    nx, ny = 53, 31
+    got = []
+    for chunks in ((140,), (1,) * 140, (3, 70, 67)):
+        h = L.lbm_create(nx, ny, RATES, 1.0, (0.0, 0.0), L.DTYPES[dtype])
+        try:
+            L.lbm_set_source(h, 52, 0, 0.01, 17.0)
+            L.lbm_init_field(h, *inp.gaussian_pulse(nx, ny, 1e-3, 4.0))
+            for n in chunks:
+                L.lbm_step(h, n)
+            got.append(L.lbm_get_populations(h))
+        finally:
+            L.lbm_destroy(h)
+    assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
