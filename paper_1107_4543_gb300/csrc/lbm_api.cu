@@ -230,7 +230,7 @@ int lbm::tune_reps(double bytes) {
 static cudaError_t launch_one(lbm_ctx *h, int from, cudaStream_t st) {
   const void *src = h->L.buf[from];
   void *dst = h->L.buf[from ^ 1];
-  if (h->L.dtype == LBM_F64) return launch_step_f64(h->L, src, dst, st, 256, h->grid_cap);
+  if (h->L.dtype == LBM_F64) return launch_step_f64(h->L, src, dst, st);
   return launch_step_dev(h->L, src, dst, st, h->block, h->L.variant);
 }
 

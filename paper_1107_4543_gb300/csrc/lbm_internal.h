@@ -161,8 +161,7 @@ inline cudaError_t upload_batch_consts(int dtype, const BatchEntry *ents, int n,
     default: return cudaSuccess;
   }
 }
-cudaError_t launch_step_f64(const Lattice &L, const void *src, void *dst,
-                            cudaStream_t st, int block, int grid_cap);
+cudaError_t launch_step_f64(const Lattice &L, const void *src, void *dst, cudaStream_t st);
 
 inline cudaError_t launch_step_dev(const Lattice &L, const void *src, void *dst,
                                    cudaStream_t st, int block, int variant) {

@@ -32,7 +32,6 @@ struct lbm_ctx {
   // with 256-thread blocks (measured +3-4% on batches, +5-7% on one FP16 or
   // BF16 lattice, FP32 8192^2 unchanged); the FP64 step keeps 256
   int block = 64;
-  int grid_cap = 0;
   bool tuned = false;
   lbm_batch_ctx *batch = nullptr;
   // acoustic point source (lbm_set_source)

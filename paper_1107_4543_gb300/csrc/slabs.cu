@@ -102,7 +102,7 @@ cudaError_t launch_rows(lbm_handle h, int from, int r0, int nr, cudaStream_t st)
   const long long off = (long long)r0 * L.g.rstride * L.esize;
   const void *src = static_cast<const char *>(L.buf[from]) + off;
   void *dst = static_cast<char *>(L.buf[from ^ 1]) + off;
-  if (L.dtype == LBM_F64) return launch_step_f64(S, src, dst, st, 256, 0);
+  if (L.dtype == LBM_F64) return launch_step_f64(S, src, dst, st);
   return launch_step_dev(S, src, dst, st, block_of(h), L.variant);
 }
 
