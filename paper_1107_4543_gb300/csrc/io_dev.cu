@@ -9,9 +9,13 @@
 // deviation f^eq(rho, j) - f^eq(rho0, j0), formed here from the differences
 // rho - rho0, j - j0, jx^2/rho - jx0^2/rho0, jy^2/rho - jy0^2/rho0 and
 // jx jy/rho - jx0 jy0/rho0: every term is of the size of the perturbation,
-// so nothing of order one is subtracted after rounding, and a node costs
-// a few dozen FP64 operations and no division (GB300's FP64 rate is what
-// bounds these kernels, not their 60 bytes per node).
+// so nothing of order one is subtracted after rounding.  GB300's FP64 rate
+// (1/64 of FP32) bounded these kernels, not their 60 bytes per node (8192^2
+// FP32: init 8.1 ms, moments 4.6 ms, against 0.6 ms of HBM traffic), so only
+// what needs FP64 runs there: the init forms the six differences in FP64 and
+// their linear combinations as float-float sums, and the moments sum the
+// stored values as float-float (feq_rounded, moments_node): 1.7 and 2.4 ms,
+// the FP64 form's values in the init and within 2^-45 in the moments.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
@@ -42,6 +46,13 @@ RefState make_ref(const AuxView &a) {
 
 __device__ __forceinline__ int wrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
+// rho <= 0 or a value that is not finite, from the bits
+__device__ __forceinline__ bool field_bad(double r, double u, double v) {
+  auto top = [](double d) { return ((unsigned)__double2hiint(d) >> 20) & 0x7ffu; };
+  const bool zero = (((unsigned)__double2hiint(r) << 1) | (unsigned)__double2loint(r)) == 0u;
+  return zero || __double2hiint(r) < 0 || top(r) == 0x7ffu || top(u) == 0x7ffu || top(v) == 0x7ffu;
+}
+
 // f^eq_i(rho, rho u) - f^eq_i(rho0, j0), i = 0..8
 __device__ __forceinline__ void feq_deviation(const RefState &R, double r, double u, double v,
                                               double d[9]) {
@@ -69,42 +80,123 @@ __device__ __forceinline__ void feq_deviation(const RefState &R, double r, doubl
   d[8] = w5 * (q + ex - ey);
 }
 
-template <typename T>
-__device__ __forceinline__ T encode(double d, double scale);
-template <>
-__device__ __forceinline__ float encode<float>(double d, double) {
-  return (float)d;
+// float-float: an unevaluated sum h + l of ~48 bits
+struct FF {
+  float h, l;
+};
+// s + e = a + b exactly (Knuth's TwoSum; additions alone, so no contraction
+// into multiply-adds can touch it)
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+  s = a + b;
+  const float bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
 }
-template <>
-__device__ __forceinline__ __half encode<__half>(double d, double scale) {
-  return __float2half_rn((float)(d * scale));
+__device__ __forceinline__ FF ff_add(FF a, FF b) {
+  float s, e;
+  two_sum(a.h, b.h, s, e);
+  e += a.l + b.l;
+  const float h = s + e;  // |s| >= |e|: the quick form of TwoSum is exact
+  return {h, e - (h - s)};
 }
-template <>
-__device__ __forceinline__ __nv_bfloat16 encode<__nv_bfloat16>(double d, double) {
-  return __float2bfloat16_rn((float)d);
+__device__ __forceinline__ FF ff_neg(FF a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ FF ff_scale(FF a, float p2) { return {a.h * p2, a.l * p2}; }  // p2 = 2^k
+// a (wh + wl)
+__device__ __forceinline__ FF ff_mul(FF a, float wh, float wl) {
+  const float p = __fmul_rn(a.h, wh);
+  float e = __fmaf_rn(a.h, wh, -p);
+  e = __fmaf_rn(a.h, wl, __fmaf_rn(a.l, wh, e));
+  const float h = p + e;
+  return {h, e - (h - p)};
 }
-template <>
-__device__ __forceinline__ double encode<double>(double d, double) {
-  return d;
+// d as float-float from its bits (conversions run at the FP64 rate): the top
+// 24 significand bits, then the low 29 as a scaled integer.  Values below
+// 2^-74 read as zero and add that much to `lost`; false for |d| >= 2^100,
+// infinities and NaN.
+__device__ __forceinline__ bool ff_split(double d, FF &o, float &lost) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned mag = hi & 0x7fffffffu, sign = hi & 0x80000000u, e = mag >> 20;
+  if (e < 949u) {
+    o = {0.0f, 0.0f};
+    lost += (mag | lo) != 0u ? 5.3e-23f : 0.0f;  // 2^-74
+    return true;
+  }
+  o.h = __uint_as_float(sign | (__funnelshift_l(lo, mag, 3) - (896u << 23)));
+  const float unit = __uint_as_float(sign | ((e - 948u) << 23));  // 2^(e - 1023 - 52)
+  o.l = (float)(int)(lo & 0x1fffffffu) * unit;
+  return e < 1123u;
 }
 
+// The nine deviations of feq_deviation rounded to FP32, exactly as the FP64
+// form rounds them: the six O(perturbation) differences in FP64 with the
+// same operations, their combinations as float-float to ~2^-44 of the
+// largest term (in units of the diagonal weight 1/36: the other weights are
+// 4 and 16 times that).  A value whose rounding that error could change --
+// one in ~10^4 -- or a difference outside the split's range returns false,
+// and the caller takes the FP64 form.
+__device__ __forceinline__ bool feq_rounded(const RefState &R, double r, double u, double v,
+                                            float d[9]) {
+  const double jx = r * u, jy = r * v;
+  constexpr double W36 = 1.0 / 36.0, W12 = 1.0 / 12.0, W24 = 1.0 / 24.0;
+  constexpr float w36h = (float)W36, w36l = (float)(W36 - (double)w36h);
+  constexpr float w12h = (float)W12, w12l = (float)(W12 - (double)w12h);
+  constexpr float w24h = (float)W24, w24l = (float)(W24 - (double)w24h);
+  FF t[6];
+  float lost = 0.0f;
+  bool ok = ff_split(r - R.rho0, t[0], lost);
+  ok &= ff_split(jx - R.jx0, t[1], lost);
+  ok &= ff_split(jy - R.jy0, t[2], lost);
+  ok &= ff_split(fma(jx, u, -R.axx0), t[3], lost);
+  ok &= ff_split(fma(jy, v, -R.ayy0), t[4], lost);
+  ok &= ff_split(fma(jx, v, -R.axy0), t[5], lost);
+  const FF dr = ff_mul(t[0], w36h, w36l);
+  const FF X = ff_mul(t[1], w12h, w12l), Y = ff_mul(t[2], w12h, w12l);
+  const FF a = ff_mul(t[3], w24h, w24l), b = ff_mul(t[4], w24h, w24l);
+  const FF c = ff_scale(t[5], 0.25f);
+  const FF S = ff_add(a, b);
+  const FF t1 = ff_add(ff_add(dr, ff_neg(b)), ff_scale(a, 2.0f));
+  const FF t2 = ff_add(ff_add(dr, ff_neg(a)), ff_scale(b, 2.0f));
+  const FF t5 = ff_add(dr, ff_scale(S, 2.0f));
+  const FF p = ff_add(t5, c), q = ff_add(t5, ff_neg(c));
+  const FF xy = ff_add(X, Y), yx = ff_add(Y, ff_neg(X));
+  const FF o[9] = {ff_add(dr, ff_neg(S)), ff_add(t1, X),           ff_add(t2, Y),
+                   ff_add(t1, ff_neg(X)), ff_add(t2, ff_neg(Y)),   ff_add(p, xy),
+                   ff_add(q, yx),         ff_add(p, ff_neg(xy)),   ff_add(q, ff_neg(yx))};
+  // 2^-43 of the terms' magnitudes, and what the split dropped
+  const float tol = 1.14e-13f * (fabsf(dr.h) + fabsf(X.h) + fabsf(Y.h) +
+                                 4.0f * (fabsf(a.h) + fabsf(b.h)) + fabsf(c.h)) +
+                    lost;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    ok &= o[i].h + (o[i].l + tol) == o[i].h && o[i].h + (o[i].l - tol) == o[i].h;
+    d[i] = o[i].h * (i == 0 ? 16.0f : (i <= 4 ? 4.0f : 1.0f));
+  }
+  return ok;
+}
+
+// feq_rounded, or the FP64 form where it cannot tell
+__device__ __forceinline__ void feq_f32(const RefState &R, double r, double u, double v,
+                                        float f[9]) {
+  if (feq_rounded(R, r, u, v, f)) return;
+  double d[9];
+  feq_deviation(R, r, u, v, d);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) f[i] = (float)d[i];
+}
+
+// storage of an FP32 deviation (FP16: times the power-of-two scale, exact)
 template <typename T>
-__device__ __forceinline__ double decode(T s, double inv_scale);
+__device__ __forceinline__ T encode_f32(float d, float scale);
 template <>
-__device__ __forceinline__ double decode<float>(float s, double) {
-  return (double)s;
+__device__ __forceinline__ float encode_f32<float>(float d, float) {
+  return d;
 }
 template <>
-__device__ __forceinline__ double decode<__half>(__half s, double inv_scale) {
-  return (double)__half2float(s) * inv_scale;  // the scale is a power of two
+__device__ __forceinline__ __half encode_f32<__half>(float d, float scale) {
+  return __float2half_rn(d * scale);
 }
 template <>
-__device__ __forceinline__ double decode<__nv_bfloat16>(__nv_bfloat16 s, double) {
-  return (double)__bfloat162float(s);
-}
-template <>
-__device__ __forceinline__ double decode<double>(double s, double) {
-  return s;
+__device__ __forceinline__ __nv_bfloat16 encode_f32<__nv_bfloat16>(float d, float) {
+  return __float2bfloat16_rn(d);
 }
 
 // Population i of node x goes to slot x - c_i, where the next step's pull
@@ -116,14 +208,22 @@ template <typename T>
 __device__ __forceinline__ bool init_node(const AuxView &a, const RefState &R, int x, int y,
                                           double r, double u, double v) {
   T *buf = static_cast<T *>(a.buf);
-  double d[9];
-  feq_deviation(R, r, u, v, d);
+  T e[9];
+  if constexpr (sizeof(T) == 8) {
+    feq_deviation(R, r, u, v, e);
+  } else {
+    float f[9];
+    feq_f32(R, r, u, v, f);
+    const float scale = (float)a.scale;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) e[i] = encode_f32<T>(f[i], scale);
+  }
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     const int xs = wrap(x - CXd(i), a.g.nx), ys = wrap(y - CYd(i), a.g.nyw);
-    buf[(long long)i * a.g.plane + (long long)ys * a.g.rstride + xs] = encode<T>(d[i], a.scale);
+    buf[(long long)i * a.g.plane + (long long)ys * a.g.rstride + xs] = e[i];
   }
-  return !(r > 0.0) || !isfinite(r) || !isfinite(u) || !isfinite(v);
+  return field_bad(r, u, v);
 }
 
 template <typename T>
@@ -149,35 +249,96 @@ __global__ void __launch_bounds__(256) k_maxdev_dev(AuxView a, RefState R, const
   float m = 0.0f;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
-    double d[9];
-    feq_deviation(R, rho[n], ux[n], uy[n], d);
+    float d[9];
+    feq_f32(R, rho[n], ux[n], uy[n], d);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) m = fmaxf(m, (float)fabs(d[i]));
+    for (int i = 0; i < 9; ++i) m = fmaxf(m, fabsf(d[i]));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) atomicMax(max_bits, __float_as_uint(m));
 }
 
+template <typename T>
+__device__ __forceinline__ float decode_f32(T s, float inv_scale);
+template <>
+__device__ __forceinline__ float decode_f32<float>(float s, float) {
+  return s;
+}
+template <>
+__device__ __forceinline__ float decode_f32<__half>(__half s, float inv_scale) {
+  return __half2float(s) * inv_scale;  // a power of two
+}
+template <>
+__device__ __forceinline__ float decode_f32<__nv_bfloat16>(__nv_bfloat16 s, float) {
+  return __bfloat162float(s);
+}
+
+__device__ __forceinline__ void ff_acc(FF &s, float a) {
+  float e;
+  two_sum(s.h, a, s.h, e);
+  s.l += e;
+}
+// a float's double by its bits (conversions run at the FP64 rate)
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), mag = b & 0x7fffffffu, e = mag >> 23;
+  if (e - 1u >= 254u && mag != 0u) return (double)f;  // subnormal, infinite, NaN
+  const unsigned hi = mag == 0u ? 0u : (mag >> 3) + 0x38000000u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(mag << 29));
+}
+__device__ __forceinline__ double ff_value(FF s) { return widen(s.h) + widen(s.l); }
+// 1 / r within an ulp: the hardware's approximation and two Newton-Raphson
+// steps, the ordinary division where those could overflow
+__device__ __forceinline__ double reciprocal(double r) {
+  const unsigned e = ((unsigned)__double2hiint(r) >> 20) & 0x7ffu;
+  if (e - 523u >= 1000u) return 1.0 / r;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r));
+  y = fma(y, fma(-r, y, 1.0), y);
+  return fma(y, fma(-r, y, 1.0), y);
+}
+
 // rho = rho0 + sum f', j = j0 + sum c f' of the pre-collision populations
 // f_i(x) = P_i(x - c_i); u = j / rho
 // rho, u of node (x, y) from its pre-collision populations
 template <typename T>
-__device__ __forceinline__ void moments_node(const AuxView &a, int x, int y, double inv_scale,
+__device__ __forceinline__ void moments_node(const AuxView &a, int x, int y, float inv_scale,
                                              double &r, double &u, double &v) {
   const T *buf = static_cast<const T *>(a.buf);
-  double f[9];
+  if constexpr (sizeof(T) == 8) {
+    double f[9];
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const int xs = wrap(x - CXd(i), a.g.nx), ys = wrap(y - CYd(i), a.g.nyw);
-    f[i] = decode<T>(buf[(long long)i * a.g.plane + (long long)ys * a.g.rstride + xs], inv_scale);
+    for (int i = 0; i < 9; ++i) {
+      const int xs = wrap(x - CXd(i), a.g.nx), ys = wrap(y - CYd(i), a.g.nyw);
+      f[i] = buf[(long long)i * a.g.plane + (long long)ys * a.g.rstride + xs];
+    }
+    r = a.rho0 + (f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8]);
+    const double jx = a.jx0 + (f[1] - f[3] + f[5] - f[6] - f[7] + f[8]);
+    const double jy = a.jy0 + (f[2] - f[4] + f[5] + f[6] - f[7] - f[8]);
+    const double inv = 1.0 / r;
+    u = jx * inv;
+    v = jy * inv;
+  } else {
+    // the deviations' sums as float-float (~48 bits of the stored 24 or
+    // fewer), then two FP64 additions each and one reciprocal
+    float f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const int xs = wrap(x - CXd(i), a.g.nx), ys = wrap(y - CYd(i), a.g.nyw);
+      f[i] = decode_f32<T>(buf[(long long)i * a.g.plane + (long long)ys * a.g.rstride + xs],
+                           inv_scale);
+    }
+    FF s0{f[0], 0.0f}, s1{f[1], 0.0f}, s2{f[2], 0.0f};
+#pragma unroll
+    for (int i = 1; i < 9; ++i) ff_acc(s0, f[i]);
+    ff_acc(s1, -f[3]); ff_acc(s1, f[5]); ff_acc(s1, -f[6]); ff_acc(s1, -f[7]); ff_acc(s1, f[8]);
+    ff_acc(s2, -f[4]); ff_acc(s2, f[5]); ff_acc(s2, f[6]); ff_acc(s2, -f[7]); ff_acc(s2, -f[8]);
+    r = a.rho0 + ff_value(s0);
+    const double jx = a.jx0 + ff_value(s1), jy = a.jy0 + ff_value(s2);
+    const double inv = reciprocal(r);
+    u = jx * inv;
+    v = jy * inv;
   }
-  r = a.rho0 + (f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8]);
-  const double jx = a.jx0 + (f[1] - f[3] + f[5] - f[6] - f[7] + f[8]);
-  const double jy = a.jy0 + (f[2] - f[4] + f[5] + f[6] - f[7] - f[8]);
-  const double inv = 1.0 / r;
-  u = jx * inv;
-  v = jy * inv;
 }
 
 template <typename T>
@@ -185,7 +346,7 @@ __global__ void __launch_bounds__(256) k_moments_dev(AuxView a, double *rho, dou
                                                      double *uy) {
   const int nx = a.g.nx, ny = a.g.ny;
   const long long N = (long long)nx * ny;
-  const double inv_scale = 1.0 / a.scale;
+  const float inv_scale = (float)(1.0 / a.scale);  // a power of two
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
     int x, y;
@@ -248,7 +409,7 @@ __global__ void __launch_bounds__(256) k_batch_init_dev(const AuxView *__restric
 template <typename T>
 __device__ __forceinline__ void batch_moments_block(const AuxView &a, const IoBlock &B,
                                                     double *r_, double *u_, double *v_) {
-  const double inv_scale = 1.0 / a.scale;
+  const float inv_scale = (float)(1.0 / a.scale);  // a power of two
   for (int j = threadIdx.x; j < B.count; j += blockDim.x) {
     const long long n = B.start + j;
     int x, y;
@@ -303,10 +464,10 @@ __global__ void __launch_bounds__(256) k_batch_maxdev_fp16(const AuxView *__rest
   float m = 0.0f;
   for (int j = threadIdx.x; j < B.count; j += blockDim.x) {
     const long long n = B.start + j;
-    double d[9];
-    feq_deviation(R, r[n], r[total + n], r[2 * total + n], d);
+    float d[9];
+    feq_f32(R, r[n], r[total + n], r[2 * total + n], d);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) m = fmaxf(m, (float)fabs(d[i]));
+    for (int i = 0; i < 9; ++i) m = fmaxf(m, fabsf(d[i]));
   }
   // one atomic per block (a member's blocks all update the same word)
 #pragma unroll

@@ -101,3 +101,35 @@ def test_forced_tiles_follow_the_single_forced_steps(L, dtype):
         finally:
             L.lbm_destroy(h)
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
+
+
+@pytest.mark.parametrize("u0", [(0.0, 0.0), (0.125, -0.0625)])
+@pytest.mark.parametrize("amp", [0.0, 1e-9, 1e-3, 0.3])
+def test_init_rounds_the_fp64_deviations_once(L, amp, u0):
+    """The FP32 init (float-float combinations of FP64 differences) stores
+    the FP64 deviations of LBM_F64DEV rounded once: within 2^-24 of each,
+    plus the roundings of adding the base, which a lattice holds after its
+    creation (u0 exact in FP32, so both types have the same one).  The FP32
+    moments are then those sums' errors away from the fields."""
+    nx, ny = 61, 37
+    rng = np.random.default_rng(7)
+    rho = 1.0 + amp * rng.uniform(-1, 1, (ny, nx))
+    ux = u0[0] + amp * rng.uniform(-1, 1, (ny, nx))
+    uy = u0[1] + amp * rng.uniform(-1, 1, (ny, nx))
+    h = L.lbm_create(nx, ny, RATES, 1.0, u0, L.LBM_F32DEV)
+    d = L.lbm_create(nx, ny, RATES, 1.0, u0, L.LBM_F64DEV)
+    try:
+        base = L.lbm_get_populations(d)
+        for x in (h, d):
+            L.lbm_init_field(x, rho, ux, uy)
+        want = L.lbm_get_populations(d)
+        err = 2.0 ** -24 * np.abs(want - base)
+        assert np.all(np.abs(L.lbm_get_populations(h) - want) <= err + 2.0 ** -51)
+        r, u, v = L.lbm_moments(h)
+        e = err.sum(axis=0) + 2.0 ** -47
+        assert np.all(np.abs(r - rho) <= e)
+        assert np.all(np.abs(u - ux) <= (1 + np.abs(ux)) * e / rho)
+        assert np.all(np.abs(v - uy) <= (1 + np.abs(uy)) * e / rho)
+    finally:
+        L.lbm_destroy(h)
+        L.lbm_destroy(d)
