@@ -161,13 +161,16 @@ __device__ __forceinline__ bool feq_rounded(const RefState &R, double r, double 
   const FF o[9] = {ff_add(dr, ff_neg(S)), ff_add(t1, X),           ff_add(t2, Y),
                    ff_add(t1, ff_neg(X)), ff_add(t2, ff_neg(Y)),   ff_add(p, xy),
                    ff_add(q, yx),         ff_add(p, ff_neg(xy)),   ff_add(q, ff_neg(yx))};
-  // 2^-43 of the terms' magnitudes, and what the split dropped
-  const float tol = 1.14e-13f * (fabsf(dr.h) + fabsf(X.h) + fabsf(Y.h) +
-                                 4.0f * (fabsf(a.h) + fabsf(b.h)) + fabsf(c.h)) +
-                    lost;
+  // 2^-43 of the terms' magnitudes (the rest population has no term linear
+  // in the velocity, which is the largest elsewhere), and what the split
+  // dropped
+  const float tol0 = 1.14e-13f * (fabsf(dr.h) + 4.0f * (fabsf(a.h) + fabsf(b.h)) + fabsf(c.h)) +
+                     lost;
+  const float tol = tol0 + 1.14e-13f * (fabsf(X.h) + fabsf(Y.h));
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    ok &= o[i].h + (o[i].l + tol) == o[i].h && o[i].h + (o[i].l - tol) == o[i].h;
+    const float t = i == 0 ? tol0 : tol;
+    ok &= o[i].h + (o[i].l + t) == o[i].h && o[i].h + (o[i].l - t) == o[i].h;
     d[i] = o[i].h * (i == 0 ? 16.0f : (i <= 4 ? 4.0f : 1.0f));
   }
   return ok;
