@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "lbm_internal.h"
+#include "plan.h"
 #include "runtime.h"
 #include "slots.h"
 
@@ -62,6 +63,10 @@ struct lbm_batch_ctx {
     BatchEntry *ents = nullptr;
     BlockRec *blocks = nullptr;
     int *limits = nullptr;  // per-entry step limits of a ragged generation
+    // records of the kRowSteps-per-launch grid (rows_group; none: the group
+    // steps one by one)
+    RowsRec *rows = nullptr;
+    long long nrows = 0;
     // entries held in shared memory for all the steps of a launch (small
     // lattices; k_batch_resident), which the block records leave out; in
     // three classes by size (up to a third, a half, all of a block's shared
@@ -171,6 +176,8 @@ static BatchList batch_list(const lbm_batch_ctx::Group &gr) {
   bl.nblocks = gr.nblocks;
   bl.ntasks = gr.ntasks;
   bl.pbase = gr.pbase;
+  bl.rows = gr.rows;
+  bl.nrows = gr.nrows;
   return bl;
 }
 
@@ -221,12 +228,32 @@ static cudaError_t batch_launch_all(lbm_batch_ctx *b, int parity, cudaStream_t s
   return cudaSuccess;
 }
 
+// n steps (kRowSteps, or 1) of every group from batch parity `parity`.
+// kRowSteps is odd, so its one launch leaves the parity that single steps
+// leave, and groups of both kinds stay together.
+static cudaError_t batch_launch_steps(lbm_batch_ctx *b, int parity, int n, cudaStream_t st) {
+  if (n == 1) return batch_launch_all(b, parity, st, b->variant);
+  for (auto &gr : b->groups) {
+    cudaError_t e = cudaSuccess;
+    if (gr.nrows > 0) {
+      e = launch_rows_batch(gr.dtype, batch_list(gr), parity, st);
+    } else {
+      for (int k = 0; k < n && e == cudaSuccess; ++k)
+        e = launch_step_batch(gr.dtype, batch_list(gr), parity ^ (k & 1), st, b->block,
+                              b->variant);
+    }
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+static_assert(kRowSteps & 1, "a batch's parity counts its steps");
+
 static void batch_drop_graphs(lbm_batch_ctx *b) {
   for (auto &kv : b->graphs) cudaGraphExecDestroy(kv.second);
   b->graphs.clear();
 }
 
-// The captured sequence of `steps` batched step launches starting at batch
+// The captured launches of `steps` steps starting at batch
 // parity 0 (captured on first use, kept until the launch variant changes).
 static int batch_graph(lbm_batch_ctx *b, long steps, cudaGraphExec_t *out) {
   auto it = b->graphs.find(steps);
@@ -240,8 +267,11 @@ static int batch_graph(lbm_batch_ctx *b, long steps, cudaGraphExec_t *out) {
   cudaGraphExec_t ex = nullptr;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    for (long k = 0; k < steps && e == cudaSuccess; ++k)
-      e = batch_launch_all(b, (int)(k & 1), cs, b->variant);
+    for (long k = 0; k < steps && e == cudaSuccess;) {
+      const int n = steps - k >= kRowSteps ? kRowSteps : 1;
+      e = batch_launch_steps(b, (int)(k & 1), n, cs);
+      k += n;
+    }
     cudaError_t e2 = cudaStreamEndCapture(cs, &gr);
     if (e == cudaSuccess) e = e2;
   }
@@ -306,7 +336,9 @@ static int tune_batch(lbm_batch_ctx *b, double *times) {
 // First step of a large batch: reuse the choice made for a batch of the
 // same composition (storage types and sizes, in order) or tune now.
 static int maybe_autotune_batch(lbm_batch_ctx *b) {
-  if (b->nodes >= (1LL << 20) && autotune_enabled()) {
+  bool single = false;  // some group's steps are single-step launches
+  for (auto &gr : b->groups) single |= gr.nblocks > 0 && gr.nrows == 0;
+  if (single && b->nodes >= (1LL << 20) && autotune_enabled()) {
     int cached = -1;
     {
       std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -365,10 +397,21 @@ int batch_step_ragged(lbm_batch_ctx *b, const long *steps, long n) {
                        cudaMemcpyHostToDevice, b->stream));
   int rrc = resident_fork(b, 0, n, true);
   if (rrc != LBM_OK) return rrc;
-  for (long k = 0; k < n; ++k)
-    for (auto &gr : b->groups)
-      CK(launch_step_batch(gr.dtype, batch_list(gr), (int)(k & 1), b->stream, b->block,
-                           b->variant, gr.limits, (int)k));
+  for (auto &gr : b->groups) {
+    const BatchList bl = batch_list(gr);
+    if (gr.nrows > 0) {
+      // whole groups of kRowSteps, then each lattice's remainder
+      for (long k = 0; k + kRowSteps <= n; k += kRowSteps)
+        CK(launch_rows_batch(gr.dtype, bl, (int)(k & 1), b->stream, gr.limits, (int)k));
+      for (int j = 0; j + 1 < kRowSteps; ++j)
+        CK(launch_step_batch(gr.dtype, bl, 0, b->stream, b->block, b->variant, gr.limits,
+                             -1 - j));
+    } else {
+      for (long k = 0; k < n; ++k)
+        CK(launch_step_batch(gr.dtype, bl, (int)(k & 1), b->stream, b->block, b->variant,
+                             gr.limits, (int)k));
+    }
+  }
   rrc = resident_join(b);
   if (rrc != LBM_OK) return rrc;
   for (size_t mi = 0; mi < nm; ++mi) {
@@ -417,6 +460,7 @@ static void batch_free(lbm_batch_ctx *b) {
   for (auto &gr : b->groups) {
     dev_free(gr.ents);
     dev_free(gr.blocks);
+    dev_free(gr.rows);
     dev_free(gr.limits);
     dev_free(gr.res);
     dev_free(gr.pstage);
@@ -601,6 +645,45 @@ static std::vector<size_t> packed_groups(const lbm_batch_ctx *b) {
   return ends;
 }
 
+// Block records of the kRowSteps-per-launch grid of a batch's members of
+// storage type dt that are not resident; none where the grid does not take
+// some member or the members together are too small for it (the threshold
+// of a single lattice's plan).  Tasks of most rows first, so that the short
+// ones fill the tail of the launch.
+static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms) {
+  std::vector<RowsRec> recs;
+  double nodes = 0, rows32 = 0;
+  for (size_t mi = 0; mi < b->members.size(); ++mi) {
+    const Lattice &L = b->members[mi]->L;
+    if (L.dtype != dt || b->member_res[mi]) continue;
+    if (!rows_fit(L.g, L.V) || L.g.ny < kRowSteps) return recs;
+    nodes += (double)L.g.nx * L.g.ny;
+    rows32 += rows_geom(L.g, 32).tasks;
+  }
+  if (nodes < rows_min_nodes(dt == LBM_F32DEV ? 4 : 2)) return recs;
+  // 32 rows per task, or 16 where that leaves fewer than six tasks per
+  // resident warp and the tail would weigh
+  const int rows = rows32 < 6.0 * sms * rows_warps(dt == LBM_F32DEV ? 4 : 2) ? 16 : 32;
+  for (size_t mi = 0; mi < b->members.size(); ++mi) {
+    const Lattice &L = b->members[mi]->L;
+    if (L.dtype != dt || b->member_res[mi]) continue;
+    RowsRec r;
+    r.g = L.g;
+    r.rg = rows_geom(L.g, rows);
+    r.buf[0] = L.buf[0];
+    r.buf[1] = L.buf[1];
+    r.lat = b->member_local[mi];
+    r.off = L.cur;
+    for (unsigned t = 0; t < (unsigned)r.rg.tasks; t += 2) {
+      r.task = t;
+      recs.push_back(r);
+    }
+  }
+  std::stable_sort(recs.begin(), recs.end(),
+                   [](const RowsRec &a, const RowsRec &c) { return a.rg.rows > c.rg.rows; });
+  return recs;
+}
+
 extern "C" {
 
 int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
@@ -694,6 +777,7 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
       ents.push_back(e);
     }
     if (ents.empty()) continue;
+    const std::vector<RowsRec> rl = rows_records(b, dt, sm_count());
     lbm_batch_ctx::Group gr;
     gr.dtype = dt;
     gr.n = (int)ents.size();
@@ -702,6 +786,8 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
     gr.ents = (BatchEntry *)dev_alloc(sizeof(BatchEntry) * ents.size());
     gr.blocks = (BlockRec *)dev_alloc(sizeof(BlockRec) * bl.size());
     gr.limits = (int *)dev_alloc(sizeof(int) * ents.size());
+    gr.nrows = (long long)rl.size();
+    if (gr.nrows > 0) gr.rows = (RowsRec *)dev_alloc(sizeof(RowsRec) * rl.size());
     std::vector<int> res;
     for (int c = 0; c < 3; ++c) {
       res.insert(res.end(), res_cls[c].begin(), res_cls[c].end());
@@ -724,7 +810,8 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
       }
     }
     b->groups.push_back(gr);
-    if (!gr.ents || !gr.blocks || !gr.limits || (gr.nres > 0 && !gr.res)) {
+    if (!gr.ents || !gr.blocks || !gr.limits || (gr.nres > 0 && !gr.res) ||
+        (gr.nrows > 0 && !gr.rows)) {
       set_error("cannot allocate batch tables");
       batch_free(b);
       return LBM_ENOMEM;
@@ -733,6 +820,8 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
                         cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
         (!bl.empty() && cudaMemcpyAsync(gr.blocks, bl.data(), sizeof(BlockRec) * bl.size(),
                                         cudaMemcpyHostToDevice, b->stream) != cudaSuccess) ||
+        (gr.nrows > 0 && cudaMemcpyAsync(gr.rows, rl.data(), sizeof(RowsRec) * rl.size(),
+                                         cudaMemcpyHostToDevice, b->stream) != cudaSuccess) ||
         (gr.nres > 0 && cudaMemcpyAsync(gr.res, res.data(), sizeof(int) * res.size(),
                                         cudaMemcpyHostToDevice, b->stream) != cudaSuccess)) {
       set_error("cannot upload batch tables");
@@ -805,9 +894,9 @@ int lbm_batch_step(lbm_batch b, long n) {
   // the per-step launches of the others
   int rrc = resident_fork(b, b->parity, n, false);
   if (rrc != LBM_OK) return rrc;
-  // whole graphs of 64 steps, the remainder as one graph of its own length
+  // whole graphs of 66 steps, the remainder as one graph of its own length
   // (both cached), so a call of n steps is a handful of graph launches
-  const long G = 64;
+  const long G = 66;  // even, and whole groups of kRowSteps
   long done = 0;
   if (b->parity == 1 && n > 0) {
     CK(batch_launch_all(b, 1, b->stream, b->variant));

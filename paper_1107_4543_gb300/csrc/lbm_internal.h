@@ -39,9 +39,10 @@ struct DevGuard {
 
 // Work split of the kernels that advance several steps per launch
 // (step_multi.cuh; chosen in plan.h).
-// k_step_rows: strips of `width` chunks, tasks of `rows` rows of one strip
+// k_step_rows: `segs` segments of `rows` rows, `tasks` warp tasks of 30 lane
+// positions
 struct RowsGeom {
-  int strips, width, rows;
+  int rows, segs, tasks;
 };
 // k_step_tile: tiles of bx x by nodes, at most `steps` steps per launch
 struct TileGeom {
@@ -96,10 +97,23 @@ struct BlockRec {
   int off;              // as BatchEntry::off
 };
 
+// One block of a batch's k_rows_batch grid: two tasks of one lattice
+struct RowsRec {
+  Geom g;
+  RowsGeom rg;
+  void *buf[2];
+  unsigned task;  // lattice task of the block's warp 0
+  int lat;        // lattice index in the entry list
+  int off;        // as BatchEntry::off
+};
+
 // Device work list of one storage type's batch members: per-lattice
 // entries and the plain grid's block records (the persistent grids stride
-// over the same records).
+// over the same records), and those of the grid that takes kRowSteps steps
+// per launch.
 struct BatchList {
+  const RowsRec *rows = nullptr;
+  long long nrows = 0;
   const BatchEntry *ents;
   int n;
   int pbase = -1;  // first slot of the type's constant table, or -1 (entries)
@@ -230,6 +244,23 @@ cudaError_t launch_tile_f16(const Lattice &L, const void *src, void *dst, cudaSt
                             int steps, const float *forced, int sx, int sy);
 cudaError_t launch_tile_bf16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
                              int steps, const float *forced, int sx, int sy);
+// kRowSteps steps of a batch's listed members from batch parity `parity`;
+// limits (may be null): lattice l takes part while k + kRowSteps <= limits[l]
+cudaError_t launch_rows_batch_f32(const BatchList &bl, int parity, cudaStream_t st,
+                                  const int *limits, int k);
+cudaError_t launch_rows_batch_f16(const BatchList &bl, int parity, cudaStream_t st,
+                                  const int *limits, int k);
+cudaError_t launch_rows_batch_bf16(const BatchList &bl, int parity, cudaStream_t st,
+                                   const int *limits, int k);
+inline cudaError_t launch_rows_batch(int dtype, const BatchList &bl, int parity, cudaStream_t st,
+                                     const int *limits = nullptr, int k = 0) {
+  switch (dtype) {
+    case LBM_F32DEV: return launch_rows_batch_f32(bl, parity, st, limits, k);
+    case LBM_F16DEV: return launch_rows_batch_f16(bl, parity, st, limits, k);
+    case LBM_BF16DEV: return launch_rows_batch_bf16(bl, parity, st, limits, k);
+    default: return cudaErrorInvalidValue;
+  }
+}
 inline cudaError_t launch_rows(const Lattice &L, const void *src, void *dst, cudaStream_t st,
                                int steps) {
   switch (L.dtype) {

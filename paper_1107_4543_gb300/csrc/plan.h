@@ -7,35 +7,32 @@
 
 namespace lbm {
 
-// k_step_rows: strips of at most 30 chunks (32 lanes less two halo chunks; 28
-// where V does not divide nx, whose seam lanes borrow idle lanes' slots), of
-// equal even width, so that a strip's stores cover whole 32-byte sectors.
-inline RowsGeom rows_geom(const Geom &g, int V, int rows) {
-  const bool ragged = g.nx % V != 0;
-  const int cap = ragged ? 28 : 30;
+// k_step_rows: segments of about `rows` rows, as even as they go, each a
+// sequence of nchunks + 2 lane positions, 30 positions to a task (the first
+// position, a halo, is no task's own).
+inline RowsGeom rows_geom(const Geom &g, int rows) {
   RowsGeom r;
-  r.strips = (g.nchunks + cap - 1) / cap;
-  if (ragged && r.strips == 1 && g.nchunks > 27) r.strips = 2;  // three seam lanes in one strip
-  const int w = (g.nchunks + r.strips - 1) / r.strips;
-  r.width = std::min(cap, (w + 1) & ~1);
-  if (ragged && r.strips == 1) r.width = std::min(r.width, 27);
-  r.strips = (g.nchunks + r.width - 1) / r.width;
-  r.rows = rows;
+  r.segs = std::max(1, (g.ny + rows / 2) / rows);
+  r.rows = (g.ny + r.segs - 1) / r.segs;
+  r.segs = (g.ny + r.rows - 1) / r.rows;
+  const long long pos = (long long)r.segs * (g.nchunks + 2);
+  r.tasks = (int)std::min<long long>((pos - 2 + 29) / 30, 1 << 30);
   return r;
 }
 
 // whether k_step_rows takes the lattice: its seam chunks are assembled from
-// whole neighbouring chunks
-inline bool rows_fit(const Geom &g, int V) { return g.nx % V == 0 || g.nchunks >= 3; }
+// whole neighbouring chunks, and its positions are 32-bit
+inline bool rows_fit(const Geom &g, int V) {
+  return (g.nx % V == 0 || g.nchunks >= 3) && (double)g.ny * (g.nchunks + 2) < 4e9;
+}
 
-// Rows per task: 32 cost 2 (kRowSteps - 1) / 32 of redundant level-1 rows;
+// Rows per segment: 32 cost 2 (kRowSteps - 1) / 32 of redundant level-1 rows;
 // fewer where the tasks would not fill the resident warps (`slots`) a
 // quarter more than once (2048^2 FP32: 16 rows 23.2 us per step, 32 rows
 // 31.1, 8 rows 24.9).
-inline RowsGeom plan_rows(const Geom &g, int V, int slots) {
-  const RowsGeom r = rows_geom(g, V, 32);
-  const double fit = (double)g.ny * r.strips / (1.25 * slots);
-  return rows_geom(g, V, (int)std::max(8.0, std::min(32.0, fit)));
+inline RowsGeom plan_rows(const Geom &g, int slots) {
+  const double fit = (double)g.ny * (g.nchunks + 2) / 30.0 / (1.25 * slots);
+  return rows_geom(g, (int)std::max(8.0, std::min(32.0, fit)));
 }
 
 // k_step_tile: the split of least estimated time per step with all tiles
@@ -70,10 +67,12 @@ inline TileGeom plan_tile(const Geom &g, int esize, int sms, double *us_per_step
 // 32- and 16-bit deviation types: tiles where they fit and are estimated
 // faster than one launch per step (2.0 + 6.1 us per 2^20 FP32 nodes, 2.7 +
 // 4.1 us in 16 bits, measured from 512^2 to 1024^2); else rows for lattices
-// whose tasks keep the warps busy (kRowsNodes: below, single steps measured
-// as fast); else, and for the FP64 types (bound by FP64 arithmetic, which
+// whose tasks keep the warps busy (rows_min_nodes: below, single steps
+// measured as fast); else, and for the FP64 types (bound by FP64 arithmetic, which
 // halos only add to), one step per launch.
-constexpr double kRowsNodes32 = 1.25e6, kRowsNodes16 = 3.0e6;
+inline double rows_min_nodes(int esize) { return esize == 4 ? 1.25e6 : 3.0e6; }
+// resident warps per SM of k_step_rows
+inline int rows_warps(int esize) { return esize == 4 ? 12 : 8; }
 
 inline void plan_lattice(Lattice &L, int sms) {
   L.plan = PLAN_SINGLE;
@@ -85,9 +84,9 @@ inline void plan_lattice(Lattice &L, int sms) {
   if (t.steps > 1 && us < single) {
     L.plan = PLAN_TILE;
     L.tile = t;
-  } else if (nodes >= (L.esize == 4 ? kRowsNodes32 : kRowsNodes16) && rows_fit(L.g, L.V)) {
+  } else if (nodes >= rows_min_nodes(L.esize) && rows_fit(L.g, L.V)) {
     L.plan = PLAN_ROWS;
-    L.rows = plan_rows(L.g, L.V, sms * (L.esize == 4 ? 12 : 8));
+    L.rows = plan_rows(L.g, sms * rows_warps(L.esize));
   }
 }
 

@@ -31,6 +31,11 @@ cudaError_t launch_rows_bf16(const Lattice &L, const void *src, void *dst, cudaS
   return launch_rows_t<__nv_bfloat16>(L, src, dst, st, steps);
 }
 
+cudaError_t launch_rows_batch_bf16(const BatchList &bl, int parity, cudaStream_t st,
+                                  const int *limits, int k) {
+  return launch_rows_batch_t<__nv_bfloat16>(bl, parity, st, limits, k);
+}
+
 cudaError_t launch_tile_bf16(const Lattice &L, const void *src, void *dst, cudaStream_t st,
                             int steps, const float *forced, int sx, int sy) {
   return launch_tile_t<__nv_bfloat16>(L, src, dst, st, steps, forced, sx, sy);

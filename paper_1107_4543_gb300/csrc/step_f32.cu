@@ -31,6 +31,11 @@ cudaError_t launch_rows_f32(const Lattice &L, const void *src, void *dst, cudaSt
   return launch_rows_t<float>(L, src, dst, st, steps);
 }
 
+cudaError_t launch_rows_batch_f32(const BatchList &bl, int parity, cudaStream_t st,
+                                  const int *limits, int k) {
+  return launch_rows_batch_t<float>(bl, parity, st, limits, k);
+}
+
 cudaError_t launch_tile_f32(const Lattice &L, const void *src, void *dst, cudaStream_t st,
                             int steps, const float *forced, int sx, int sy) {
   return launch_tile_t<float>(L, src, dst, st, steps, forced, sx, sy);

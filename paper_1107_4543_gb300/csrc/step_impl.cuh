@@ -135,6 +135,21 @@ k_step_dev(const T *__restrict__ src, T *__restrict__ dst, Geom g,
     step_task<T>(src, dst, g, P, task, lane);
 }
 
+// Whether lattice `lat` takes part in single step k of a ragged generation
+// (limits null: every lattice does).  k < 0: tail step -1 - k of a
+// generation whose whole groups of kRowSteps steps ran before (k_rows_batch):
+// the lattice still owes limits[lat] mod kRowSteps steps, from the parity of
+// the steps it has taken.
+__device__ __forceinline__ bool limit_takes(const int *__restrict__ limits, int lat, int k,
+                                            int &parity) {
+  if (limits == nullptr) return true;
+  const int n = limits[lat];
+  if (k >= 0) return k < n;
+  const int rest = n % kRowSteps, done = n - rest + (-1 - k);
+  parity = done & 1;
+  return -1 - k < rest;
+}
+
 // Batched, plain grid: every lattice starts on a block boundary and block b
 // reads its lattice's geometry and buffers from blocks[b] (one load before
 // the pull can start; a search over the lattices' task offsets, or a
@@ -169,7 +184,7 @@ __device__ __forceinline__ void batch_block(const BatchEntry *__restrict__ ents,
   const long long task = B.task_base + (threadIdx.x >> 5);
   if (task >= B.g.tasks) return;                         // warp-uniform
   if (!bounds::ok(B.lat >= 0 && B.lat < nents, bounds::BATCH_REC)) return;
-  if (limits != nullptr && k >= limits[B.lat]) return;   // block-uniform
+  if (!limit_takes(limits, B.lat, k, parity)) return;  // block-uniform
   const int from = parity ^ B.off;
   const T *src = static_cast<const T *>(B.buf[from]);
   T *dst = static_cast<T *>(B.buf[from ^ 1]);
@@ -240,9 +255,10 @@ k_step_batch_stride(const BatchEntry *__restrict__ ents, const BlockRec *__restr
     if (nb < nblocks && lane < NW) next = __ldg(reinterpret_cast<const uint32_t *>(blocks + nb) + lane);
     const BlockRec &B = rec[s][w];
     const long long task = B.task_base + w;
+    int par = parity;
     if (task < B.g.tasks && bounds::ok(B.lat >= 0 && B.lat < nents, bounds::BATCH_REC) &&
-        !(limits != nullptr && k >= limits[B.lat])) {  // warp-uniform
-      const int from = parity ^ B.off;
+        limit_takes(limits, B.lat, k, par)) {  // warp-uniform
+      const int from = par ^ B.off;
       step_task<T>(static_cast<const T *>(B.buf[from]), static_cast<T *>(B.buf[from ^ 1]), B.g,
                    ents[B.lat].dp, task, lane);
     }

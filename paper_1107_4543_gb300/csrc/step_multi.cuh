@@ -10,9 +10,8 @@
 // launch.  Both kernels here trade a halo of redundant nodes for fewer
 // passes over memory and fewer launches:
 //
-//   k_step_rows  (large lattices, batches): each warp marches along y over a
-//     strip of 30 chunks of V nodes, kRowSteps time levels deep; level l of
-//     row y needs level l-1 of rows y-1, y, y+1, which the warp has just
+//   k_step_rows  (large lattices, batches): each warp marches along y over
+//     30 chunks of V nodes, kRowSteps time levels deep; level l of row y needs level l-1 of rows y-1, y, y+1, which the warp has just
 //     computed, so intermediate levels live in lane-private shared-memory
 //     slots and no warp waits for another.
 //   k_step_tile  (small lattices): each block loads a tile with a halo as
@@ -125,111 +124,124 @@ __device__ __forceinline__ void cp_async16(uint4 *smem, const void *g) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(g) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void *smem, const void *g) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(g) : "memory");
+}
 
-// Elements sh .. sh + V - 1 of chunk *a and the chunk `spare` slots after it
-// (shared memory) laid end to end, the first `keep` of them replaced by w's.
-template <typename T>
-__device__ __forceinline__ void seam_chunk(uint32_t (&w)[4], const uint4 *a, int spare, int sh,
+// 16-bit types: elements sh .. sh + 7 of chunks *a, *b (shared memory) laid
+// end to end, the first `keep` of them replaced by w's.
+__device__ __forceinline__ void seam_chunk(uint32_t (&w)[4], const uint4 *a, int ab, int sh,
                                            int keep) {
   const uint32_t *p = reinterpret_cast<const uint32_t *>(a);
-  constexpr int PER = 4 / (int)sizeof(T);  // elements per word
-  const int k0 = sh / PER, far = 4 * spare - 4;
+  const int k0 = sh / 2, far = 4 * ab - 4;  // b is ab 16-byte words after a
   uint32_t v[5];
 #pragma unroll
-  for (int q = 0; q < (PER == 2 ? 5 : 4); ++q) {
-    const int k = k0 + q;  // at most 8: the funnel of an even shift ignores it
+  for (int q = 0; q < 5; ++q) {
+    const int k = k0 + q;  // at most 8, which an even shift ignores
     v[q] = p[k < 4 ? k : min(k, 7) + far];
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    if constexpr (PER == 2) {
-      const uint32_t u = (sh & 1) ? __byte_perm(v[q], v[q + 1], 0x5432) : v[q];
-      const uint32_t own = 2 * q + 1 < keep ? 0xffffffffu : (2 * q < keep ? 0xffffu : 0u);
-      w[q] = (w[q] & own) | (u & ~own);
-    } else {
-      w[q] = q < keep ? w[q] : v[q];
-    }
+    const uint32_t u = (sh & 1) ? __byte_perm(v[q], v[q + 1], 0x5432) : v[q];
+    const uint32_t own = 2 * q + 1 < keep ? 0xffffffffu : (2 * q < keep ? 0xffffu : 0u);
+    w[q] = (w[q] & own) | (u & ~own);
   }
 }
 
 // shared memory of one warp of k_step_rows, in 16-byte words: two stages of
-// 9 incoming vectors and, per level boundary, 3 delayed by one row and 3 by
-// two rows, for 32 lanes
-constexpr int rows_smem_words(int steps) { return (18 + 9 * (steps - 1)) * 32; }
+// 9 incoming vectors, per level boundary 3 delayed by one row and 3 by two
+// rows, and for the 16-bit types the seam lanes' second chunks, for 32 lanes
+template <typename T>
+constexpr int rows_smem_words(int steps) {
+  return (18 + 9 * (steps - 1) + (sizeof(T) == 2 ? 18 : 0)) * 32;
+}
 
-// Task `task` of a lattice (at least three chunks per row where V does not
-// divide nx): strip task % strips of the chunks, rows
-// [y0, y0 + rows).  Lane l holds the chunk of virtual nodes
-// [(c0 - 1 + l) V, ... + V), taken periodically: lanes 1 .. cnt are the
-// strip's own chunks, lanes 0 and cnt + 1 its halo.  After each level one
-// more node of each halo chunk is invalid, so STEPS <= V levels leave the
-// strip's nodes exact; in y each level loses one row per side, so level l
-// (1 .. STEPS) covers rows y0 - (STEPS - l) .. y1 - 1 + (STEPS - l).
-// In iteration j level 1 takes row y0 - (STEPS - 1) + j and level l the row
-// l - 1 below it: its populations with c_y = -1 come from the row just
-// computed (registers), those with c_y = 0 from the iteration before and
-// those with c_y = +1 from two before (the delay slots, which only this
-// lane touches: no synchronization).  Incoming rows are copied to shared
-// memory one iteration ahead (cp.async), so no register holds a load in
-// flight: with the loads in registers the compiler spilled (FP32 152 bytes
-// at 168 registers) and the two-step form ran at 125 instead of 174 GLUPS.
-// Where V does not divide the row length, up to three chunks of a row lie
-// across its end (the halo chunk before node 0, the partial last chunk, the
-// halo chunk after it): their lanes copy two aligned chunks, the second into
-// the slot of an idle lane (strips are then at most 28 chunks wide), and
-// assemble them.  A template on the seam, or element-wise gathers, ran
-// ragged lattices at half the speed (4097 x 3071 FP16: 85 and 138 us per
-// step).
+// The lattice's rows are cut into segments of rg.rows; a segment is a
+// sequence of nchunks + 2 lane positions (the chunk before chunk 0, chunks 0
+// .. nchunks - 1, the chunk after the last, taken periodically), the
+// segments' sequences follow one another, and task t takes positions 30 t ..
+// 30 t + 31: its lanes 1 .. 30 advance their chunks, each with its
+// neighbours in the neighbouring lanes, lanes 0 and 31 are halo, and a warp
+// spans segments freely.  (Strips of whole warps left 20% of the lanes of
+// the 128-lattice FP32 sweep idle and 27% in FP16.)
+//
+// After each level one more node of each halo chunk is invalid, so STEPS <=
+// V levels leave the own chunks exact; in y each level loses one row per
+// side, so level l (1 .. STEPS) covers rows y0 - (STEPS - l) .. y1 - 1 +
+// (STEPS - l).  In iteration j level 1 takes row y0 - (STEPS - 1) + j and
+// level l the row l - 1 below it: its populations with c_y = -1 come from
+// the row just computed (registers), those with c_y = 0 from the iteration
+// before and those with c_y = +1 from two before (the delay slots, which
+// only this lane touches: no synchronization).  Incoming rows are copied to
+// shared memory one iteration ahead (cp.async), so no register holds a load
+// in flight: with the loads in registers the compiler spilled (FP32 152
+// bytes at 168 registers) and the two-step form ran at 125 instead of 174
+// GLUPS.
+//
+// Where V does not divide the row length, three chunks of a row lie across
+// its end (the one before node 0, the partial last one, the one after it).
+// Their lanes copy four elements one by one (FP32), or two aligned chunks
+// and assemble them (16 bits: an element is smaller than any copy).
 template <typename T, int STEPS, typename K>
 __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restrict__ dst,
                                           const Geom &g, const RowsGeom &rg, const K &par,
                                           unsigned task, int lane, uint4 *sm) {
   constexpr int V = Elem<T>::V;
   static_assert(STEPS >= 2 && STEPS <= V, "the halo chunk covers V nodes");
-  const unsigned seg = task / (unsigned)rg.strips, strip = task - seg * (unsigned)rg.strips;
+  const unsigned per = (unsigned)g.nchunks + 2u, pos = task * 30u + (unsigned)lane;
+  unsigned seg = pos / per;
+  const int vc = (int)(pos - seg * per) - 1, vx = vc * V;  // chunk, first virtual node
+  const bool in = seg < (unsigned)rg.segs;
+  if (!in) seg = 0;
+  const bool out = in && lane >= 1 && lane <= 30 && vc >= 0 && vc < g.nchunks;
   const int y0 = (int)seg * rg.rows, y1 = min(y0 + rg.rows, g.ny);
-  const int c0 = (int)strip * rg.width, cnt = min(rg.width, g.nchunks - c0);
-  const bool in = lane < cnt + 2, out = lane >= 1 && lane <= cnt;
-  const int vc = in ? c0 - 1 + lane : 0, vx = vc * V;  // chunk, first virtual node
   const int part = g.nx & (V - 1);  // nodes of a partial last chunk (0: none)
-  int ca = vc < 0 ? vc + g.nchunks : (vc >= g.nchunks ? vc - g.nchunks : vc), cb = 0;
-  // seam lanes: element e of the chunk is element e + sh of the chunks ca, cb
-  // laid end to end (a partial last chunk keeps its own first `part`)
   const bool seam = in && part != 0 && (vc < 0 || vc >= g.nchunks - 1);
-  int sh = 0, spare = 0;
-  if (seam) {
+  int ca = vc < 0 ? vc + g.nchunks : (vc >= g.nchunks ? vc - g.nchunks : vc);
+  // 16 bits: element e of a seam chunk is element e + sh of chunks ca, cb
+  // laid end to end (a partial last chunk keeps its own first `part`)
+  int cb = 0, sh = 0;
+  if (sizeof(T) == 2 && seam) {
     sh = vc < 0 ? part : V - part;
     if (vc < 0) ca = g.nchunks - 2;
     cb = vc < 0 ? g.nchunks - 1 : (vc == g.nchunks ? 1 : 0);
-    // (vc < 0 and vc = nchunks share a warp only in a lattice of one strip)
-    spare = 31 - (vc < 0 ? 0 : (vc == g.nchunks - 1 ? 1 : (rg.strips == 1 ? 2 : 0))) - lane;
   }
-  const int x0 = ca * V;
+  const int x0 = sizeof(T) == 4 && seam ? 0 : ca * V;
   const int ya = y0 - (STEPS - 1);
-  const int n = y1 - y0 + 2 * (STEPS - 1);
+  const int n = rg.rows + 2 * (STEPS - 1);
   auto row_of = [&](int y) -> const T * {
     while (y < 0) y += g.ny;
     while (y >= g.ny) y -= g.ny;
     return src + (long long)y * g.rstride;
   };
+  constexpr int kB = (18 + 9 * (STEPS - 1)) * 32;  // the second chunks
   uint4 *raw = sm + lane, *dly = sm + 18 * 32 + lane;
   const T *pm = row_of(ya - 1) + x0, *pc = row_of(ya) + x0, *pp = row_of(ya + 1) + x0;
   int fetched = 0;
   auto fetch = [&]() {  // level 1's row ya + fetched into stage fetched & 1
     if (fetched < n) {
       uint4 *q = raw + (fetched & 1) * (9 * 32);
-      if (in) {  // an idle lane's slots may be a seam lane's
+      auto from = [&](int i) {
+        return (CYd(i) == 1 ? pm : (CYd(i) == -1 ? pp : pc)) + (long long)i * g.plane;
+      };
+      if (in && !(sizeof(T) == 4 && seam)) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-          const T *row = (CYd(i) == 1 ? pm : (CYd(i) == -1 ? pp : pc)) + (long long)i * g.plane;
-          cp_async16(q + i * 32, row);
-        }
+        for (int i = 0; i < 9; ++i) cp_async16(q + i * 32, from(i));
       }
       if (seam) {
+        if constexpr (sizeof(T) == 4) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-          const T *row = (CYd(i) == 1 ? pm : (CYd(i) == -1 ? pp : pc)) + (long long)i * g.plane;
-          cp_async16(q + i * 32 + spare, row + (cb - ca) * V);
+          for (int e = 0; e < 4; ++e) {
+            int x = vx + e;
+            x = x < 0 ? x + g.nx : (x >= g.nx ? x - g.nx : x);
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+              cp_async4(reinterpret_cast<uint32_t *>(q + i * 32) + e, from(i) + x);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 9; ++i) cp_async16(q + kB + i * 32, from(i) + (cb - ca) * V);
         }
       }
       ++fetched;
@@ -241,7 +253,7 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
   };
   fetch();
   T *drow = dst + (long long)y0 * g.rstride + (out ? vx : 0);
-  const bool fill = (g.nchunks & 1) && out && vx + V >= g.nx;  // see fills_sector
+  const bool fill = (g.nchunks & 1) && out && vc == g.nchunks - 1;  // see fills_sector
   for (int j = 0; j < n; ++j) {
     fetch();
     asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -250,10 +262,10 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
       const uint4 *q = raw + (j & 1) * (9 * 32);
 #pragma unroll
       for (int i = 0; i < 9; ++i) set4(w[i], q[i * 32]);
-      if (seam) {
+      if (sizeof(T) == 2 && seam) {
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-          seam_chunk<T>(w[i], q + i * 32, spare, sh, vc == g.nchunks - 1 ? part : 0);
+          seam_chunk(w[i], q + i * 32, kB, sh, vc == g.nchunks - 1 ? part : 0);
       }
     }
 #pragma unroll
@@ -280,7 +292,7 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
       collide_chunk<T>(w, par);
     }
     if (j >= 2 * (STEPS - 1)) {
-      if (out) {
+      if (out && y0 + j - 2 * (STEPS - 1) < y1) {
 #pragma unroll
         for (int i = 0; i < 9; ++i)
           *reinterpret_cast<uint4 *>(drow + (long long)i * g.plane) = get4(w[i]);
@@ -305,7 +317,7 @@ k_step_rows(const T *__restrict__ src, T *__restrict__ dst, Geom g, RowsGeom rg,
   const unsigned warp = threadIdx.x >> 5, task = blockIdx.x * 2 + warp;
   pdl_wait();
   if (task >= ntasks) return;
-  uint4 *sm = rows_smem + warp * rows_smem_words(STEPS);
+  uint4 *sm = rows_smem + warp * rows_smem_words<T>(STEPS);
   if constexpr (sizeof(T) == 4)
     rows_task<T, STEPS>(src, dst, g, rg, P, task, threadIdx.x & 31, sm);
   else
@@ -314,11 +326,11 @@ k_step_rows(const T *__restrict__ src, T *__restrict__ dst, Geom g, RowsGeom rg,
 
 template <typename T, int STEPS>
 cudaError_t launch_rows_steps(const Lattice &L, const void *src, void *dst, cudaStream_t st) {
-  constexpr size_t smem = 2 * rows_smem_words(STEPS) * sizeof(uint4);
+  constexpr size_t smem = 2 * rows_smem_words<T>(STEPS) * sizeof(uint4);
   cudaError_t e = cudaFuncSetAttribute(
       k_step_rows<T, STEPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;
-  const long long nt = (long long)L.rows.strips * ((L.g.ny + L.rows.rows - 1) / L.rows.rows);
+  const long long nt = L.rows.tasks;
   return launch_pdl(k_step_rows<T, STEPS>, (unsigned)((nt + 1) / 2), 64, smem, st,
                     static_cast<const T *>(src), static_cast<T *>(dst), L.g, L.rows,
                     pair_params<T>(L.dp), (unsigned)nt);
@@ -330,6 +342,73 @@ cudaError_t launch_rows_t(const Lattice &L, const void *src, void *dst, cudaStre
   if (steps == 3) return launch_rows_steps<T, 3>(L, src, dst, st);
   if (steps == 2) return launch_rows_steps<T, 2>(L, src, dst, st);
   return cudaErrorInvalidValue;
+}
+
+// The batched form: every block reads its lattice's record and collision
+// constants into shared memory (a lattice's constants cannot be kernel
+// parameters here, and 25 broadcast pairs in registers would spill), then
+// its two warps take one task each.
+template <typename T> struct RowsShared;
+template <> struct RowsShared<float> {
+  RowsRec rec;
+  HlPairs pairs;
+  static constexpr int COUNT = HL_COUNT;
+  static __device__ __forceinline__ float value(const DevParams &P, int k) { return hl_const(P, k); }
+  __device__ __forceinline__ float2 *table() { return pairs.c; }
+  __device__ __forceinline__ const HlPairs &constants() const { return pairs; }
+};
+template <typename T> struct RowsShared {
+  RowsRec rec;
+  float2 c[PC_COUNT];
+  static constexpr int COUNT = PC_COUNT;
+  static __device__ __forceinline__ float value(const DevParams &P, int k) {
+    return pair_const(P, k);
+  }
+  __device__ __forceinline__ float2 *table() { return c; }
+  __device__ __forceinline__ SharedPairs constants() const { return SharedPairs{c}; }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(64, sizeof(T) == 4 ? 6 : 4)
+k_rows_batch(const BatchEntry *__restrict__ ents, const RowsRec *__restrict__ recs, int nents,
+             int parity, const int *__restrict__ limits, int k) {
+  extern __shared__ uint4 rows_smem[];
+  RowsShared<T> &S =
+      *reinterpret_cast<RowsShared<T> *>(rows_smem + 2 * rows_smem_words<T>(kRowSteps));
+  constexpr int NW = sizeof(RowsRec) / 4;
+  static_assert(sizeof(RowsRec) % 4 == 0 && NW <= 64, "a record is copied one word per thread");
+  if (threadIdx.x < NW)
+    reinterpret_cast<uint32_t *>(&S.rec)[threadIdx.x] =
+        reinterpret_cast<const uint32_t *>(recs + blockIdx.x)[threadIdx.x];
+  pdl_wait();
+  __syncthreads();
+  const int lat = S.rec.lat;
+  if (!bounds::ok(lat >= 0 && lat < nents, bounds::BATCH_REC)) return;
+  if (limits != nullptr && k + kRowSteps > limits[lat]) return;  // block-uniform
+  if (threadIdx.x < RowsShared<T>::COUNT) {
+    const float v = RowsShared<T>::value(ents[lat].dp, threadIdx.x);
+    S.table()[threadIdx.x] = make_float2(v, v);
+  }
+  __syncthreads();
+  const RowsGeom &rg = S.rec.rg;
+  const unsigned warp = threadIdx.x >> 5, task = S.rec.task + warp;
+  if (task >= (unsigned)rg.tasks) return;
+  const int from = parity ^ S.rec.off;
+  rows_task<T, kRowSteps>(static_cast<const T *>(S.rec.buf[from]),
+                          static_cast<T *>(S.rec.buf[from ^ 1]), S.rec.g, rg, S.constants(), task,
+                          threadIdx.x & 31, rows_smem + warp * rows_smem_words<T>(kRowSteps));
+}
+
+template <typename T>
+cudaError_t launch_rows_batch_t(const BatchList &bl, int parity, cudaStream_t st,
+                                const int *limits, int k) {
+  if (bl.nrows < 1) return cudaSuccess;
+  constexpr size_t smem = 2 * rows_smem_words<T>(kRowSteps) * sizeof(uint4) + sizeof(RowsShared<T>);
+  cudaError_t e = cudaFuncSetAttribute(
+      k_rows_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_rows_batch<T>, (unsigned)bl.nrows, 64, smem, st, bl.ents, bl.rows, bl.n,
+                    parity, limits, k);
 }
 
 // ------------------------------------------------------------------ tile

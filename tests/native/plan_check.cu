@@ -33,21 +33,29 @@ static void check(int nx, int ny, int dtype, int esize) {
   L.V = V;
   L.g = make_geom(nx, ny, V, esize);
   plan_lattice(L, sms);
-  // rows: strips of 1 .. 30 chunks, each chunk in one strip, at any rows
+  // rows: every chunk of every row is some task's own exactly once (lanes 1
+  // .. 30 of its 32 positions), for small lattices by enumeration
   for (int rows : {1, 8, 32}) {
-    const RowsGeom r = rows_geom(L.g, V, rows);
-    CHECK(r.width >= 1 && r.width <= 30, "width %d nx %d", r.width, nx);
-    // seam lanes of a ragged row: left halo (strip 0), partial chunk and
-    // right halo (last strip), each with an idle lane's slot of its own
-    if (nx % V != 0)
-      CHECK(32 - (std::min(r.width, L.g.nchunks) + 2) >= (r.strips == 1 ? 3 : 2), "idle lanes: width %d strips %d",
-            r.width, r.strips);
-    CHECK((long long)r.strips * r.width >= L.g.nchunks &&
-              (long long)(r.strips - 1) * r.width < L.g.nchunks,
-          "strips %d x %d for %d chunks", r.strips, r.width, L.g.nchunks);
+    const RowsGeom r = rows_geom(L.g, rows);
+    CHECK(r.rows >= 1 && r.segs >= 1 && (long long)r.segs * r.rows >= ny &&
+              (long long)(r.segs - 1) * r.rows < ny,
+          "segs %d x %d of %d rows", r.segs, r.rows, ny);
+    const int per = L.g.nchunks + 2;
+    if ((long long)nx * ny > 20000) continue;
+    std::vector<int> seen((size_t)r.segs * per, 0);
+    for (int t = 0; t < r.tasks; ++t)
+      for (int lane = 1; lane <= 30; ++lane) {
+        const long long p = 30LL * t + lane;
+        if (p < (long long)seen.size()) seen[(size_t)p]++;
+      }
+    for (size_t p = 0; p < seen.size(); ++p) {
+      const int c = (int)(p % per) - 1;
+      CHECK((c < 0 || c >= L.g.nchunks) ? seen[p] <= 1 : seen[p] == 1, "position %zu seen %d", p,
+            seen[p]);
+    }
   }
-  const RowsGeom r = plan_rows(L.g, V, sms * 12);
-  CHECK(r.rows >= 8 && r.rows <= 32, "rows %d", r.rows);
+  const RowsGeom r = plan_rows(L.g, sms * 12);
+  CHECK(r.rows >= 1 && r.rows <= 48, "rows %d", r.rows);
   double us = 0;
   const TileGeom t = plan_tile(L.g, esize, sms, &us);
   if (t.steps > 0) {

@@ -133,3 +133,77 @@ def test_init_rounds_the_fp64_deviations_once(L, amp, u0):
     finally:
         L.lbm_destroy(h)
         L.lbm_destroy(d)
+
+
+# members that together pass the size from which a batch's group takes three
+# steps per launch (FP32 and FP16; the BF16 pair stays below it)
+BATCH = [("f32", 700, 600), ("f32", 333, 1201), ("f32", 57, 9001), ("f32", 1000, 400),
+         ("f32", 20, 20), ("f16", 1201, 1000), ("f16", 801, 1500), ("f16", 330, 2500),
+         ("bf16", 130, 90), ("bf16", 61, 200)]
+
+
+def alone(L, dtype, nx, ny, f, steps):
+    h = L.lbm_create(nx, ny, RATES, 1.0, (0.0, 0.0), L.DTYPES[dtype])
+    try:
+        L.lbm_init_field(h, *f)
+        L.lbm_step(h, steps)
+        return L.lbm_get_populations(h), L.lbm_moments(h)
+    finally:
+        L.lbm_destroy(h)
+
+
+def test_batch_rows_equal_alone(L):
+    """Groups of three-step launches, of single steps and a resident member
+    in one batch, from either buffer and over calls of every remainder."""
+    fields = [inp.gaussian_pulse(nx, ny, 1e-3, 5.0, xc=3.0, yc=ny - 2.0) for _, nx, ny in BATCH]
+    hs, b = [], None
+    try:
+        for (dt, nx, ny), f in zip(BATCH, fields):
+            h = L.lbm_create(nx, ny, RATES, 1.0, (0.0, 0.0), L.DTYPES[dt])
+            L.lbm_init_field(h, *f)
+            hs.append(h)
+        L.lbm_step(hs[1], 1)  # one member starts on its other buffer
+        b = L.lbm_batch_create(hs)
+        for n in (1, 2, 3, 7, 69):
+            L.lbm_batch_step(b, n)
+        got = [L.lbm_get_populations(h) for h in hs]
+    finally:
+        if b is not None:
+            L.lbm_batch_destroy(b)
+        for h in hs:
+            L.lbm_destroy(h)
+    for k, ((dt, nx, ny), f) in enumerate(zip(BATCH, fields)):
+        want, _ = alone(L, dt, nx, ny, f, 82 + (k == 1))
+        assert np.array_equal(got[k], want), (k, dt, nx, ny)
+
+
+def test_served_generations_of_rows_equal_alone(L):
+    """A server's ragged generations: members stop after step counts of every
+    remainder, some inside a generation's last three-step launch."""
+    import time
+
+    steps = [5, 22, 23, 24, 9, 11, 31, 3, 1, 12]
+    fields = [inp.gaussian_pulse(nx, ny, 1e-3, 5.0, xc=2.0, yc=1.0) for _, nx, ny in BATCH]
+    s = L.lbm_server_create(2 ** 33, 11)
+    try:
+        ids, keep = [], []
+        for (dt, nx, ny), f, n in zip(BATCH, fields, steps):
+            req, kept = L.make_request(nx, ny, RATES, n, dtype=dt, init_kind=L.LBM_INIT_FIELDS,
+                                       fields=f)
+            keep.append(kept)
+            ids.append(L.lbm_submit(s, req))
+        got, t0 = {}, time.time()
+        while len(got) < len(ids) and time.time() - t0 < 120:
+            for k, rid in enumerate(ids):
+                if k not in got:
+                    rc, *out = L.lbm_poll(s, rid, BATCH[k][1], BATCH[k][2])
+                    if rc == L.LBM_OK:
+                        got[k] = out[:3]
+            time.sleep(0.01)
+    finally:
+        L.lbm_server_destroy(s)
+    assert len(got) == len(ids)
+    for k, ((dt, nx, ny), f) in enumerate(zip(BATCH, fields)):
+        _, want = alone(L, dt, nx, ny, f, steps[k])
+        for a, w in zip(got[k], want):
+            assert np.array_equal(a, w), (k, dt, nx, ny)
