@@ -658,18 +658,18 @@ static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms
     if (L.dtype != dt || b->member_res[mi]) continue;
     if (!rows_fit(L.g, L.V) || L.g.ny < kRowSteps) return recs;
     nodes += (double)L.g.nx * L.g.ny;
-    rows32 += rows_geom(L.g, 32).tasks;
+    rows32 += rows_geom(L.g, L.V, 32).tasks;
   }
   if (nodes < rows_min_nodes(dt == LBM_F32DEV ? 4 : 2)) return recs;
   // 32 rows per task, or 16 where that leaves fewer than six tasks per
   // resident warp and the tail would weigh
-  const int rows = rows32 < 6.0 * sms * rows_warps(dt == LBM_F32DEV ? 4 : 2) ? 16 : 32;
+    const int rows = rows32 < 6.0 * sms * rows_warps(dt == LBM_F32DEV ? 4 : 2) ? 16 : 32;
   for (size_t mi = 0; mi < b->members.size(); ++mi) {
     const Lattice &L = b->members[mi]->L;
     if (L.dtype != dt || b->member_res[mi]) continue;
     RowsRec r;
     r.g = L.g;
-    r.rg = rows_geom(L.g, rows);
+    r.rg = rows_geom(L.g, L.V, rows);
     r.buf[0] = L.buf[0];
     r.buf[1] = L.buf[1];
     r.lat = b->member_local[mi];

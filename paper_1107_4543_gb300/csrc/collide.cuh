@@ -205,11 +205,19 @@ __host__ __device__ __forceinline__ float pair_const(const DevParams &P, int c) 
   }
 }
 
+// two constants (collide_pair takes them k, k + 1 with k even: a source in
+// shared memory reads both with one 16-byte load)
+struct F2x2 {
+  F2 a, b;
+};
+
 // The constants straight from a DevParams (kernel parameters of a single
 // lattice, or an entry in global memory)
 struct ParamPairs {
   const DevParams &P;
-  __device__ __forceinline__ F2 operator()(PairConst c) const { return f2s(pair_const(P, c)); }
+  __device__ __forceinline__ F2x2 two(PairConst c) const {
+    return {f2s(pair_const(P, c)), f2s(pair_const(P, c + 1))};
+  }
 };
 
 // collide_dev<false, SCALED> for two nodes, one per lane of the F2 values:
@@ -232,12 +240,13 @@ __device__ __forceinline__ void collide_pair(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2
   const F2 jx_p = d13 + dxd;
   const F2 jy_p = d24 + dyd;
 
-  const F2 IS = P(PC_IS);
+  const F2x2 c0 = P.two(PC_IS), c2j = P.two(PC_2JX), cj = P.two(PC_JX);
+  const F2 IS = c0.a, R0 = c0.b;
   const F2 rho_phys = SCALED ? rho_p * IS : rho_p;
   // -rho'/rho per lane by the hardware reciprocal (the sign folded into
   // the numerator, which is exact): rho' * rcp(rho) without __fdividef's
   // handling of denominators above 2^126, the same bits below
-  const F2 den = P(PC_R0) + rho_phys;
+  const F2 den = R0 + rho_phys;
   float rl, rh, dl, dh;
   f2split(rho_phys, rl, rh);
   f2split(den, dl, dh);
@@ -248,13 +257,14 @@ __device__ __forceinline__ void collide_pair(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2
     jyy = jyy * IS;
     jxy = jxy * IS;
   }
-  const F2 tx = fma2(P(PC_2JX), jx_p, jxx);  // jx^2 - jx0^2
-  const F2 ty = fma2(P(PC_2JY), jy_p, jyy);
-  const F2 txy = fma2(P(PC_JX), jy_p, fma2(jx_p, P(PC_JY), jxy));
-  const F2 R0 = P(PC_R0), I2 = P(PC_I2);
-  const F2 nj = fma2(R0, tx + ty, rho_p * P(PC_NQ0)) * I2;
-  const F2 np = fma2(R0, tx - ty, rho_p * P(PC_ND0)) * I2;
-  const F2 nx = fma2(R0, txy, rho_p * P(PC_NX0)) * I2;
+  const F2 tx = fma2(c2j.a, jx_p, jxx);  // jx^2 - jx0^2
+  const F2 ty = fma2(c2j.b, jy_p, jyy);
+  const F2 txy = fma2(cj.a, jy_p, fma2(jx_p, cj.b, jxy));
+  const F2x2 ci = P.two(PC_I2), cn = P.two(PC_ND0);
+  const F2 I2 = ci.a;
+  const F2 nj = fma2(R0, tx + ty, rho_p * ci.b) * I2;
+  const F2 np = fma2(R0, tx - ty, rho_p * cn.a) * I2;
+  const F2 nx = fma2(R0, txy, rho_p * cn.b) * I2;
   const F2 djsq = fma2(nj, nc, nj);  // |j|^2/rho - |j0|^2/rho0
   const F2 dpxx = fma2(np, nc, np);
   const F2 dpxy = fma2(nx, nc, nx);
@@ -266,12 +276,13 @@ __device__ __forceinline__ void collide_pair(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2
   const F2 m6 = fma2(f2s(-2.0f), dyd, d24);
   const F2 n7 = (s13 - s24) - dpxx;
   const F2 n8 = (s57 - s68) - dpxy;
-  const F2 r3 = n3 * P(PC_K3);
-  const F2 r4 = n4 * P(PC_K4);
-  const F2 r5 = m5 * P(PC_NK5);
-  const F2 r6 = m6 * P(PC_NK6);
-  const F2 r7 = n7 * P(PC_K7);
-  const F2 r8 = n8 * P(PC_K8);
+  const F2x2 k34 = P.two(PC_K3), k56 = P.two(PC_NK5), k78 = P.two(PC_K7);
+  const F2 r3 = n3 * k34.a;
+  const F2 r4 = n4 * k34.b;
+  const F2 r5 = m5 * k56.a;
+  const F2 r6 = m6 * k56.b;
+  const F2 r7 = n7 * k78.a;
+  const F2 r8 = n8 * k78.b;
 
   const F2 TWO = f2s(2.0f), NTWO = f2s(-2.0f);
   const F2 a = fma2(TWO, r4, r3);  // axis velocities: -r3 - 2 r4
@@ -293,7 +304,7 @@ __device__ __forceinline__ void collide_pair(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2
 // (collide_dev's PRECISE form), each broadcast to both lanes of a pair,
 // doublings and negations folded in (exact).
 enum HlConst {
-  HL_R0, HL_2JX, HL_2JY, HL_JX, HL_JY,               // rho0, 2 j0, j0
+  HL_R0, HL_2JX, HL_2JY, HL_JX, HL_JY, HL_PAD,       // rho0, 2 j0, j0
   HL_NQ0H, HL_NQ0L, HL_ND0H, HL_ND0L, HL_NX0H, HL_NX0L,  // -|j0|^2, ...
   HL_I2H, HL_I2L,                                    // 1 / rho0^2
   HL_K3H, HL_K3L, HL_K4H, HL_K4L, HL_NK5H, HL_NK5L,  // rates / D
@@ -307,7 +318,8 @@ __host__ __device__ __forceinline__ float hl_const(const DevParams &P, int c) {
     case HL_2JX: return 2.0f * P.jx0;
     case HL_2JY: return 2.0f * P.jy0;
     case HL_JX: return P.jx0;
-    case HL_JY: return P.jy0;
+    case HL_JY:
+    case HL_PAD: return P.jy0;
     case HL_NQ0H: return -P.q0h;
     case HL_NQ0L: return -P.q0l;
     case HL_ND0H: return -P.d0h;
@@ -331,10 +343,14 @@ __host__ __device__ __forceinline__ float hl_const(const DevParams &P, int c) {
   }
 }
 
-// the broadcast pairs, as a kernel parameter or in shared memory
-struct HlPairs {
+// the broadcast pairs, as a kernel parameter or in shared memory; two(k), k
+// even, reads constants k and k + 1 with one 16-byte load
+struct alignas(16) HlPairs {
   float2 c[HL_COUNT];
-  __device__ __forceinline__ F2 operator()(HlConst k) const { return f2(c[k].x, c[k].y); }
+  __device__ __forceinline__ F2x2 two(HlConst k) const {
+    const float4 v = *reinterpret_cast<const float4 *>(c + k);
+    return {f2(v.x, v.y), f2(v.z, v.w)};
+  }
 };
 
 inline HlPairs hl_pairs(const DevParams &P) {
@@ -344,7 +360,7 @@ inline HlPairs hl_pairs(const DevParams &P) {
 }
 
 // a * (h + l), as mul_hl<true>
-__device__ __forceinline__ F2 mul_hl2(F2 a, F2 h, F2 l) { return fma2(a, h, a * l); }
+__device__ __forceinline__ F2 mul_hl2(F2 a, const F2x2 &k) { return fma2(a, k.a, a * k.b); }
 
 // collide_dev<true, false> (FP32 storage) for two nodes, one per lane: the
 // same operations in the same order, so each lane's result equals the scalar
@@ -366,19 +382,20 @@ __device__ __forceinline__ void collide_pair_hl(F2 &f0, F2 &f1, F2 &f2_, F2 &f3,
   const F2 jy_p = d24 + dyd;
 
   // -rho'/rho per lane (the sign folded into the numerator, exact)
-  const F2 R0 = P(HL_R0);
+  const F2x2 c0 = P.two(HL_R0), c1 = P.two(HL_2JY);  // rho0, 2 jx0; 2 jy0, jx0
+  const F2 R0 = c0.a;
   const F2 den = R0 + rho_p;
   float rl, rh, dl, dh;
   f2split(rho_p, rl, rh);
   f2split(den, dl, dh);
   const F2 nc = f2(-rl * rcp_approx(dl), -rh * rcp_approx(dh));
-  const F2 tx = fma2(P(HL_2JX), jx_p, jx_p * jx_p);
-  const F2 ty = fma2(P(HL_2JY), jy_p, jy_p * jy_p);
-  const F2 txy = fma2(P(HL_JX), jy_p, fma2(jx_p, P(HL_JY), jx_p * jy_p));
-  const F2 I2H = P(HL_I2H), I2L = P(HL_I2L);
-  const F2 nj = mul_hl2(fma2(R0, tx + ty, mul_hl2(rho_p, P(HL_NQ0H), P(HL_NQ0L))), I2H, I2L);
-  const F2 np = mul_hl2(fma2(R0, tx - ty, mul_hl2(rho_p, P(HL_ND0H), P(HL_ND0L))), I2H, I2L);
-  const F2 nx = mul_hl2(fma2(R0, txy, mul_hl2(rho_p, P(HL_NX0H), P(HL_NX0L))), I2H, I2L);
+  const F2 tx = fma2(c0.b, jx_p, jx_p * jx_p);
+  const F2 ty = fma2(c1.a, jy_p, jy_p * jy_p);
+  const F2 txy = fma2(c1.b, jy_p, fma2(jx_p, P.two(HL_JY).a, jx_p * jy_p));
+  const F2x2 i2 = P.two(HL_I2H);
+  const F2 nj = mul_hl2(fma2(R0, tx + ty, mul_hl2(rho_p, P.two(HL_NQ0H))), i2);
+  const F2 np = mul_hl2(fma2(R0, tx - ty, mul_hl2(rho_p, P.two(HL_ND0H))), i2);
+  const F2 nx = mul_hl2(fma2(R0, txy, mul_hl2(rho_p, P.two(HL_NX0H))), i2);
   const F2 djsq = fma2(nj, nc, nj);
   const F2 dpxx = fma2(np, nc, np);
   const F2 dpxy = fma2(nx, nc, nx);
@@ -390,12 +407,12 @@ __device__ __forceinline__ void collide_pair_hl(F2 &f0, F2 &f1, F2 &f2_, F2 &f3,
   const F2 m6 = fma2(NTWO, dyd, d24);
   const F2 n7 = (s13 - s24) - dpxx;
   const F2 n8 = (s57 - s68) - dpxy;
-  const F2 r3 = mul_hl2(n3, P(HL_K3H), P(HL_K3L));
-  const F2 r4 = mul_hl2(n4, P(HL_K4H), P(HL_K4L));
-  const F2 r5 = mul_hl2(m5, P(HL_NK5H), P(HL_NK5L));
-  const F2 r6 = mul_hl2(m6, P(HL_NK6H), P(HL_NK6L));
-  const F2 r7 = mul_hl2(n7, P(HL_K7H), P(HL_K7L));
-  const F2 r8 = mul_hl2(n8, P(HL_K8H), P(HL_K8L));
+  const F2 r3 = mul_hl2(n3, P.two(HL_K3H));
+  const F2 r4 = mul_hl2(n4, P.two(HL_K4H));
+  const F2 r5 = mul_hl2(m5, P.two(HL_NK5H));
+  const F2 r6 = mul_hl2(m6, P.two(HL_NK6H));
+  const F2 r7 = mul_hl2(n7, P.two(HL_K7H));
+  const F2 r8 = mul_hl2(n8, P.two(HL_K8H));
 
   const F2 a = fma2(TWO, r4, r3);
   const F2 b = fma2(TWO, r3, r4);

@@ -39,10 +39,10 @@ struct DevGuard {
 
 // Work split of the kernels that advance several steps per launch
 // (step_multi.cuh; chosen in plan.h).
-// k_step_rows: `segs` segments of `rows` rows, `tasks` warp tasks of 30 lane
-// positions
+// k_step_rows: `segs` segments of `rows` rows, `tasks` warp tasks of 32 lanes
+// of which `halo` on each side are
 struct RowsGeom {
-  int rows, segs, tasks;
+  int rows, segs, halo, tasks;
 };
 // k_step_tile: tiles of bx x by nodes, at most `steps` steps per launch
 struct TileGeom {

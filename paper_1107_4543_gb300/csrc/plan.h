@@ -8,31 +8,33 @@
 namespace lbm {
 
 // k_step_rows: segments of about `rows` rows, as even as they go, each a
-// sequence of nchunks + 2 lane positions, 30 positions to a task (the first
-// position, a halo, is no task's own).
-inline RowsGeom rows_geom(const Geom &g, int rows) {
+// sequence of nchunks + 2 halo lane positions, 32 - 2 halo of them to a task
+// (the first ones, halo, are no task's own).
+inline RowsGeom rows_geom(const Geom &g, int V, int rows) {
   RowsGeom r;
   r.segs = std::max(1, (g.ny + rows / 2) / rows);
   r.rows = (g.ny + r.segs - 1) / r.segs;
   r.segs = (g.ny + r.rows - 1) / r.rows;
-  const long long pos = (long long)r.segs * (g.nchunks + 2);
-  r.tasks = (int)std::min<long long>((pos - 2 + 29) / 30, 1 << 30);
+  r.halo = g.nx % V != 0 && g.nx % V < kRowSteps ? 2 : 1;
+  const int own = 32 - 2 * r.halo;
+  const long long pos = (long long)r.segs * (g.nchunks + 2 * r.halo);
+  r.tasks = (int)std::min<long long>((pos - 2 * r.halo + own - 1) / own, 1 << 30);
   return r;
 }
 
-// whether k_step_rows takes the lattice: its seam chunks are assembled from
-// whole neighbouring chunks, and its positions are 32-bit
+// whether k_step_rows takes the lattice: its halo chunks are chunks of their
+// own, and its positions are 32-bit
 inline bool rows_fit(const Geom &g, int V) {
-  return (g.nx % V == 0 || g.nchunks >= 3) && (double)g.ny * (g.nchunks + 2) < 4e9;
+  return (g.nx % V == 0 || g.nchunks >= 3) && (double)g.ny * (g.nchunks + 4) < 4e9;
 }
 
 // Rows per segment: 32 cost 2 (kRowSteps - 1) / 32 of redundant level-1 rows;
 // fewer where the tasks would not fill the resident warps (`slots`) a
 // quarter more than once (2048^2 FP32: 16 rows 23.2 us per step, 32 rows
 // 31.1, 8 rows 24.9).
-inline RowsGeom plan_rows(const Geom &g, int slots) {
+inline RowsGeom plan_rows(const Geom &g, int V, int slots) {
   const double fit = (double)g.ny * (g.nchunks + 2) / 30.0 / (1.25 * slots);
-  return rows_geom(g, (int)std::max(8.0, std::min(32.0, fit)));
+  return rows_geom(g, V, (int)std::max(8.0, std::min(32.0, fit)));
 }
 
 // k_step_tile: the split of least estimated time per step with all tiles
@@ -86,7 +88,7 @@ inline void plan_lattice(Lattice &L, int sms) {
     L.tile = t;
   } else if (nodes >= rows_min_nodes(L.esize) && rows_fit(L.g, L.V)) {
     L.plan = PLAN_ROWS;
-    L.rows = plan_rows(L.g, sms * rows_warps(L.esize));
+    L.rows = plan_rows(L.g, L.V, sms * rows_warps(L.esize));
   }
 }
 

@@ -47,7 +47,9 @@ static __constant__ DevParams c_dev[kDevTable];
 
 struct ConstPairs {
   int base;  // first constant of the lattice: slot * PC_COUNT
-  __device__ __forceinline__ F2 operator()(PairConst c) const { return f2s(c_pairs[base + c]); }
+  __device__ __forceinline__ F2x2 two(PairConst c) const {
+    return {f2s(c_pairs[base + c]), f2s(c_pairs[base + c + 1])};
+  }
 };
 
 // 16-bit storage: unpack / collide / repack the packed populations two

@@ -38,8 +38,11 @@ inline typename PairParams<T>::type pair_params(const DevParams &P) {
 
 // 16-bit constants as broadcast pairs in shared memory (PairConst order)
 struct SharedPairs {
-  const float2 *c;
-  __device__ __forceinline__ F2 operator()(PairConst k) const { return f2(c[k].x, c[k].y); }
+  const float2 *c;  // 16-byte aligned
+  __device__ __forceinline__ F2x2 two(PairConst k) const {
+    const float4 v = *reinterpret_cast<const float4 *>(c + k);
+    return {f2(v.x, v.y), f2(v.z, v.w)};
+  }
 };
 
 // two nodes of a storage type (the FP32 values, or the unpacked 16-bit ones)
@@ -53,13 +56,37 @@ __device__ __forceinline__ void collide_two(F2 (&f)[9], const K &P) {
 }
 
 // ------------------------------------------------------------------ rows
+// The end of a row whose last chunk is partial: that chunk's lane hands its
+// last real node, element el, to the next lane (chunk 0) and takes that
+// lane's node 0 after it.  `warp`: some lane of the warp holds such a chunk
+// (warp-uniform, so the other warps skip the selects).
+struct Seam {
+  bool warp, last;
+  int el;
+  // all ones for this lane's word that holds element el (a comparison per
+  // word instead is turned into an indexed array in local memory, at half
+  // the speed), and the shift that brings a 16-bit el to the word's high half
+  uint32_t word[4];
+  int up;
+};
+
 // One lane's chunk of a plane (V nodes as four words) shifted by the x
 // component of the plane's velocity: the missing element comes from the
 // neighbouring lane, whose chunk is the neighbouring one.
 template <typename T>
-__device__ __forceinline__ void shift_chunk(uint32_t (&w)[4], int cx) {
+__device__ __forceinline__ void shift_chunk(uint32_t (&w)[4], int cx, const Seam &S) {
   if (cx == 1) {
-    const uint32_t prev = __shfl_up_sync(0xffffffffu, w[3], 1);
+    uint32_t tail = w[3];
+    if (S.warp) {
+      uint32_t own = 0, any = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        own |= w[q] & S.word[q];
+        any |= S.word[q];
+      }
+      tail = ((tail & ~any) | own) << S.up;
+    }
+    const uint32_t prev = __shfl_up_sync(0xffffffffu, tail, 1);
     if constexpr (sizeof(T) == 4) {
       w[3] = w[2]; w[2] = w[1]; w[1] = w[0]; w[0] = prev;
     } else {
@@ -77,6 +104,19 @@ __device__ __forceinline__ void shift_chunk(uint32_t (&w)[4], int cx) {
       w[1] = __byte_perm(w[1], w[2], 0x5432);
       w[2] = __byte_perm(w[2], w[3], 0x5432);
       w[3] = __byte_perm(w[3], next, 0x5432);
+    }
+    if (S.warp) {
+      // node 0 takes the element after the last one
+      uint32_t keep = 0, put = next;
+      if constexpr (sizeof(T) == 2) {
+        keep = (S.el & 1) ? 0xffffu : 0xffff0000u;
+        put = (S.el & 1) ? next << 16 : next & 0xffffu;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t m = S.word[q] & ~keep;
+        w[q] = (w[q] & ~m) | (put & m);
+      }
     }
   }
 }
@@ -124,47 +164,22 @@ __device__ __forceinline__ void cp_async16(uint4 *smem, const void *g) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(g) : "memory");
 }
-__device__ __forceinline__ void cp_async4(void *smem, const void *g) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(g) : "memory");
-}
-
-// 16-bit types: elements sh .. sh + 7 of chunks *a, *b (shared memory) laid
-// end to end, the first `keep` of them replaced by w's.
-__device__ __forceinline__ void seam_chunk(uint32_t (&w)[4], const uint4 *a, int ab, int sh,
-                                           int keep) {
-  const uint32_t *p = reinterpret_cast<const uint32_t *>(a);
-  const int k0 = sh / 2, far = 4 * ab - 4;  // b is ab 16-byte words after a
-  uint32_t v[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    const int k = k0 + q;  // at most 8, which an even shift ignores
-    v[q] = p[k < 4 ? k : min(k, 7) + far];
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint32_t u = (sh & 1) ? __byte_perm(v[q], v[q + 1], 0x5432) : v[q];
-    const uint32_t own = 2 * q + 1 < keep ? 0xffffffffu : (2 * q < keep ? 0xffffu : 0u);
-    w[q] = (w[q] & own) | (u & ~own);
-  }
-}
-
-// shared memory of one warp of k_step_rows, in 16-byte words: two stages of
-// 9 incoming vectors, per level boundary 3 delayed by one row and 3 by two
-// rows, and for the 16-bit types the seam lanes' second chunks, for 32 lanes
-template <typename T>
-constexpr int rows_smem_words(int steps) {
-  return (18 + 9 * (steps - 1) + (sizeof(T) == 2 ? 18 : 0)) * 32;
-}
+// shared memory of one warp of k_step_rows, in 16-byte words: 9 incoming
+// vectors and, per level boundary, 3 delayed by one row and 3 by two rows,
+// for 32 lanes
+constexpr int rows_smem_words(int steps) { return (9 + 9 * (steps - 1)) * 32; }
 
 // The lattice's rows are cut into segments of rg.rows; a segment is a
-// sequence of nchunks + 2 lane positions (the chunk before chunk 0, chunks 0
-// .. nchunks - 1, the chunk after the last, taken periodically), the
-// segments' sequences follow one another, and task t takes positions 30 t ..
-// 30 t + 31: its lanes 1 .. 30 advance their chunks, each with its
-// neighbours in the neighbouring lanes, lanes 0 and 31 are halo, and a warp
-// spans segments freely.  (Strips of whole warps left 20% of the lanes of
-// the 128-lattice FP32 sweep idle and 27% in FP16.)
+// sequence of halo + nchunks + halo lane positions (the chunks before chunk
+// 0, chunks 0 .. nchunks - 1, those after the last, taken periodically), the
+// segments' sequences follow one another, and task t takes the 32 positions
+// from (32 - 2 halo) t: its middle lanes advance their chunks, each with its
+// neighbours in the neighbouring lanes, and a warp spans segments freely.
+// (Strips of whole warps left 20% of the lanes of the 128-lattice FP32 sweep
+// idle and 27% in FP16.)  halo is 1 lane, or 2 where a partial last chunk
+// has fewer nodes than the launch has steps.  (Making the chunks around the
+// end of such a row whole instead, by element-wise copies or by assembling
+// two aligned chunks, cost 25 - 35% of the rate of ragged FP32 lattices.)
 //
 // After each level one more node of each halo chunk is invalid, so STEPS <=
 // V levels leave the own chunks exact; in y each level loses one row per
@@ -173,41 +188,38 @@ constexpr int rows_smem_words(int steps) {
 // level l the row l - 1 below it: its populations with c_y = -1 come from
 // the row just computed (registers), those with c_y = 0 from the iteration
 // before and those with c_y = +1 from two before (the delay slots, which
-// only this lane touches: no synchronization).  Incoming rows are copied to
-// shared memory one iteration ahead (cp.async), so no register holds a load
+// only this lane touches: no synchronization).  The next incoming row is copied to
+// shared memory (cp.async) as soon as this one's values have been shifted --
+// consumed, so the lane's own slots are free -- and no register holds a load
 // in flight: with the loads in registers the compiler spilled (FP32 152
 // bytes at 168 registers) and the two-step form ran at 125 instead of 174
 // GLUPS.
 //
-// Where V does not divide the row length, three chunks of a row lie across
-// its end (the one before node 0, the partial last one, the one after it).
-// Their lanes copy four elements one by one (FP32), or two aligned chunks
-// and assemble them (16 bits: an element is smaller than any copy).
 template <typename T, int STEPS, typename K>
 __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restrict__ dst,
                                           const Geom &g, const RowsGeom &rg, const K &par,
                                           unsigned task, int lane, uint4 *sm) {
   constexpr int V = Elem<T>::V;
   static_assert(STEPS >= 2 && STEPS <= V, "the halo chunk covers V nodes");
-  const unsigned per = (unsigned)g.nchunks + 2u, pos = task * 30u + (unsigned)lane;
+  const int H = rg.halo;
+  const unsigned per = (unsigned)(g.nchunks + 2 * H);
+  const unsigned pos = task * (unsigned)(32 - 2 * H) + (unsigned)lane;
   unsigned seg = pos / per;
-  const int vc = (int)(pos - seg * per) - 1, vx = vc * V;  // chunk, first virtual node
+  const int vc = (int)(pos - seg * per) - H;  // chunk before the wrap
   const bool in = seg < (unsigned)rg.segs;
   if (!in) seg = 0;
-  const bool out = in && lane >= 1 && lane <= 30 && vc >= 0 && vc < g.nchunks;
+  const bool out = in && lane >= H && lane < 32 - H && vc >= 0 && vc < g.nchunks;
   const int y0 = (int)seg * rg.rows, y1 = min(y0 + rg.rows, g.ny);
-  const int part = g.nx & (V - 1);  // nodes of a partial last chunk (0: none)
-  const bool seam = in && part != 0 && (vc < 0 || vc >= g.nchunks - 1);
-  int ca = vc < 0 ? vc + g.nchunks : (vc >= g.nchunks ? vc - g.nchunks : vc);
-  // 16 bits: element e of a seam chunk is element e + sh of chunks ca, cb
-  // laid end to end (a partial last chunk keeps its own first `part`)
-  int cb = 0, sh = 0;
-  if (sizeof(T) == 2 && seam) {
-    sh = vc < 0 ? part : V - part;
-    if (vc < 0) ca = g.nchunks - 2;
-    cb = vc < 0 ? g.nchunks - 1 : (vc == g.nchunks ? 1 : 0);
-  }
-  const int x0 = sizeof(T) == 4 && seam ? 0 : ca * V;
+  const int c = vc < 0 ? vc + g.nchunks : (vc >= g.nchunks ? vc - g.nchunks : vc);
+  const int x0 = c * V;
+  Seam S;
+  S.el = (g.nx - 1) & (V - 1);
+  S.last = c == g.nchunks - 1;
+  S.warp = S.el != V - 1 && __any_sync(0xffffffffu, S.last);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    S.word[q] = S.last && S.el * (int)sizeof(T) / 4 == q ? 0xffffffffu : 0u;
+  S.up = sizeof(T) == 2 && S.last && !(S.el & 1) ? 16 : 0;
   const int ya = y0 - (STEPS - 1);
   const int n = rg.rows + 2 * (STEPS - 1);
   auto row_of = [&](int y) -> const T * {
@@ -215,34 +227,15 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
     while (y >= g.ny) y -= g.ny;
     return src + (long long)y * g.rstride;
   };
-  constexpr int kB = (18 + 9 * (STEPS - 1)) * 32;  // the second chunks
-  uint4 *raw = sm + lane, *dly = sm + 18 * 32 + lane;
+  uint4 *raw = sm + lane, *dly = sm + 9 * 32 + lane;
   const T *pm = row_of(ya - 1) + x0, *pc = row_of(ya) + x0, *pp = row_of(ya + 1) + x0;
   int fetched = 0;
-  auto fetch = [&]() {  // level 1's row ya + fetched into stage fetched & 1
+  auto fetch = [&]() {  // level 1's row ya + fetched
     if (fetched < n) {
-      uint4 *q = raw + (fetched & 1) * (9 * 32);
-      auto from = [&](int i) {
-        return (CYd(i) == 1 ? pm : (CYd(i) == -1 ? pp : pc)) + (long long)i * g.plane;
-      };
-      if (in && !(sizeof(T) == 4 && seam)) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) cp_async16(q + i * 32, from(i));
-      }
-      if (seam) {
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            int x = vx + e;
-            x = x < 0 ? x + g.nx : (x >= g.nx ? x - g.nx : x);
-#pragma unroll
-            for (int i = 0; i < 9; ++i)
-              cp_async4(reinterpret_cast<uint32_t *>(q + i * 32) + e, from(i) + x);
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 9; ++i) cp_async16(q + kB + i * 32, from(i) + (cb - ca) * V);
-        }
+      for (int i = 0; i < 9; ++i) {
+        const T *row = CYd(i) == 1 ? pm : (CYd(i) == -1 ? pp : pc);
+        cp_async16(raw + i * 32, row + (long long)i * g.plane);
       }
       ++fetched;
       pm = pc;
@@ -252,24 +245,16 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   fetch();
-  T *drow = dst + (long long)y0 * g.rstride + (out ? vx : 0);
-  const bool fill = (g.nchunks & 1) && out && vc == g.nchunks - 1;  // see fills_sector
+  T *drow = dst + (long long)y0 * g.rstride + x0;
+  const bool fill = (g.nchunks & 1) && out && S.last;  // see fills_sector
   for (int j = 0; j < n; ++j) {
-    fetch();
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     uint32_t w[9][4];
-    {
-      const uint4 *q = raw + (j & 1) * (9 * 32);
 #pragma unroll
-      for (int i = 0; i < 9; ++i) set4(w[i], q[i * 32]);
-      if (sizeof(T) == 2 && seam) {
+    for (int i = 0; i < 9; ++i) set4(w[i], raw[i * 32]);
 #pragma unroll
-        for (int i = 0; i < 9; ++i)
-          seam_chunk(w[i], q + i * 32, kB, sh, vc == g.nchunks - 1 ? part : 0);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) shift_chunk<T>(w[i], CXd(i));
+    for (int i = 0; i < 9; ++i) shift_chunk<T>(w[i], CXd(i), S);
+    fetch();
     collide_chunk<T>(w, par);
 #pragma unroll
     for (int l = 1; l < STEPS; ++l) {
@@ -287,7 +272,7 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
 #pragma unroll
           for (int q = 0; q < 4; ++q) w[i][q] = u[i][q];
         }
-        shift_chunk<T>(w[i], CXd(i));
+        shift_chunk<T>(w[i], CXd(i), S);
       }
       collide_chunk<T>(w, par);
     }
@@ -307,17 +292,20 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
   }
 }
 
-// Register budgets: 64-thread blocks, 168 registers (FP32; no spills, 12
-// warps per SM) or 255 (16 bits: 224, 8 warps; at 168 it spills 24 bytes).
+// Register budgets, 64-thread blocks: FP32 128 (116 used; 16 warps per SM,
+// which their 13.8 KB of shared memory per warp allows too), 16 bits 255
+// (210 used, 8 warps; at 168 registers, 12 warps, they spill and run 4097 x
+// 3071 FP16 at 6.5 instead of 5.5 ms per 100 steps).  The FMA pipe is 70%
+// busy on 8192^2 FP32 (251 GLUPS), with 54% of the issue slots used.
 template <typename T, int STEPS>
-__global__ void __launch_bounds__(64, sizeof(T) == 4 ? 6 : 4)
+__global__ void __launch_bounds__(64, sizeof(T) == 4 ? 8 : 4)
 k_step_rows(const T *__restrict__ src, T *__restrict__ dst, Geom g, RowsGeom rg,
             typename PairParams<T>::type P, unsigned ntasks) {
   extern __shared__ uint4 rows_smem[];
   const unsigned warp = threadIdx.x >> 5, task = blockIdx.x * 2 + warp;
   pdl_wait();
   if (task >= ntasks) return;
-  uint4 *sm = rows_smem + warp * rows_smem_words<T>(STEPS);
+  uint4 *sm = rows_smem + warp * rows_smem_words(STEPS);
   if constexpr (sizeof(T) == 4)
     rows_task<T, STEPS>(src, dst, g, rg, P, task, threadIdx.x & 31, sm);
   else
@@ -326,7 +314,7 @@ k_step_rows(const T *__restrict__ src, T *__restrict__ dst, Geom g, RowsGeom rg,
 
 template <typename T, int STEPS>
 cudaError_t launch_rows_steps(const Lattice &L, const void *src, void *dst, cudaStream_t st) {
-  constexpr size_t smem = 2 * rows_smem_words<T>(STEPS) * sizeof(uint4);
+  constexpr size_t smem = 2 * rows_smem_words(STEPS) * sizeof(uint4);
   cudaError_t e = cudaFuncSetAttribute(
       k_step_rows<T, STEPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;
@@ -346,20 +334,12 @@ cudaError_t launch_rows_t(const Lattice &L, const void *src, void *dst, cudaStre
 
 // The batched form: every block reads its lattice's record and collision
 // constants into shared memory (a lattice's constants cannot be kernel
-// parameters here, and 25 broadcast pairs in registers would spill), then
-// its two warps take one task each.
-template <typename T> struct RowsShared;
-template <> struct RowsShared<float> {
-  RowsRec rec;
-  HlPairs pairs;
-  static constexpr int COUNT = HL_COUNT;
-  static __device__ __forceinline__ float value(const DevParams &P, int k) { return hl_const(P, k); }
-  __device__ __forceinline__ float2 *table() { return pairs.c; }
-  __device__ __forceinline__ const HlPairs &constants() const { return pairs; }
-};
+// parameters here, and 25 broadcast pairs in registers would spill; read in
+// pairs of 16 bytes: one by one the 128-lattice FP32 sweep took 52.9 instead
+// of 49.3 ms), then its two warps take one task each.
 template <typename T> struct RowsShared {
   RowsRec rec;
-  float2 c[PC_COUNT];
+  alignas(16) float2 c[PC_COUNT];
   static constexpr int COUNT = PC_COUNT;
   static __device__ __forceinline__ float value(const DevParams &P, int k) {
     return pair_const(P, k);
@@ -368,13 +348,22 @@ template <typename T> struct RowsShared {
   __device__ __forceinline__ SharedPairs constants() const { return SharedPairs{c}; }
 };
 
+template <> struct RowsShared<float> {
+  RowsRec rec;
+  HlPairs pairs;
+  static constexpr int COUNT = HL_COUNT;
+  static __device__ __forceinline__ float value(const DevParams &P, int k) { return hl_const(P, k); }
+  __device__ __forceinline__ float2 *table() { return pairs.c; }
+  __device__ __forceinline__ const HlPairs &constants() const { return pairs; }
+};
+
 template <typename T>
-__global__ void __launch_bounds__(64, sizeof(T) == 4 ? 6 : 4)
+__global__ void __maxnreg__(sizeof(T) == 4 ? 168 : 255)
 k_rows_batch(const BatchEntry *__restrict__ ents, const RowsRec *__restrict__ recs, int nents,
              int parity, const int *__restrict__ limits, int k) {
   extern __shared__ uint4 rows_smem[];
   RowsShared<T> &S =
-      *reinterpret_cast<RowsShared<T> *>(rows_smem + 2 * rows_smem_words<T>(kRowSteps));
+      *reinterpret_cast<RowsShared<T> *>(rows_smem + 2 * rows_smem_words(kRowSteps));
   constexpr int NW = sizeof(RowsRec) / 4;
   static_assert(sizeof(RowsRec) % 4 == 0 && NW <= 64, "a record is copied one word per thread");
   if (threadIdx.x < NW)
@@ -396,14 +385,14 @@ k_rows_batch(const BatchEntry *__restrict__ ents, const RowsRec *__restrict__ re
   const int from = parity ^ S.rec.off;
   rows_task<T, kRowSteps>(static_cast<const T *>(S.rec.buf[from]),
                           static_cast<T *>(S.rec.buf[from ^ 1]), S.rec.g, rg, S.constants(), task,
-                          threadIdx.x & 31, rows_smem + warp * rows_smem_words<T>(kRowSteps));
+                          threadIdx.x & 31, rows_smem + warp * rows_smem_words(kRowSteps));
 }
 
 template <typename T>
 cudaError_t launch_rows_batch_t(const BatchList &bl, int parity, cudaStream_t st,
                                 const int *limits, int k) {
   if (bl.nrows < 1) return cudaSuccess;
-  constexpr size_t smem = 2 * rows_smem_words<T>(kRowSteps) * sizeof(uint4) + sizeof(RowsShared<T>);
+  constexpr size_t smem = 2 * rows_smem_words(kRowSteps) * sizeof(uint4) + sizeof(RowsShared<T>);
   cudaError_t e = cudaFuncSetAttribute(
       k_rows_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;

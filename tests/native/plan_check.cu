@@ -33,28 +33,30 @@ static void check(int nx, int ny, int dtype, int esize) {
   L.V = V;
   L.g = make_geom(nx, ny, V, esize);
   plan_lattice(L, sms);
-  // rows: every chunk of every row is some task's own exactly once (lanes 1
-  // .. 30 of its 32 positions), for small lattices by enumeration
+  // rows: every chunk of every row is some task's own exactly once (its lanes
+  // but `halo` on each side), for small lattices by enumeration
   for (int rows : {1, 8, 32}) {
-    const RowsGeom r = rows_geom(L.g, rows);
+    const RowsGeom r = rows_geom(L.g, V, rows);
     CHECK(r.rows >= 1 && r.segs >= 1 && (long long)r.segs * r.rows >= ny &&
               (long long)(r.segs - 1) * r.rows < ny,
           "segs %d x %d of %d rows", r.segs, r.rows, ny);
-    const int per = L.g.nchunks + 2;
+    const int per = L.g.nchunks + 2 * r.halo;
+    // a halo lane of the partial last chunk alone must hold a node per step
+    CHECK(r.halo == 2 || nx % V == 0 || nx % V >= kRowSteps, "halo %d nx %d", r.halo, nx);
     if ((long long)nx * ny > 20000) continue;
     std::vector<int> seen((size_t)r.segs * per, 0);
     for (int t = 0; t < r.tasks; ++t)
-      for (int lane = 1; lane <= 30; ++lane) {
-        const long long p = 30LL * t + lane;
+      for (int lane = r.halo; lane < 32 - r.halo; ++lane) {
+        const long long p = (32LL - 2 * r.halo) * t + lane;
         if (p < (long long)seen.size()) seen[(size_t)p]++;
       }
     for (size_t p = 0; p < seen.size(); ++p) {
-      const int c = (int)(p % per) - 1;
+      const int c = (int)(p % per) - r.halo;
       CHECK((c < 0 || c >= L.g.nchunks) ? seen[p] <= 1 : seen[p] == 1, "position %zu seen %d", p,
             seen[p]);
     }
   }
-  const RowsGeom r = plan_rows(L.g, sms * 12);
+  const RowsGeom r = plan_rows(L.g, V, sms * 12);
   CHECK(r.rows >= 1 && r.rows <= 48, "rows %d", r.rows);
   double us = 0;
   const TileGeom t = plan_tile(L.g, esize, sms, &us);
