@@ -647,23 +647,31 @@ static std::vector<size_t> packed_groups(const lbm_batch_ctx *b) {
 
 // Block records of the kRowSteps-per-launch grid of a batch's members of
 // storage type dt that are not resident; none where the grid does not take
-// some member or the members together are too small for it (the threshold
-// of a single lattice's plan).  Tasks of most rows first, so that the short
-// ones fill the tail of the launch.
+// some member or is not estimated to save at least 5% of the single-step
+// launches (plan.h; 16-bit batches of narrow or few lattices, whose
+// populations fit in L2, step as fast one by one).  Tasks of most rows
+// first, so that the short ones fill the tail of the launch.
 static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms) {
   std::vector<RowsRec> recs;
-  double nodes = 0, rows32 = 0;
+  constexpr int kChoices = sizeof(kRowChoices) / sizeof(kRowChoices[0]);
+  RowsWork work[kChoices];
+  const int esize = dt == LBM_F32DEV ? 4 : 2;
+  double nodes = 0;
   for (size_t mi = 0; mi < b->members.size(); ++mi) {
     const Lattice &L = b->members[mi]->L;
     if (L.dtype != dt || b->member_res[mi]) continue;
-    if (!rows_fit(L.g, L.V) || L.g.ny < kRowSteps) return recs;
+    if (!rows_fit(L.g, L.V)) return recs;
     nodes += (double)L.g.nx * L.g.ny;
-    rows32 += rows_geom(L.g, L.V, 32).tasks;
+    for (int k = 0; k < kChoices; ++k) work[k].add(rows_geom(L.g, L.V, kRowChoices[k]), L.V);
   }
-  if (nodes < rows_min_nodes(dt == LBM_F32DEV ? 4 : 2)) return recs;
-  // 32 rows per task, or 16 where that leaves fewer than six tasks per
-  // resident warp and the tail would weigh
-    const int rows = rows32 < 6.0 * sms * rows_warps(dt == LBM_F32DEV ? 4 : 2) ? 16 : 32;
+  double us = 0.95 * single_us(nodes, esize);
+  int rows = 0;
+  for (int k = 0; k < kChoices; ++k)
+    if (nodes > 0 && rows_us(work[k], esize, sms) < us) {
+      us = rows_us(work[k], esize, sms);
+      rows = kRowChoices[k];
+    }
+  if (rows == 0) return recs;
   for (size_t mi = 0; mi < b->members.size(); ++mi) {
     const Lattice &L = b->members[mi]->L;
     if (L.dtype != dt || b->member_res[mi]) continue;

@@ -28,13 +28,60 @@ inline bool rows_fit(const Geom &g, int V) {
   return (g.nx % V == 0 || g.nchunks >= 3) && (double)g.ny * (g.nchunks + 4) < 4e9;
 }
 
-// Rows per segment: 32 cost 2 (kRowSteps - 1) / 32 of redundant level-1 rows;
-// fewer where the tasks would not fill the resident warps (`slots`) a
-// quarter more than once (2048^2 FP32: 16 rows 23.2 us per step, 32 rows
-// 31.1, 8 rows 24.9).
-inline RowsGeom plan_rows(const Geom &g, int V, int slots) {
-  const double fit = (double)g.ny * (g.nchunks + 2) / 30.0 / (1.25 * slots);
-  return rows_geom(g, V, (int)std::max(8.0, std::min(32.0, fit)));
+// resident warps per SM of k_step_rows
+inline int rows_warps(int esize) { return esize == 4 ? 16 : 8; }
+
+// Work of k_step_rows over a lattice, or summed over a batch's: its tasks and
+// the nodes they compute per step (idle lanes, halo lanes and rows included).
+struct RowsWork {
+  double tasks = 0, nodes = 0;
+  void add(const RowsGeom &r, int V) {
+    tasks += r.tasks;
+    nodes += (double)r.tasks * 32 * V * (r.rows + kRowSteps - 1);
+  }
+};
+
+// Estimated us per step: 285 (FP32) or 300 (16 bits) such nodes per ns with
+// all warp slots busy, less where there are few tasks per slot.  Measured /
+// estimated: 8192^2 276 / 277 FP32 and 262 / 262 FP16, 1024^2 FP32 7.3 / 7.7,
+// 700^2 FP32 4.7 / 5.1, 4097 x 3071 FP16 59.6 / 59, 2500 x 2001 FP16 26 /
+// 24.6.
+inline double rows_us(const RowsWork &w, int esize, int sms) {
+  const double per_slot = w.tasks / ((double)sms * rows_warps(esize));
+  const double rate = (esize == 4 ? 285e3 : 300e3) * per_slot / (per_slot + 0.25);
+  return w.nodes / rate;
+}
+
+// Estimated us of one single-step launch over `nodes` nodes: its latency and
+// the L2's rate while both buffers fit there, HBM's beyond.  Measured: FP32
+// 1024^2 8.4, 1500 x 1111 16.4, 2048^2 45; 16 bits 1500 x 1111 9.4, 1732^2
+// 17.5, 2048^2 24.5 us.
+inline double single_us(double nodes, int esize) {
+  const double m = nodes * 1e-6;
+  return esize == 4 ? std::max(2.0 + 6.0 * m, 10.8 * m - 2.0) : std::max(2.7 + 3.9 * m, 5.7 * m);
+}
+
+// The segment heights tried: low ones cost redundant rows (2 (kRowSteps - 1)
+// per segment), high ones leave too few tasks.
+constexpr int kRowChoices[] = {8, 12, 16, 24, 32};
+
+// k_step_rows' best split of one lattice and its estimate (rows = 0: the
+// lattice does not fit it)
+inline RowsGeom plan_rows(const Geom &g, int V, int esize, int sms, double *us) {
+  RowsGeom best = {};
+  *us = 1e30;
+  if (!rows_fit(g, V)) return best;
+  for (int rows : kRowChoices) {
+    const RowsGeom r = rows_geom(g, V, rows);
+    RowsWork w;
+    w.add(r, V);
+    const double t = rows_us(w, esize, sms);
+    if (t < *us) {
+      *us = t;
+      best = r;
+    }
+  }
+  return best;
 }
 
 // k_step_tile: the split of least estimated time per step with all tiles
@@ -66,29 +113,24 @@ inline TileGeom plan_tile(const Geom &g, int esize, int sms, double *us_per_step
   return best;
 }
 
-// 32- and 16-bit deviation types: tiles where they fit and are estimated
-// faster than one launch per step (2.0 + 6.1 us per 2^20 FP32 nodes, 2.7 +
-// 4.1 us in 16 bits, measured from 512^2 to 1024^2); else rows for lattices
-// whose tasks keep the warps busy (rows_min_nodes: below, single steps
-// measured as fast); else, and for the FP64 types (bound by FP64 arithmetic, which
-// halos only add to), one step per launch.
-inline double rows_min_nodes(int esize) { return esize == 4 ? 1.25e6 : 3.0e6; }
-// resident warps per SM of k_step_rows
-inline int rows_warps(int esize) { return esize == 4 ? 12 : 8; }
-
+// The estimated fastest of tiles, rows and single steps for the 32- and
+// 16-bit deviation types (several steps per launch only where they save at
+// least 5%); one step per launch for the FP64 types, which FP64 arithmetic
+// bounds and halos would only add to.
 inline void plan_lattice(Lattice &L, int sms) {
   L.plan = PLAN_SINGLE;
   if (L.esize == 8) return;
-  const double nodes = (double)L.g.nx * L.g.ny;
-  double us = 0;
+  double best = 0.95 * single_us((double)L.g.nx * L.g.ny, L.esize), us = 0;
   const TileGeom t = plan_tile(L.g, L.esize, sms, &us);
-  const double single = L.esize == 4 ? 2.0 + 5.8e-6 * nodes : 2.7 + 3.9e-6 * nodes;
-  if (t.steps > 1 && us < single) {
+  if (t.steps > 1 && us < best) {
     L.plan = PLAN_TILE;
     L.tile = t;
-  } else if (nodes >= rows_min_nodes(L.esize) && rows_fit(L.g, L.V)) {
+    best = us;
+  }
+  const RowsGeom r = plan_rows(L.g, L.V, L.esize, sms, &us);
+  if (r.rows > 0 && us < best) {
     L.plan = PLAN_ROWS;
-    L.rows = plan_rows(L.g, L.V, sms * rows_warps(L.esize));
+    L.rows = r;
   }
 }
 

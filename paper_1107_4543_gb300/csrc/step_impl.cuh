@@ -14,6 +14,7 @@
 
 #include "bounds.cuh"
 #include "lbm_internal.h"
+#include "pdl.cuh"
 
 namespace lbm {
 
@@ -133,6 +134,7 @@ k_step_dev(const T *__restrict__ src, T *__restrict__ dst, Geom g,
   const int lane = threadIdx.x & 31;
   const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+  pdl_wait();
   for (long long task = warp0; task < ntasks; task += nwarps)
     step_task<T>(src, dst, g, P, task, lane);
 }
@@ -286,9 +288,9 @@ cudaError_t launch_step_dev_t(const Lattice &L, const void *src, void *dst, cuda
   if constexpr (std::is_same<T, double>::value) P = &L.dp64;
   else P = &L.dp;
   switch (variant) {
-    case 0: k_step_dev<T, 1><<<(unsigned)grid, block, 0, st>>>(s, d, L.g, *P, nt); break;
-    case 1: k_step_dev<T, 2><<<(unsigned)grid, block, 0, st>>>(s, d, L.g, *P, nt); break;
-    default: k_step_dev<T, 3><<<(unsigned)grid, block, 0, st>>>(s, d, L.g, *P, nt); break;
+    case 0: return launch_pdl(k_step_dev<T, 1>, (unsigned)grid, block, 0, st, s, d, L.g, *P, nt);
+    case 1: return launch_pdl(k_step_dev<T, 2>, (unsigned)grid, block, 0, st, s, d, L.g, *P, nt);
+    default: return launch_pdl(k_step_dev<T, 3>, (unsigned)grid, block, 0, st, s, d, L.g, *P, nt);
   }
   return cudaGetLastError();
 }

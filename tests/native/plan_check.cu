@@ -56,8 +56,9 @@ static void check(int nx, int ny, int dtype, int esize) {
             seen[p]);
     }
   }
-  const RowsGeom r = plan_rows(L.g, V, sms * 12);
-  CHECK(r.rows >= 1 && r.rows <= 48, "rows %d", r.rows);
+  double rus = 0;
+  const RowsGeom r = plan_rows(L.g, V, esize, sms, &rus);
+  CHECK(rows_fit(L.g, V) ? (r.rows >= 1 && r.rows <= 48 && rus > 0) : r.rows == 0, "rows %d", r.rows);
   double us = 0;
   const TileGeom t = plan_tile(L.g, esize, sms, &us);
   if (t.steps > 0) {
@@ -90,6 +91,21 @@ int main() {
                    4097, 8192, 20000})
       for (int ny : {2, 3, 5, 8, 16, 23, 101, 512, 777, 1111, 3071, 8192}) check(nx, ny, dtype, esize);
   }
+  // the lattices with which the GPU tests reach k_step_rows
+  auto rows_plan = [](int nx, int ny, int dtype) {
+    Lattice L;
+    L.dtype = dtype;
+    L.esize = dtype == LBM_F32DEV ? 4 : 2;
+    L.V = vec_nodes(dtype);
+    L.g = make_geom(nx, ny, L.V, L.esize);
+    plan_lattice(L, 152);
+    CHECK(L.plan == PLAN_ROWS, "plan of %d x %d: %d", nx, ny, (int)L.plan);
+  };
+  for (int k = 0; k < 4; ++k) rows_plan(1200 + k, 1101, LBM_F32DEV);
+  rows_plan(700001, 2, LBM_F32DEV);
+  rows_plan(420003, 3, LBM_F32DEV);
+  for (int k = 0; k < 8; ++k) rows_plan(2496 + k, 2101, LBM_F16DEV);
+  rows_plan(2501, 2101, LBM_BF16DEV);
   // the FP64 types step one by one
   for (int dtype : {LBM_F64, LBM_F64DEV}) {
     Lattice L;

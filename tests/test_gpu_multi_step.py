@@ -54,14 +54,11 @@ def test_tiles_equal_single_steps(L, nx, ny, dtype):
             L.lbm_slabs_destroy(s)
 
 
-# rows of the least lattices the rows kernel takes: shorter than a chunk, one
-# and two strips, a partial last chunk of every kind, two rows
-ROW_SIZES = [("f32", nx, ny) for nx, ny in [(2, 700001), (3, 420001), (5, 260001), (9, 150001), (10, 130001),
-                                            (11, 120001), (109, 12001), (119, 10601),
-                                            (121, 10501), (242, 5203), (1203, 1101), (700001, 2),
-                                            (420003, 3)]]
-ROW_SIZES += [(d, nx, ny) for d in ("f16", "bf16")
-              for nx, ny in [(17, 190001), (22, 140001), (219, 14001), (239, 12601), (241, 12501), (1500001, 2), (4097, 737)]]
+# lattices that take the rows kernel (tests/native/plan_check.cu checks that
+# they do): whole rows, a partial last chunk of every kind, few rows
+ROW_SIZES = [("f32", nx, ny) for nx, ny in [(1200, 1101), (1201, 1101), (1202, 1101), (1203, 1101),
+                                            (700001, 2), (420003, 3)]]
+ROW_SIZES += [("f16", 2496 + k, 2101) for k in range(8)] + [("bf16", 2501, 2101)]
 
 
 @pytest.mark.parametrize("dtype,nx,ny", ROW_SIZES)
@@ -135,11 +132,13 @@ def test_init_rounds_the_fp64_deviations_once(L, amp, u0):
         L.lbm_destroy(d)
 
 
-# members that together pass the size from which a batch's group takes three
-# steps per launch (FP32 and FP16; the BF16 pair stays below it)
-BATCH = [("f32", 700, 600), ("f32", 333, 1201), ("f32", 57, 9001), ("f32", 1000, 400),
-         ("f32", 20, 20), ("f16", 1201, 1000), ("f16", 801, 1500), ("f16", 330, 2500),
-         ("bf16", 130, 90), ("bf16", 61, 200)]
+# members whose groups take three steps per launch in FP32 and FP16 (one large
+# member each, and narrow ones around a chunk, three chunks and a warp); the
+# BF16 pair steps one by one, one member is resident
+BATCH = [("f32", 2000, 1001), ("f32", 9, 3001), ("f32", 10, 3001), ("f32", 11, 3001),
+         ("f32", 109, 901), ("f32", 119, 903), ("f32", 121, 905), ("f32", 333, 1201),
+         ("f32", 20, 20), ("f16", 2600, 2103), ("f16", 17, 4001), ("f16", 22, 3001),
+         ("f16", 239, 501), ("f16", 241, 503), ("bf16", 130, 90), ("bf16", 61, 200)]
 
 
 def alone(L, dtype, nx, ny, f, steps):
@@ -182,7 +181,7 @@ def test_served_generations_of_rows_equal_alone(L):
     remainder, some inside a generation's last three-step launch."""
     import time
 
-    steps = [5, 22, 23, 24, 9, 11, 31, 3, 1, 12]
+    steps = [5, 22, 23, 24, 9, 11, 31, 3, 1, 12, 10, 2, 33, 32, 7, 4]
     fields = [inp.gaussian_pulse(nx, ny, 1e-3, 5.0, xc=2.0, yc=1.0) for _, nx, ny in BATCH]
     s = L.lbm_server_create(2 ** 33, 11)
     try:
