@@ -68,13 +68,11 @@ struct lbm_batch_ctx {
     RowsRec *rows = nullptr;
     long long nrows = 0;
     // entries held in shared memory for all the steps of a launch (small
-    // lattices; k_batch_resident), which the block records leave out; in
-    // three classes by size (up to a third, a half, all of a block's shared
-    // memory), one launch each, so that small ones share an SM
+    // lattices; k_batch_resident), which the block records leave out, largest
+    // first, and the bytes of the largest one's planes
     int nres = 0;
     int *res = nullptr;
-    int res_count[3] = {0, 0, 0};
-    size_t res_smem[3] = {0, 0, 0};  // shared memory of a block of the class
+    size_t res_planes = 0;
     // the group's slots in its type's constant table (-1: none) and the
     // device staging of their refresh (n x const_slot_bytes(dtype))
     int pbase = -1;
@@ -205,11 +203,9 @@ static int resident_fork(lbm_batch_ctx *b, int parity, long steps, bool ragged) 
   CK(cudaEventRecord(b->res_fork, b->stream));
   CK(cudaStreamWaitEvent(b->res_stream, b->res_fork, 0));
   for (auto &gr : b->groups)
-    for (int c = 0, off = 0; c < 3; off += gr.res_count[c++])
-      if (gr.res_count[c] > 0)
-        CK(launch_batch_resident(gr.dtype, gr.ents, gr.res + off, gr.res_count[c], gr.n,
-                                 gr.res_smem[c], parity, steps, ragged ? gr.limits : nullptr,
-                                 b->res_stream));
+    if (gr.nres > 0)
+      CK(launch_batch_resident(gr.dtype, gr.ents, gr.res, gr.nres, gr.n, gr.res_planes, parity,
+                               steps, ragged ? gr.limits : nullptr, b->res_stream));
   CK(cudaEventRecord(b->res_join, b->res_stream));
   return LBM_OK;
 }
@@ -742,8 +738,7 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
   for (int dt : {LBM_F32DEV, LBM_F16DEV, LBM_BF16DEV}) {
     std::vector<BatchEntry> ents;
     std::vector<BlockRec> bl;  // the plain grid's blocks
-    std::vector<int> res_cls[3];  // resident entries by size class
-    size_t res_smem[3] = {0, 0, 0};
+    std::vector<int> res;  // resident entries
     long long t0 = 0;
     {
       size_t nb = 0;  // an upper bound of the records (a server builds ~10^5 per generation)
@@ -765,9 +760,7 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
       const size_t rb = resident_bytes(m->L.g.nx, m->L.g.ny, m->L.esize);
       if (rb <= res_max) {
         b->member_res[mi] = 1;
-        const int c = rb <= res_max / 3 ? 0 : (rb <= res_max / 2 ? 1 : 2);
-        res_cls[c].push_back((int)ents.size());
-        res_smem[c] = std::max(res_smem[c], rb);
+        res.push_back((int)ents.size());
         ents.push_back(e);
         continue;
       }
@@ -796,12 +789,11 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
     gr.limits = (int *)dev_alloc(sizeof(int) * ents.size());
     gr.nrows = (long long)rl.size();
     if (gr.nrows > 0) gr.rows = (RowsRec *)dev_alloc(sizeof(RowsRec) * rl.size());
-    std::vector<int> res;
-    for (int c = 0; c < 3; ++c) {
-      res.insert(res.end(), res_cls[c].begin(), res_cls[c].end());
-      gr.res_count[c] = (int)res_cls[c].size();
-      gr.res_smem[c] = res_smem[c];
-    }
+    auto nodes_of = [&](int k) { return (long long)ents[k].g.nx * ents[k].g.ny; };
+    std::stable_sort(res.begin(), res.end(),
+                     [&](int p, int q) { return nodes_of(p) > nodes_of(q); });
+    if (!res.empty())
+      gr.res_planes = (size_t)9 * nodes_of(res[0]) * (dt == LBM_F32DEV ? 4 : 2);
     gr.nres = (int)res.size();
     if (gr.nres > 0) {
       gr.res = (int *)dev_alloc(sizeof(int) * res.size());

@@ -367,8 +367,9 @@ __device__ __forceinline__ F2 mul_hl2(F2 a, const F2x2 &k) { return fma2(a, k.a,
 // form's bit for bit (its one product that the compiler contracts, the
 // -3 dJ of n3, is an explicit multiply-add here; products by powers of two
 // are exact either way).
+template <typename K>
 __device__ __forceinline__ void collide_pair_hl(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2 &f4, F2 &f5,
-                                                F2 &f6, F2 &f7, F2 &f8, const HlPairs &P) {
+                                                F2 &f6, F2 &f7, F2 &f8, const K &P) {
   const F2 s13 = f1 + f3, s24 = f2_ + f4;
   const F2 d13 = f1 - f3, d24 = f2_ - f4;
   const F2 s57 = f5 + f7, s68 = f6 + f8;

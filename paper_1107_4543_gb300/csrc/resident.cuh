@@ -1,59 +1,50 @@
 // Batched step for small lattices held in shared memory for all the time
 // steps of one launch (section 2.1, Eq. blbs, as the per-step kernels): one
 // thread block per member loads the member's nine planes into shared memory,
-// runs its n steps there (pull with periodic wrap, collide, store into the
-// other buffer, block barrier, swap) and writes the result back once: its
-// 9 x nx ny elements cross HBM once in and once out for the whole launch
-// instead of in and out at every step.
+// runs its n steps there and writes the result back once: its 9 x nx ny
+// elements cross HBM once in and once out for the whole launch instead of in
+// and out at every step.
 //
-// The arithmetic is the per-step kernels' own (collide_dev for FP32,
-// collide_pair for the 16-bit types, the same storage rounding), node by
-// node, so a member's result is bit-identical to the per-step path's.
+// The steps work in place (the "AA" access pattern of Bailey, Myre, Walsh,
+// Lilja and Saar, ICPP 2009): even steps pull population i of node x from
+// slot (i, x - c_i) and put the post-collision population of the opposite
+// direction there, so that odd steps find what streams to node x in its own
+// slots, each in the slot of the opposite direction, and leave the
+// post-collision populations in their own.  Every slot is read and written
+// by one node per step, so one set of planes is enough where a second buffer
+// had left most members alone on their SM: two members per SM now hide each
+// other's latency and barriers.
+//
+// The arithmetic is the per-step kernels' own (collide_pair_hl, the packed
+// form of collide_dev, for FP32, collide_pair for the 16-bit types, the same
+// storage rounding), node by node, so a member's result is bit-identical to
+// the per-step path's.
 #pragma once
 #include <type_traits>
 
 #include "bounds.cuh"
 #include "lbm_internal.h"
+#include "step_multi.cuh"
 
 namespace lbm {
 
-// 512 threads (16 warps) per member; two blocks per SM at the 64-register
-// cap (256 threads: 135 against 152 GLUPS on 4,096 lattices of 32^2 - 56^2)
-constexpr int kResidentThreads = 512;
+// 384 threads (12 warps) per member, two blocks per SM at the 80-register
+// cap, no FP32 spills: 1,024 lattices of 32^2 - 56^2 take 4.9 ms for 500 steps
+// (512 threads at 64 registers, 100 bytes of spills: 6.5; 320: 5.2; two step
+// buffers, one node per thread, 512 threads: 7.65)
+constexpr int kResidentThreads = 384;
 
 template <typename T>
 __device__ __forceinline__ uint32_t bits16(const T *p) {
   return (uint32_t) * reinterpret_cast<const unsigned short *>(p);
 }
 
-// Node r = y nx + x of the plane arrays A (9 planes of N compact elements):
-// the element plane i pulls into (x, y), i.e. the one at (x - c_ix, y - c_iy)
-// with periodic wrap.
-struct Nbr {
-  int r0;          // y * nx
-  int xm, x, xp;   // x - 1, x, x + 1 (wrapped)
-  int ym, yp;      // (y - 1) nx, (y + 1) nx (wrapped)
-  __device__ __forceinline__ int at(int i) const {
-    const int cx = CXd(i), cy = CYd(i);
-    const int row = cy == 1 ? ym : (cy == -1 ? yp : r0);
-    const int col = cx == 1 ? xm : (cx == -1 ? xp : x);
-    return row + col;
-  }
-};
-
-__device__ __forceinline__ Nbr nbr(int x, int y, int nx, int ny) {
-  Nbr n;
-  n.x = x;
-  n.r0 = y * nx;
-  n.xm = x == 0 ? nx - 1 : x - 1;
-  n.xp = x == nx - 1 ? 0 : x + 1;
-  n.ym = (y == 0 ? ny - 1 : y - 1) * nx;
-  n.yp = (y == ny - 1 ? 0 : y + 1) * nx;
-  return n;
+__device__ constexpr int opposite(int i) {
+  return i == 0 ? 0 : (i <= 2 ? i + 2 : (i <= 4 ? i - 2 : (i <= 6 ? i + 2 : i - 2)));
 }
 
-// (x, y) of node r, advanced by a fixed stride of (dx, dy) = (stride mod nx,
-// stride / nx) nodes without a division per node
+// (x, y) of item r, advanced by a fixed stride of (dx, dy) = (stride mod nx,
+// stride / nx) without a division per item
 struct Walk {
   int x, y, dx, dy, nx;
   __device__ __forceinline__ Walk(int r, int stride, int nx_) : nx(nx_) {
@@ -72,13 +63,85 @@ struct Walk {
   }
 };
 
+// Node (x, y) and the slots that the directions pull from, periodic
+struct Nbr {
+  int r0;          // y nx
+  int xm, x, xp;   // x - 1, x, x + 1 (wrapped)
+  int ym, yp;      // (y - 1) nx, (y + 1) nx (wrapped)
+  __device__ __forceinline__ int at(int i) const {
+    const int cx = CXd(i), cy = CYd(i);
+    return (cy == 1 ? ym : (cy == -1 ? yp : r0)) + (cx == 1 ? xm : (cx == -1 ? xp : x));
+  }
+};
+__device__ __forceinline__ Nbr nbr(int x, int y, int nx, int ny) {
+  Nbr n;
+  n.x = x;
+  n.r0 = y * nx;
+  n.xm = x == 0 ? nx - 1 : x - 1;
+  n.xp = x == nx - 1 ? 0 : x + 1;
+  n.ym = (y == 0 ? ny - 1 : y - 1) * nx;
+  n.yp = (y == ny - 1 ? 0 : y + 1) * nx;
+  return n;
+}
+
+// the collision constants, behind the planes
+template <typename T> struct ResidentConst;
+template <> struct ResidentConst<float> {
+  using Table = HlPairs;
+  static constexpr int COUNT = HL_COUNT;
+  static __device__ __forceinline__ float value(const DevParams &P, int k) { return hl_const(P, k); }
+  static __device__ __forceinline__ const HlPairs &of(const Table &t) { return t; }
+};
+template <typename T> struct ResidentConst {
+  struct alignas(16) Table {
+    float2 c[PC_COUNT];
+  };
+  static constexpr int COUNT = PC_COUNT;
+  static __device__ __forceinline__ float value(const DevParams &P, int k) {
+    return pair_const(P, k);
+  }
+  static __device__ __forceinline__ SharedPairs of(const Table &t) { return SharedPairs{t.c}; }
+};
+
+// Slots (ia, ib) of the planes as the two nodes of a pair
+template <typename T>
+__device__ __forceinline__ F2 slot_load(const T *A, int ia, int ib) {
+  if constexpr (sizeof(T) == 4) {
+    return f2(A[ia], A[ib]);
+  } else {
+    float u[2];
+    Elem<T>::unpack2(bits16(A + ia) | bits16(A + ib) << 16, u);
+    return f2(u[0], u[1]);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void slot_store(T *A, int ia, int ib, bool two, F2 f) {
+  float u, v;
+  f2split(f, u, v);
+  if constexpr (sizeof(T) == 4) {
+    A[ia] = u;
+    if (two) A[ib] = v;
+  } else {
+    const uint32_t w = Elem<T>::pack2(u, v);
+    reinterpret_cast<unsigned short *>(A)[ia] = (unsigned short)(w & 0xffffu);
+    if (two) reinterpret_cast<unsigned short *>(A)[ib] = (unsigned short)(w >> 16);
+  }
+}
+
 // idx[b]: the entry block b steps.  Each member takes min(steps, limits[e])
 // steps (limits may be null) from buffer parity ^ off and leaves its state
 // in the buffer that parity of steps selects, as the per-step launches do.
+//
+// A thread takes two nodes at a time for the packed collisions: node p and
+// node p + ceil(N / 2) of the row-major order, so that a warp's accesses to
+// either are consecutive words whatever the row length (adjacent nodes would
+// hit every bank twice, half rows apart a warp spans rows and does so too:
+// 37% of the shared-memory wavefronts, which bound the kernel, were
+// conflicts).
 template <typename T>
 __global__ void __launch_bounds__(kResidentThreads, 2)
 k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ idx, int nents,
-                 int parity, int steps, const int *__restrict__ limits) {
+                 int parity, int steps, const int *__restrict__ limits, int consts_at) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int e = idx[blockIdx.x];
   if (!bounds::ok(e >= 0 && e < nents, bounds::BATCH_REC)) return;  // block-uniform
@@ -91,80 +154,77 @@ k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ id
   const T *src = static_cast<const T *>(E.buf[from]);
   T *dst = static_cast<T *>(E.buf[from ^ (n & 1)]);
   T *A = reinterpret_cast<T *>(smem_raw);
-  T *B = A + 9 * N;
+  using RC = ResidentConst<T>;
+  typename RC::Table &table = *reinterpret_cast<typename RC::Table *>(smem_raw + consts_at);
+  if (threadIdx.x < RC::COUNT) {
+    const float v = RC::value(E.dp, threadIdx.x);
+    table.c[threadIdx.x] = make_float2(v, v);
+  }
   for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
     const int i = q / N, r = q - i * N, y = r / nx;
     A[q] = src[(long long)i * E.g.plane + (long long)y * E.g.rstride + (r - y * nx)];
   }
   __syncthreads();
-  const DevParams &P = E.dp;
+  const int half = (N + 1) >> 1;
   for (int t = 0; t < n; ++t) {
-    if constexpr (sizeof(T) == 4) {
-      Walk wk(threadIdx.x, blockDim.x, nx);
-      for (int r = threadIdx.x; r < N; r += blockDim.x, wk.next()) {
-        const Nbr nb = nbr(wk.x, wk.y, nx, ny);
-        float f[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = A[i * N + nb.at(i)];
-        collide_dev<true, false>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7], f[8], P);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) B[i * N + r] = f[i];
-      }
-    } else {
-      // two nodes per thread, one per lane of the packed pair collision
-      constexpr bool SCALED = std::is_same<T, __half>::value;
-      Walk wk(2 * threadIdx.x, 2 * blockDim.x, nx);
-      for (int r0 = 2 * threadIdx.x; r0 < N; r0 += 2 * blockDim.x, wk.next()) {
-        const int r1 = r0 + 1 < N ? r0 + 1 : r0;
-        // node r0 + 1 is (x + 1, y), or the start of the next row
-        const int x1 = wk.x + 1 < nx ? wk.x + 1 : 0;
-        const int y1 = wk.x + 1 < nx ? wk.y : wk.y + 1;
-        const Nbr n0 = nbr(wk.x, wk.y, nx, ny);
-        const Nbr n1 = r1 != r0 ? nbr(x1, y1, nx, ny) : n0;
+    if (!(t & 1)) {
+      Walk wa(threadIdx.x, blockDim.x, nx), wb(threadIdx.x + half, blockDim.x, nx);
+      for (int p = threadIdx.x; p < half; p += blockDim.x, wa.next(), wb.next()) {
+        // an odd lattice's last pair is one node (taken twice, stored once)
+        const bool two = p + half < N;
+        const Nbr a = nbr(wa.x, wa.y, nx, ny);
+        const Nbr b = two ? nbr(wb.x, wb.y, nx, ny) : a;
         F2 f[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-          float u[2];
-          Elem<T>::unpack2(bits16(&A[i * N + n0.at(i)]) | bits16(&A[i * N + n1.at(i)]) << 16, u);
-          f[i] = f2(u[0], u[1]);
-        }
-        collide_pair<SCALED>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7], f[8],
-                             ParamPairs{P});
+        for (int i = 0; i < 9; ++i) f[i] = slot_load(A, i * N + a.at(i), i * N + b.at(i));
+        collide_two<T>(f, RC::of(table));
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-          float u[2];
-          f2split(f[i], u[0], u[1]);
-          const uint32_t w = Elem<T>::pack2(u[0], u[1]);
-          reinterpret_cast<unsigned short *>(B)[i * N + r0] = (unsigned short)(w & 0xffffu);
-          if (r1 != r0) reinterpret_cast<unsigned short *>(B)[i * N + r1] = (unsigned short)(w >> 16);
-        }
+        for (int i = 0; i < 9; ++i)
+          slot_store(A, i * N + a.at(i), i * N + b.at(i), two, f[opposite(i)]);
+      }
+    } else {
+      for (int p = threadIdx.x; p < half; p += blockDim.x) {
+        const bool two = p + half < N;
+        const int q = two ? p + half : p;
+        F2 f[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[opposite(i)] = slot_load(A, i * N + p, i * N + q);
+        collide_two<T>(f, RC::of(table));
+#pragma unroll
+        for (int i = 0; i < 9; ++i) slot_store(A, i * N + p, i * N + q, two, f[i]);
       }
     }
     __syncthreads();
-    T *tmp = A;
-    A = B;
-    B = tmp;
   }
   for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
-    const int i = q / N, r = q - i * N, y = r / nx;
-    dst[(long long)i * E.g.plane + (long long)y * E.g.rstride + (r - y * nx)] = A[q];
+    const int i = q / N, r = q - i * N, y = r / nx, x = r - y * nx;
+    int at = q;
+    if (n & 1) {  // post-collision population i of x is in slot (opposite i, x + c_i)
+      const int xs = x + CXd(i), ys = y + CYd(i);
+      at = opposite(i) * N + (ys < 0 ? ny - 1 : (ys == ny ? 0 : ys)) * nx +
+           (xs < 0 ? nx - 1 : (xs == nx ? 0 : xs));
+    }
+    dst[(long long)i * E.g.plane + (long long)y * E.g.rstride + x] = A[at];
   }
 }
 
+// planes: bytes of the largest member's nine planes
 template <typename T>
 cudaError_t launch_resident_t(const BatchEntry *ents, const int *idx, int nres, int nents,
-                              size_t smem, int parity, long steps, const int *limits,
+                              size_t planes, int parity, long steps, const int *limits,
                               cudaStream_t st) {
   if (nres < 1 || steps < 1) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_batch_resident<T>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t at = (planes + 15) / 16 * 16;
+  const size_t smem = at + sizeof(typename ResidentConst<T>::Table);
+  cudaError_t e = cudaFuncSetAttribute(
+      k_batch_resident<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;
   // launches of at most 2^30 steps (the step count is an int on the device)
   const long chunk = 1L << 30;
   for (long done = 0; done < steps; done += chunk) {
     const long k = steps - done < chunk ? steps - done : chunk;
     k_batch_resident<T><<<(unsigned)nres, kResidentThreads, smem, st>>>(
-        ents, idx, nents, parity ^ (int)(done & 1), (int)k, limits);
+        ents, idx, nents, parity ^ (int)(done & 1), (int)k, limits, (int)at);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
