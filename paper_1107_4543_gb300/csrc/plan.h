@@ -98,16 +98,16 @@ inline TileGeom plan_tile(const Geom &g, int esize, int sms, double *us_per_step
     const int bx = ((g.nx + ntx - 1) / ntx + 1) & ~1;
     ntx = (g.nx + bx - 1) / bx;
     if (ntx > sms) continue;
-    for (int nty = 1; nty <= std::min(g.ny, sms / ntx); ++nty) {
-      const int by = (g.ny + nty - 1) / nty;
-      if (nty > 1 && by == (g.ny + nty - 2) / (nty - 1)) continue;  // same split
-      if (tile_bytes(by, T, esize) > (size_t)kMaxSmem) continue;
-      double us = 1.2 + 0.05 * (by + 2 * T);
-      for (int s = 1; s <= T; ++s) us += 0.33 + 0.04 * (by + 2 * (T - s));
-      if (us / T < *us_per_step) {
-        *us_per_step = us / T;
-        best = {bx, by, ntx, (g.ny + by - 1) / by, T};
-      }
+    // both the estimate and the tile's size grow with its height: the lowest
+    // tiles that are resident at once
+    const int nty = std::min(g.ny, sms / ntx);
+    const int by = (g.ny + nty - 1) / nty;
+    if (tile_bytes(by, T, esize) > (size_t)kMaxSmem) continue;
+    double us = 1.2 + 0.05 * (by + 2 * T);
+    for (int s = 1; s <= T; ++s) us += 0.33 + 0.04 * (by + 2 * (T - s));
+    if (us / T < *us_per_step) {
+      *us_per_step = us / T;
+      best = {bx, by, ntx, (g.ny + by - 1) / by, T};
     }
   }
   return best;
