@@ -668,16 +668,18 @@ int create_lattice(int nx, int ny, const double S[9], double rho0, const double 
     q.rho0 = h->rho0;
     q.jx0 = h->j0[0];
     q.jy0 = h->j0[1];
+    q.jx2 = 2.0 * q.jx0;
+    q.jy2 = 2.0 * q.jy0;
     q.k3 = h->S_paper[3] / 36.0;
-    q.k4 = h->S_paper[4] / 36.0;
+    q.k4 = h->S_paper[4] / 12.0;
     q.k5 = h->S_paper[5] / 12.0;
     q.k6 = h->S_paper[6] / 12.0;
     q.k7 = h->S_paper[7] / 4.0;
     q.k8 = h->S_paper[8] / 4.0;
-    q.q0 = q.jx0 * q.jx0 + q.jy0 * q.jy0;
-    q.d0 = q.jx0 * q.jx0 - q.jy0 * q.jy0;
-    q.x0 = q.jx0 * q.jy0;
-    q.i2 = 1.0 / (q.rho0 * q.rho0);
+    q.k6x2 = 2.0 * q.k6;
+    q.q0 = -(q.jx0 * q.jx0 + q.jy0 * q.jy0) / q.rho0;
+    q.d0 = -(q.jx0 * q.jx0 - q.jy0 * q.jy0) / q.rho0;
+    q.x0 = -q.jx0 * q.jy0 / q.rho0;
   }
   F64Params &fp = h->L.fp;
   fp.s3 = h->S_paper[3];
