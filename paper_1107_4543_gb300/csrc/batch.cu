@@ -656,9 +656,9 @@ static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms
   for (size_t mi = 0; mi < b->members.size(); ++mi) {
     const Lattice &L = b->members[mi]->L;
     if (L.dtype != dt || b->member_res[mi]) continue;
-    if (!rows_fit(L.g, L.V)) return recs;
+    if (!rows_fit(L.g)) return recs;
     nodes += (double)L.g.nx * L.g.ny;
-    for (int k = 0; k < kChoices; ++k) work[k].add(rows_geom(L.g, L.V, kRowChoices[k]), L.V);
+    for (int k = 0; k < kChoices; ++k) work[k].add(rows_geom(L.g, kRowChoices[k]));
   }
   double us = 0.95 * single_us(nodes, esize);
   int rows = 0;
@@ -673,7 +673,7 @@ static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms
     if (L.dtype != dt || b->member_res[mi]) continue;
     RowsRec r;
     r.g = L.g;
-    r.rg = rows_geom(L.g, L.V, rows);
+    r.rg = rows_geom(L.g, rows);
     r.buf[0] = L.buf[0];
     r.buf[1] = L.buf[1];
     r.lat = b->member_local[mi];

@@ -49,6 +49,10 @@ struct TileGeom {
   int bx, by, ntx, nty, steps;
 };
 constexpr int kRowSteps = 3;       // steps per k_step_rows launch (2 for a remainder)
+// k_step_rows: nodes per lane and plane (a chunk of its own, half the vector of
+// the single-step kernels for the 16-bit types)
+constexpr int kRowsV = 4;
+__host__ __device__ inline int rows_chunks(const Geom &g) { return (g.nx + kRowsV - 1) / kRowsV; }
 constexpr int kTileCols = 64;      // columns of a tile with its halo: 32 lanes of 2 nodes
 constexpr int kTileThreads = 512;
 constexpr int kMaxTileSteps = 8;

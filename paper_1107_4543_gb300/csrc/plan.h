@@ -10,22 +10,23 @@ namespace lbm {
 // k_step_rows: segments of about `rows` rows, as even as they go, each a
 // sequence of nchunks + 2 halo lane positions, 32 - 2 halo of them to a task
 // (the first ones, halo, are no task's own).
-inline RowsGeom rows_geom(const Geom &g, int V, int rows) {
+inline RowsGeom rows_geom(const Geom &g, int rows) {
+  constexpr int V = kRowsV;
   RowsGeom r;
   r.segs = std::max(1, (g.ny + rows / 2) / rows);
   r.rows = (g.ny + r.segs - 1) / r.segs;
   r.segs = (g.ny + r.rows - 1) / r.rows;
   r.halo = g.nx % V != 0 && g.nx % V < kRowSteps ? 2 : 1;
   const int own = 32 - 2 * r.halo;
-  const long long pos = (long long)r.segs * (g.nchunks + 2 * r.halo);
+  const long long pos = (long long)r.segs * (rows_chunks(g) + 2 * r.halo);
   r.tasks = (int)std::min<long long>((pos - 2 * r.halo + own - 1) / own, 1 << 30);
   return r;
 }
 
 // whether k_step_rows takes the lattice: its halo chunks are chunks of their
 // own, and its positions are 32-bit
-inline bool rows_fit(const Geom &g, int V) {
-  return (g.nx % V == 0 || g.nchunks >= 3) && (double)g.ny * (g.nchunks + 4) < 4e9;
+inline bool rows_fit(const Geom &g) {
+  return (g.nx % kRowsV == 0 || rows_chunks(g) >= 3) && (double)g.ny * (rows_chunks(g) + 4) < 4e9;
 }
 
 // resident warps per SM of k_step_rows
@@ -35,9 +36,9 @@ inline int rows_warps(int esize) { return esize == 4 ? 16 : 8; }
 // the nodes they compute per step (idle lanes, halo lanes and rows included).
 struct RowsWork {
   double tasks = 0, nodes = 0;
-  void add(const RowsGeom &r, int V) {
+  void add(const RowsGeom &r) {
     tasks += r.tasks;
-    nodes += (double)r.tasks * 32 * V * (r.rows + kRowSteps - 1);
+    nodes += (double)r.tasks * 32 * kRowsV * (r.rows + kRowSteps - 1);
   }
 };
 
@@ -67,14 +68,14 @@ constexpr int kRowChoices[] = {8, 12, 16, 24, 32};
 
 // k_step_rows' best split of one lattice and its estimate (rows = 0: the
 // lattice does not fit it)
-inline RowsGeom plan_rows(const Geom &g, int V, int esize, int sms, double *us) {
+inline RowsGeom plan_rows(const Geom &g, int esize, int sms, double *us) {
   RowsGeom best = {};
   *us = 1e30;
-  if (!rows_fit(g, V)) return best;
+  if (!rows_fit(g)) return best;
   for (int rows : kRowChoices) {
-    const RowsGeom r = rows_geom(g, V, rows);
+    const RowsGeom r = rows_geom(g, rows);
     RowsWork w;
-    w.add(r, V);
+    w.add(r);
     const double t = rows_us(w, esize, sms);
     if (t < *us) {
       *us = t;
@@ -127,7 +128,7 @@ inline void plan_lattice(Lattice &L, int sms) {
     L.tile = t;
     best = us;
   }
-  const RowsGeom r = plan_rows(L.g, L.V, L.esize, sms, &us);
+  const RowsGeom r = plan_rows(L.g, L.esize, sms, &us);
   if (r.rows > 0 && us < best) {
     L.plan = PLAN_ROWS;
     L.rows = r;

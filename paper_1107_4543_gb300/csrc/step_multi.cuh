@@ -60,50 +60,45 @@ __device__ __forceinline__ void collide_two(F2 (&f)[9], const K &P) {
 // last real node, element el, to the next lane (chunk 0) and takes that
 // lane's node 0 after it.  `warp`: some lane of the warp holds such a chunk
 // (warp-uniform, so the other warps skip the selects).
+template <int W>
 struct Seam {
   bool warp, last;
   int el;
   // all ones for this lane's word that holds element el (a comparison per
   // word instead is turned into an indexed array in local memory, at half
   // the speed), and the shift that brings a 16-bit el to the word's high half
-  uint32_t word[4];
+  uint32_t word[W];
   int up;
 };
 
-// One lane's chunk of a plane (V nodes as four words) shifted by the x
+// One lane's chunk of a plane (kRowsV nodes in W words) shifted by the x
 // component of the plane's velocity: the missing element comes from the
 // neighbouring lane, whose chunk is the neighbouring one.
-template <typename T>
-__device__ __forceinline__ void shift_chunk(uint32_t (&w)[4], int cx, const Seam &S) {
+template <typename T, int W>
+__device__ __forceinline__ void shift_chunk(uint32_t (&w)[W], int cx, const Seam<W> &S) {
   if (cx == 1) {
-    uint32_t tail = w[3];
+    uint32_t tail = w[W - 1];
     if (S.warp) {
       uint32_t own = 0, any = 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < W; ++q) {
         own |= w[q] & S.word[q];
         any |= S.word[q];
       }
       tail = ((tail & ~any) | own) << S.up;
     }
     const uint32_t prev = __shfl_up_sync(0xffffffffu, tail, 1);
-    if constexpr (sizeof(T) == 4) {
-      w[3] = w[2]; w[2] = w[1]; w[1] = w[0]; w[0] = prev;
-    } else {
-      w[3] = __byte_perm(w[2], w[3], 0x5432);
-      w[2] = __byte_perm(w[1], w[2], 0x5432);
-      w[1] = __byte_perm(w[0], w[1], 0x5432);
-      w[0] = __byte_perm(prev, w[0], 0x5432);
+#pragma unroll
+    for (int q = W - 1; q >= 0; --q) {
+      const uint32_t before = q > 0 ? w[q > 0 ? q - 1 : 0] : prev;
+      w[q] = sizeof(T) == 4 ? before : __byte_perm(before, w[q], 0x5432);
     }
   } else if (cx == -1) {
     const uint32_t next = __shfl_down_sync(0xffffffffu, w[0], 1);
-    if constexpr (sizeof(T) == 4) {
-      w[0] = w[1]; w[1] = w[2]; w[2] = w[3]; w[3] = next;
-    } else {
-      w[0] = __byte_perm(w[0], w[1], 0x5432);
-      w[1] = __byte_perm(w[1], w[2], 0x5432);
-      w[2] = __byte_perm(w[2], w[3], 0x5432);
-      w[3] = __byte_perm(w[3], next, 0x5432);
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+      const uint32_t after = q < W - 1 ? w[q < W - 1 ? q + 1 : 0] : next;
+      w[q] = sizeof(T) == 4 ? after : __byte_perm(w[q], after, 0x5432);
     }
     if (S.warp) {
       // node 0 takes the element after the last one
@@ -113,7 +108,7 @@ __device__ __forceinline__ void shift_chunk(uint32_t (&w)[4], int cx, const Seam
         put = (S.el & 1) ? next << 16 : next & 0xffffu;
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < W; ++q) {
         const uint32_t m = S.word[q] & ~keep;
         w[q] = (w[q] & ~m) | (put & m);
       }
@@ -122,11 +117,10 @@ __device__ __forceinline__ void shift_chunk(uint32_t (&w)[4], int cx, const Seam
 }
 
 // all nodes of a lane's chunk, two at a time
-template <typename T, typename K>
-__device__ __forceinline__ void collide_chunk(uint32_t (&w)[9][4], const K &P) {
-  constexpr int PAIRS = sizeof(T) == 4 ? 2 : 4;
+template <typename T, int W, typename K>
+__device__ __forceinline__ void collide_chunk(uint32_t (&w)[9][W], const K &P) {
 #pragma unroll
-  for (int k = 0; k < PAIRS; ++k) {
+  for (int k = 0; k < kRowsV / 2; ++k) {
     F2 f[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -153,21 +147,31 @@ __device__ __forceinline__ void collide_chunk(uint32_t (&w)[9][4], const K &P) {
   }
 }
 
-__device__ __forceinline__ void set4(uint32_t (&w)[4], const uint4 &v) {
+// a lane's chunk in memory
+template <typename T> struct RowsVec { using type = uint2; };
+template <> struct RowsVec<float> { using type = uint4; };
+__device__ __forceinline__ void set_words(uint32_t (&w)[4], const uint4 &v) {
   w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
 }
-__device__ __forceinline__ uint4 get4(const uint32_t (&w)[4]) {
+__device__ __forceinline__ void set_words(uint32_t (&w)[2], const uint2 &v) {
+  w[0] = v.x; w[1] = v.y;
+}
+__device__ __forceinline__ uint4 get_words(const uint32_t (&w)[4]) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
+__device__ __forceinline__ uint2 get_words(const uint32_t (&w)[2]) { return make_uint2(w[0], w[1]); }
 
-__device__ __forceinline__ void cp_async16(uint4 *smem, const void *g) {
+__device__ __forceinline__ void cp_async(uint4 *smem, const void *g) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(g) : "memory");
 }
-// shared memory of one warp of k_step_rows, in 16-byte words: 9 incoming
-// vectors and, per level boundary, 3 delayed by one row and 3 by two rows,
-// for 32 lanes
-constexpr int rows_smem_words(int steps) { return (9 + 9 * (steps - 1)) * 32; }
+__device__ __forceinline__ void cp_async(uint2 *smem, const void *g) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(a), "l"(g) : "memory");
+}
+// shared memory of one warp of k_step_rows, in chunks: 9 incoming ones and,
+// per level boundary, 3 delayed by one row and 3 by two rows, for 32 lanes
+constexpr int rows_smem_chunks(int steps) { return (9 + 9 * (steps - 1)) * 32; }
 
 // The lattice's rows are cut into segments of rg.rows; a segment is a
 // sequence of halo + nchunks + halo lane positions (the chunks before chunk
@@ -198,26 +202,27 @@ constexpr int rows_smem_words(int steps) { return (9 + 9 * (steps - 1)) * 32; }
 template <typename T, int STEPS, typename K>
 __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restrict__ dst,
                                           const Geom &g, const RowsGeom &rg, const K &par,
-                                          unsigned task, int lane, uint4 *sm) {
-  constexpr int V = Elem<T>::V;
+                                          unsigned task, int lane, typename RowsVec<T>::type *sm) {
+  constexpr int V = kRowsV, W = V * (int)sizeof(T) / 4;
+  using Vec = typename RowsVec<T>::type;
   static_assert(STEPS >= 2 && STEPS <= V, "the halo chunk covers V nodes");
-  const int H = rg.halo;
-  const unsigned per = (unsigned)(g.nchunks + 2 * H);
+  const int H = rg.halo, nchunks = rows_chunks(g);
+  const unsigned per = (unsigned)(nchunks + 2 * H);
   const unsigned pos = task * (unsigned)(32 - 2 * H) + (unsigned)lane;
   unsigned seg = pos / per;
   const int vc = (int)(pos - seg * per) - H;  // chunk before the wrap
   const bool in = seg < (unsigned)rg.segs;
   if (!in) seg = 0;
-  const bool out = in && lane >= H && lane < 32 - H && vc >= 0 && vc < g.nchunks;
+  const bool out = in && lane >= H && lane < 32 - H && vc >= 0 && vc < nchunks;
   const int y0 = (int)seg * rg.rows, y1 = min(y0 + rg.rows, g.ny);
-  const int c = vc < 0 ? vc + g.nchunks : (vc >= g.nchunks ? vc - g.nchunks : vc);
+  const int c = vc < 0 ? vc + nchunks : (vc >= nchunks ? vc - nchunks : vc);
   const int x0 = c * V;
-  Seam S;
+  Seam<W> S;
   S.el = (g.nx - 1) & (V - 1);
-  S.last = c == g.nchunks - 1;
+  S.last = c == nchunks - 1;
   S.warp = S.el != V - 1 && __any_sync(0xffffffffu, S.last);
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < W; ++q)
     S.word[q] = S.last && S.el * (int)sizeof(T) / 4 == q ? 0xffffffffu : 0u;
   S.up = sizeof(T) == 2 && S.last && !(S.el & 1) ? 16 : 0;
   const int ya = y0 - (STEPS - 1);
@@ -227,7 +232,7 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
     while (y >= g.ny) y -= g.ny;
     return src + (long long)y * g.rstride;
   };
-  uint4 *raw = sm + lane, *dly = sm + 9 * 32 + lane;
+  Vec *raw = sm + lane, *dly = sm + 9 * 32 + lane;
   const T *pm = row_of(ya - 1) + x0, *pc = row_of(ya) + x0, *pp = row_of(ya + 1) + x0;
   int fetched = 0;
   auto fetch = [&]() {  // level 1's row ya + fetched
@@ -235,7 +240,7 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         const T *row = CYd(i) == 1 ? pm : (CYd(i) == -1 ? pp : pc);
-        cp_async16(raw + i * 32, row + (long long)i * g.plane);
+        cp_async(raw + i * 32, row + (long long)i * g.plane);
       }
       ++fetched;
       pm = pc;
@@ -246,45 +251,47 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
   };
   fetch();
   T *drow = dst + (long long)y0 * g.rstride + x0;
-  const bool fill = (g.nchunks & 1) && out && S.last;  // see fills_sector
+  // padding chunks that complete the row's last sector (see fills_sector)
+  constexpr int SECTOR = 32 / (int)sizeof(Vec);
+  const int fill = out && S.last ? (SECTOR - nchunks % SECTOR) % SECTOR : 0;
   for (int j = 0; j < n; ++j) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    uint32_t w[9][4];
+    uint32_t w[9][W];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) set4(w[i], raw[i * 32]);
+    for (int i = 0; i < 9; ++i) set_words(w[i], raw[i * 32]);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) shift_chunk<T>(w[i], CXd(i), S);
+    for (int i = 0; i < 9; ++i) shift_chunk<T, W>(w[i], CXd(i), S);
     fetch();
-    collide_chunk<T>(w, par);
+    collide_chunk<T, W>(w, par);
 #pragma unroll
     for (int l = 1; l < STEPS; ++l) {
       if (j < 2 * (l - 1)) break;  // level l has no row yet
-      uint4 *a = dly + (l - 1) * (9 * 32), *b = a + (3 + 3 * (j & 1)) * 32;
-      uint32_t u[9][4];
-      set4(u[0], a[0]); set4(u[1], a[32]); set4(u[3], a[64]);
-      set4(u[2], b[0]); set4(u[5], b[32]); set4(u[6], b[64]);
-      a[0] = get4(w[0]); a[32] = get4(w[1]); a[64] = get4(w[3]);
-      b[0] = get4(w[2]); b[32] = get4(w[5]); b[64] = get4(w[6]);
+      Vec *a = dly + (l - 1) * (9 * 32), *b = a + (3 + 3 * (j & 1)) * 32;
+      uint32_t u[9][W];
+      set_words(u[0], a[0]); set_words(u[1], a[32]); set_words(u[3], a[64]);
+      set_words(u[2], b[0]); set_words(u[5], b[32]); set_words(u[6], b[64]);
+      a[0] = get_words(w[0]); a[32] = get_words(w[1]); a[64] = get_words(w[3]);
+      b[0] = get_words(w[2]); b[32] = get_words(w[5]); b[64] = get_words(w[6]);
       if (j < 2 * l) break;
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         if (CYd(i) != -1) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) w[i][q] = u[i][q];
+          for (int q = 0; q < W; ++q) w[i][q] = u[i][q];
         }
-        shift_chunk<T>(w[i], CXd(i), S);
+        shift_chunk<T, W>(w[i], CXd(i), S);
       }
-      collide_chunk<T>(w, par);
+      collide_chunk<T, W>(w, par);
     }
     if (j >= 2 * (STEPS - 1)) {
       if (out && y0 + j - 2 * (STEPS - 1) < y1) {
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-          *reinterpret_cast<uint4 *>(drow + (long long)i * g.plane) = get4(w[i]);
-        if (fill) {
+          *reinterpret_cast<Vec *>(drow + (long long)i * g.plane) = get_words(w[i]);
+        for (int k = 1; k <= fill; ++k) {
 #pragma unroll
           for (int i = 0; i < 9; ++i)
-            *reinterpret_cast<uint4 *>(drow + (long long)i * g.plane + V) = make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<Vec *>(drow + (long long)i * g.plane + k * V) = Vec{};
         }
       }
       drow += g.rstride;
@@ -298,14 +305,15 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
 // 3071 FP16 at 6.5 instead of 5.5 ms per 100 steps).  The FMA pipe is 70%
 // busy on 8192^2 FP32 (251 GLUPS), with 54% of the issue slots used.
 template <typename T, int STEPS>
-__global__ void __launch_bounds__(64, sizeof(T) == 4 ? 8 : 4)
+__global__ void __launch_bounds__(64, 8)
 k_step_rows(const T *__restrict__ src, T *__restrict__ dst, Geom g, RowsGeom rg,
             typename PairParams<T>::type P, unsigned ntasks) {
   extern __shared__ uint4 rows_smem[];
   const unsigned warp = threadIdx.x >> 5, task = blockIdx.x * 2 + warp;
   pdl_wait();
   if (task >= ntasks) return;
-  uint4 *sm = rows_smem + warp * rows_smem_words(STEPS);
+  using Vec = typename RowsVec<T>::type;
+  Vec *sm = reinterpret_cast<Vec *>(rows_smem) + warp * rows_smem_chunks(STEPS);
   if constexpr (sizeof(T) == 4)
     rows_task<T, STEPS>(src, dst, g, rg, P, task, threadIdx.x & 31, sm);
   else
@@ -314,7 +322,7 @@ k_step_rows(const T *__restrict__ src, T *__restrict__ dst, Geom g, RowsGeom rg,
 
 template <typename T, int STEPS>
 cudaError_t launch_rows_steps(const Lattice &L, const void *src, void *dst, cudaStream_t st) {
-  constexpr size_t smem = 2 * rows_smem_words(STEPS) * sizeof(uint4);
+  constexpr size_t smem = 2 * rows_smem_chunks(STEPS) * sizeof(typename RowsVec<T>::type);
   cudaError_t e = cudaFuncSetAttribute(
       k_step_rows<T, STEPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;
@@ -358,12 +366,14 @@ template <> struct RowsShared<float> {
 };
 
 template <typename T>
-__global__ void __maxnreg__(sizeof(T) == 4 ? 168 : 255)
+__global__ void __maxnreg__(sizeof(T) == 4 ? 168 : 128)
 k_rows_batch(const BatchEntry *__restrict__ ents, const RowsRec *__restrict__ recs, int nents,
              int parity, const int *__restrict__ limits, int k) {
   extern __shared__ uint4 rows_smem[];
+  using Vec = typename RowsVec<T>::type;
   RowsShared<T> &S =
-      *reinterpret_cast<RowsShared<T> *>(rows_smem + 2 * rows_smem_words(kRowSteps));
+      *reinterpret_cast<RowsShared<T> *>(reinterpret_cast<Vec *>(rows_smem) +
+                                         2 * rows_smem_chunks(kRowSteps));
   constexpr int NW = sizeof(RowsRec) / 4;
   static_assert(sizeof(RowsRec) % 4 == 0 && NW <= 64, "a record is copied one word per thread");
   if (threadIdx.x < NW)
@@ -385,14 +395,16 @@ k_rows_batch(const BatchEntry *__restrict__ ents, const RowsRec *__restrict__ re
   const int from = parity ^ S.rec.off;
   rows_task<T, kRowSteps>(static_cast<const T *>(S.rec.buf[from]),
                           static_cast<T *>(S.rec.buf[from ^ 1]), S.rec.g, rg, S.constants(), task,
-                          threadIdx.x & 31, rows_smem + warp * rows_smem_words(kRowSteps));
+                          threadIdx.x & 31,
+                          reinterpret_cast<Vec *>(rows_smem) + warp * rows_smem_chunks(kRowSteps));
 }
 
 template <typename T>
 cudaError_t launch_rows_batch_t(const BatchList &bl, int parity, cudaStream_t st,
                                 const int *limits, int k) {
   if (bl.nrows < 1) return cudaSuccess;
-  constexpr size_t smem = 2 * rows_smem_words(kRowSteps) * sizeof(uint4) + sizeof(RowsShared<T>);
+  constexpr size_t smem =
+      2 * rows_smem_chunks(kRowSteps) * sizeof(typename RowsVec<T>::type) + sizeof(RowsShared<T>);
   cudaError_t e = cudaFuncSetAttribute(
       k_rows_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;

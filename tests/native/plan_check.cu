@@ -36,13 +36,13 @@ static void check(int nx, int ny, int dtype, int esize) {
   // rows: every chunk of every row is some task's own exactly once (its lanes
   // but `halo` on each side), for small lattices by enumeration
   for (int rows : {1, 8, 32}) {
-    const RowsGeom r = rows_geom(L.g, V, rows);
+    const RowsGeom r = rows_geom(L.g, rows);
     CHECK(r.rows >= 1 && r.segs >= 1 && (long long)r.segs * r.rows >= ny &&
               (long long)(r.segs - 1) * r.rows < ny,
           "segs %d x %d of %d rows", r.segs, r.rows, ny);
-    const int per = L.g.nchunks + 2 * r.halo;
+    const int per = rows_chunks(L.g) + 2 * r.halo;
     // a halo lane of the partial last chunk alone must hold a node per step
-    CHECK(r.halo == 2 || nx % V == 0 || nx % V >= kRowSteps, "halo %d nx %d", r.halo, nx);
+    CHECK(r.halo == 2 || nx % kRowsV == 0 || nx % kRowsV >= kRowSteps, "halo %d nx %d", r.halo, nx);
     if ((long long)nx * ny > 20000) continue;
     std::vector<int> seen((size_t)r.segs * per, 0);
     for (int t = 0; t < r.tasks; ++t)
@@ -52,13 +52,13 @@ static void check(int nx, int ny, int dtype, int esize) {
       }
     for (size_t p = 0; p < seen.size(); ++p) {
       const int c = (int)(p % per) - r.halo;
-      CHECK((c < 0 || c >= L.g.nchunks) ? seen[p] <= 1 : seen[p] == 1, "position %zu seen %d", p,
+      CHECK((c < 0 || c >= rows_chunks(L.g)) ? seen[p] <= 1 : seen[p] == 1, "position %zu seen %d", p,
             seen[p]);
     }
   }
   double rus = 0;
-  const RowsGeom r = plan_rows(L.g, V, esize, sms, &rus);
-  CHECK(rows_fit(L.g, V) ? (r.rows >= 1 && r.rows <= 48 && rus > 0) : r.rows == 0, "rows %d", r.rows);
+  const RowsGeom r = plan_rows(L.g, esize, sms, &rus);
+  CHECK(rows_fit(L.g) ? (r.rows >= 1 && r.rows <= 48 && rus > 0) : r.rows == 0, "rows %d", r.rows);
   double us = 0;
   const TileGeom t = plan_tile(L.g, esize, sms, &us);
   if (t.steps > 0) {
