@@ -30,7 +30,7 @@ inline bool rows_fit(const Geom &g) {
 }
 
 // resident warps per SM of k_step_rows
-inline int rows_warps(int esize) { return esize == 4 ? 16 : 8; }
+constexpr int kRowsWarps = 16;
 
 // Work of k_step_rows over a lattice, or summed over a batch's: its tasks and
 // the nodes they compute per step (idle lanes, halo lanes and rows included).
@@ -48,7 +48,7 @@ struct RowsWork {
 // 700^2 FP32 4.7 / 5.1, 4097 x 3071 FP16 59.6 / 59, 2500 x 2001 FP16 26 /
 // 24.6.
 inline double rows_us(const RowsWork &w, int esize, int sms) {
-  const double per_slot = w.tasks / ((double)sms * rows_warps(esize));
+  const double per_slot = w.tasks / ((double)sms * kRowsWarps);
   const double rate = (esize == 4 ? 285e3 : 300e3) * per_slot / (per_slot + 0.25);
   return w.nodes / rate;
 }

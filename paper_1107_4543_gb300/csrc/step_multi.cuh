@@ -11,9 +11,10 @@
 // passes over memory and fewer launches:
 //
 //   k_step_rows  (large lattices, batches): each warp marches along y over
-//     30 chunks of V nodes, kRowSteps time levels deep; level l of row y needs level l-1 of rows y-1, y, y+1, which the warp has just
-//     computed, so intermediate levels live in lane-private shared-memory
-//     slots and no warp waits for another.
+//     30 chunks of kRowsV nodes, kRowSteps time levels deep; level l of row y
+//     needs level l-1 of rows y-1, y, y+1, which the warp has just computed,
+//     so intermediate levels live in lane-private shared-memory slots and no
+//     warp waits for another.
 //   k_step_tile  (small lattices): each block loads a tile with a halo as
 //     wide as the steps of the launch into shared memory and steps it there,
 //     the valid part shrinking by one node per side and step.
@@ -186,7 +187,7 @@ constexpr int rows_smem_chunks(int steps) { return (9 + 9 * (steps - 1)) * 32; }
 // two aligned chunks, cost 25 - 35% of the rate of ragged FP32 lattices.)
 //
 // After each level one more node of each halo chunk is invalid, so STEPS <=
-// V levels leave the own chunks exact; in y each level loses one row per
+// kRowsV levels leave the own chunks exact; in y each level loses one row per
 // side, so level l (1 .. STEPS) covers rows y0 - (STEPS - l) .. y1 - 1 +
 // (STEPS - l).  In iteration j level 1 takes row y0 - (STEPS - 1) + j and
 // level l the row l - 1 below it: its populations with c_y = -1 come from
@@ -299,11 +300,12 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
   }
 }
 
-// Register budgets, 64-thread blocks: FP32 128 (116 used; 16 warps per SM,
-// which their 13.8 KB of shared memory per warp allows too), 16 bits 255
-// (210 used, 8 warps; at 168 registers, 12 warps, they spill and run 4097 x
-// 3071 FP16 at 6.5 instead of 5.5 ms per 100 steps).  The FMA pipe is 70%
-// busy on 8192^2 FP32 (251 GLUPS), with 54% of the issue slots used.
+// Register budgets, 64-thread blocks: 128 (116 used in FP32, 120 in 16 bits,
+// no spills), 16 warps per SM, which their shared memory (13.8 KB per warp in
+// FP32) allows too.  The FMA pipe is 70% busy on 8192^2 FP32 (251 GLUPS), with
+// 54% of the issue slots used.  16 bits: chunks of eight nodes per lane took
+// 210 registers, 8 warps, FMA pipe 65% (the conversions run on it); four nodes
+// take the 128-lattice FP16 sweep from 43.3 to 42.1 ms.
 template <typename T, int STEPS>
 __global__ void __launch_bounds__(64, 8)
 k_step_rows(const T *__restrict__ src, T *__restrict__ dst, Geom g, RowsGeom rg,
