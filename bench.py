@@ -4,17 +4,18 @@
 Default workload (one JSON line): 512 independent periodic lattices, areas
 log-uniform in [32^2, 1024^2] (6.7e7 nodes), per-lattice relaxation rates,
 Gaussian pulses, FP32 deviation storage.  One benchmark step = the whole
-batch advanced 500 time steps (500 batched fused step launches replayed from
-CUDA graphs) followed by the FP64 drift check of every lattice (one batched
+batch advanced 500 time steps (batched fused launches of three steps each,
+replayed from CUDA graphs) followed by the FP64 drift check of every lattice (one batched
 reduction).
 
   value      MLUPS with the populations resident in HBM
   e2e        MLUPS through the C ABI with host buffers: every step uploads
              the initial fields (rho, ux, uy) from pinned host memory
              (packed batch I/O), steps, and downloads rho, ux, uy
-  roofline   the batched step kernel: algorithmic 72 B per lattice update
-             over its average launch time against the measured HBM copy
-             bandwidth
+  roofline   the batched step kernel: algorithmic 72 B per node and launch
+             (one read and one write of the populations for its three time
+             steps) over its average launch time against the measured HBM
+             copy bandwidth; its FP32 arithmetic is the nearer bound
   fp64_plain the plain FP64 path on one 8192^2 lattice, for comparison
   cpu_baseline  the FP64 CPU oracle on a bounded sample of the workload
 
@@ -46,9 +47,19 @@ sys.path.insert(0, ROOT)
 import lbm_inputs as inp  # noqa: E402
 
 BYTES_PER_LU = {"f64": 144, "f64dev": 144, "f32": 72, "f16": 36, "bf16": 36}
+# time steps per launch on large lattices and batches of the 32- and 16-bit
+# types (kRowSteps in csrc/lbm_internal.h); the FP64 types take one
+STEPS_PER_LAUNCH = 3
+
+
+def hbm_bytes_per_update(dtype):
+    """HBM bytes of one lattice update: the populations cross once each way per launch."""
+    return BYTES_PER_LU[dtype] / (1 if dtype.startswith("f64") else STEPS_PER_LAUNCH)
+
+
 KERNEL_SOURCES = ["csrc/step_impl.cuh", "csrc/d2q9_pull.cuh", "csrc/collide.cuh",
                   "csrc/step_f32.cu", "csrc/step_f16.cu", "csrc/step_bf16.cu", "csrc/step_f64.cu",
-                  "csrc/step_f64dev.cu", "csrc/resident.cuh"]
+                  "csrc/step_f64dev.cu", "csrc/resident.cuh", "csrc/step_multi.cuh"]
 
 
 def parser():
@@ -380,13 +391,6 @@ def bench_batched(args, L, torch, rank, ws):
     resident = L.lbm_batch_resident(b)
     res_nodes = sum(s["nx"] * s["ny"] for s, r in zip(specs, resident) if r)
     step_nodes = nodes - res_nodes  # the per-step kernel's lattice updates
-    # one resident launch per non-empty size class (up to a third, a half,
-    # all of a block's shared memory) per call
-    optin = torch.cuda.get_device_properties(dev).shared_memory_per_block_optin
-    esize = {"f32": 4, "f16": 2, "bf16": 2}[bdt]
-    res_classes = len({0 if rb <= optin // 3 else (1 if rb <= optin // 2 else 2)
-                       for rb in (2 * 9 * s["nx"] * s["ny"] * esize
-                                  for s, r in zip(specs, resident) if r)})
     # one launch per call refreshes the batch's slots of the constant table
     # (a single storage type here) when it holds any
     table_fills = int(L.lbm_batch_const_table(b).any())
@@ -398,7 +402,6 @@ def bench_batched(args, L, torch, rank, ws):
     for _ in range(args.warmup):
         one_step()
     torch.cuda.synchronize()
-    variant = L.lbm_batch_get_variant(b)
     if ws > 1:
         torch.distributed.barrier()
     clocks = Clocks(dev)
@@ -421,10 +424,13 @@ def bench_batched(args, L, torch, rank, ws):
     lu_per_step = nodes * lbm_steps
     lu_job = reduce_sum(lu_per_step * args.steps)  # every rank's lattice updates
     value = job_mlups(lu_job, total_ms * 1e-3)
-    launch_ms = float(np.mean(step_ms)) / lbm_steps  # one batched kernel per time step
-    # batched steps, the resident launches, the constant-table refresh and
-    # one drift launch pair
-    launches = args.steps * (lbm_steps + 2 + res_classes + table_fills)
+    # batched launches of STEPS_PER_LAUNCH time steps, single ones for the
+    # remainder
+    step_launches = lbm_steps // STEPS_PER_LAUNCH + lbm_steps % STEPS_PER_LAUNCH
+    launch_ms = float(np.mean(step_ms)) / (lbm_steps / STEPS_PER_LAUNCH)
+    # those, the resident launch, the constant-table refresh and one drift
+    # launch pair
+    launches = args.steps * (step_launches + 2 + int(resident.any()) + table_fills)
 
     # e2e: host fields in, moments out, through the public API: one
     # lbm_batch_solve_packed call per benchmark step (upload of the fields
@@ -484,13 +490,13 @@ def bench_batched(args, L, torch, rank, ws):
     kname = {"f32": "float", "f16": "__half", "bf16": "__nv_bfloat16"}[bdt]
     sname = {"f32": "FP32", "f16": "FP16", "bf16": "BF16"}[bdt]
     achieved = BYTES_PER_LU[bdt] * step_nodes / (launch_ms * 1e-3) / 1e9
-    tr = traffic_record("k_step_batch<%s>" % kname)
-    roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
+    tr = traffic_record("k_rows_batch<%s>" % kname)
+    roofline = {"bound": "fma", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4),
                 # ncu DRAM bytes per lattice update of a smaller capture of the
                 # same kernel, scaled to this launch's lattice updates
                 "traffic": (round(tr["dram_bytes_per_lu"] * step_nodes) if tr else None),
-                "kernel": "k_step_batch<%s> (launch variant %d)" % (kname, variant),
+                "kernel": "k_rows_batch<%s>" % kname, "steps_per_launch": STEPS_PER_LAUNCH,
                 "peak_source": peak_kind,
                 "algorithmic_bytes_per_launch": BYTES_PER_LU[bdt] * step_nodes,
                 "avg_launch_ms": round(launch_ms, 4),
@@ -574,14 +580,15 @@ def bench_large(args, L, torch, rank, ws):
     peak, peak_kind = peaks()
     for dtype in args.dtypes.split(","):
         lbm_steps = 50 if not dtype.startswith("f64") else 10
-        mlups, launch_ms = large_one(L, torch, stream, n, dtype, lbm_steps, args.steps,
-                                     args.warmup)
-        achieved = BYTES_PER_LU[dtype] * n * n / (launch_ms * 1e-3) / 1e9
+        mlups, step_ms = large_one(L, torch, stream, n, dtype, lbm_steps, args.steps,
+                                   args.warmup)
+        achieved = hbm_bytes_per_update(dtype) * n * n / (step_ms * 1e-3) / 1e9
         lines.append({"metric": "MLUPS, single %dx%d lattice" % (n, n), "value": round(mlups, 1),
                       "unit": "MLUPS", "dtype": dtype, "n_gpus": ws, "steps": args.steps,
                       "warmup": args.warmup, "higher_is_better": True,
                       "config": {"workload": "single-%dx%d-%s" % (n, n, dtype)},
-                      "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
+                      "roofline": {"bound": "fp64-alu" if dtype.startswith("f64") else "fma",
+                                   "achieved": round(achieved, 1), "peak": peak,
                                    "unit": "GB/s", "frac": round(achieved / peak, 4),
                                    "peak_source": peak_kind}})
     return lines
@@ -590,22 +597,23 @@ def bench_large(args, L, torch, rank, ws):
 def config3_record(L, torch):
     """Config 3 at its stated size: one 8192^2 lattice, 1000 time steps, per
     storage type (FP32, FP16, BF16 deviation and plain FP64), each with the
-    roofline of its step kernel (algorithmic bytes per lattice update over
-    the average step time against the measured HBM copy rate; FP64 is bound
-    by GB300's FP64 pipe, its fraction is of the same HBM peak)."""
+    roofline of its step kernel (the populations' bytes, once each way per
+    launch, over the average time against the measured HBM copy rate; the FMA
+    pipe bounds the 32- and 16-bit types, the FP64 pipe FP64: their fractions
+    are of the same HBM peak)."""
     stream = torch.cuda.current_stream()
     peak, peak_kind = peaks()
     n, steps = 8192, 1000
     out = {"workload": "single-8192x8192-1000-steps", "note": "one timed run of 1000 steps "
            "after 2 x 50 warm-up steps; 2.4-9.7 GB of populations per type (> L2)"}
-    kern = {"f32": "k_step_dev<float>", "f16": "k_step_dev<__half>",
-            "bf16": "k_step_dev<__nv_bfloat16>", "f64": "k_step_f64",
+    kern = {"f32": "k_step_rows<float>", "f16": "k_step_rows<__half>",
+            "bf16": "k_step_rows<__nv_bfloat16>", "f64": "k_step_f64",
             "f64dev": "k_step_dev<double>"}
     for dtype in ("f32", "f16", "bf16", "f64", "f64dev"):
         mlups, ms = large_one(L, torch, stream, n, dtype, steps, 1, 2)
-        achieved = BYTES_PER_LU[dtype] * n * n / (ms * 1e-3) / 1e9
+        achieved = hbm_bytes_per_update(dtype) * n * n / (ms * 1e-3) / 1e9
         out[dtype] = {"mlups": round(mlups, 1), "ms_per_lbm_step": round(ms, 4),
-                      "roofline": {"bound": "hbm" if not dtype.startswith("f64") else "fp64-alu",
+                      "roofline": {"bound": "fma" if not dtype.startswith("f64") else "fp64-alu",
                                    "kernel": kern[dtype], "achieved": round(achieved, 1),
                                    "peak": peak, "unit": "GB/s",
                                    "frac": round(achieved / peak, 4), "peak_source": peak_kind}}
