@@ -649,7 +649,7 @@ static std::vector<size_t> packed_groups(const lbm_batch_ctx *b) {
 // first, so that the short ones fill the tail of the launch.
 static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms) {
   std::vector<RowsRec> recs;
-  constexpr int kChoices = sizeof(kRowChoices) / sizeof(kRowChoices[0]);
+  constexpr int kChoices = sizeof(kBatchRowChoices) / sizeof(kBatchRowChoices[0]);
   RowsWork work[kChoices];
   const int esize = dt == LBM_F32DEV ? 4 : 2;
   double nodes = 0;
@@ -658,14 +658,14 @@ static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms
     if (L.dtype != dt || b->member_res[mi]) continue;
     if (!rows_fit(L.g)) return recs;
     nodes += (double)L.g.nx * L.g.ny;
-    for (int k = 0; k < kChoices; ++k) work[k].add(rows_geom(L.g, kRowChoices[k]));
+    for (int k = 0; k < kChoices; ++k) work[k].add(rows_geom(L.g, kBatchRowChoices[k]));
   }
   double us = 0.95 * single_us(nodes, esize);
   int rows = 0;
   for (int k = 0; k < kChoices; ++k)
-    if (nodes > 0 && rows_us(work[k], esize, sms) < us) {
-      us = rows_us(work[k], esize, sms);
-      rows = kRowChoices[k];
+    if (nodes > 0 && rows_batch_us(work[k], esize, sms) < us) {
+      us = rows_batch_us(work[k], esize, sms);
+      rows = kBatchRowChoices[k];
     }
   if (rows == 0) return recs;
   for (size_t mi = 0; mi < b->members.size(); ++mi) {

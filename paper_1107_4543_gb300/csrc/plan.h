@@ -47,10 +47,20 @@ struct RowsWork {
 // estimated: 8192^2 276 / 277 FP32 and 262 / 262 FP16, 1024^2 FP32 7.3 / 7.7,
 // 700^2 FP32 4.7 / 5.1, 4097 x 3071 FP16 59.6 / 59, 2500 x 2001 FP16 26 /
 // 24.6.
-inline double rows_us(const RowsWork &w, int esize, int sms) {
+inline double rows_us(const RowsWork &w, int esize, int sms, double half = 0.25) {
   const double per_slot = w.tasks / ((double)sms * kRowsWarps);
-  const double rate = (esize == 4 ? 285e3 : 300e3) * per_slot / (per_slot + 0.25);
+  const double rate = (esize == 4 ? 285e3 : 300e3) * per_slot / (per_slot + half);
   return w.nodes / rate;
+}
+
+// The same for a batch (k_rows_batch): its constants come from shared memory,
+// and where it has more than a task or two per slot, short segments fill the
+// tail.
+// Measured / estimated, 128 lattices of 32^2 .. 1024^2: FP32 in segments of 8,
+// 16, 28, 32 rows 91 / 83, 85 / 79, 81 / 77, 81 / 77 us, FP16 83 / 79, 80 /
+// 74, 78 / 73, 79 / 73.
+inline double rows_batch_us(const RowsWork &w, int esize, int sms) {
+  return std::max(rows_us(w, esize, sms), 1.15 * rows_us(w, esize, sms, 0.1));
 }
 
 // Estimated us of one single-step launch over `nodes` nodes: its latency and
@@ -65,6 +75,7 @@ inline double single_us(double nodes, int esize) {
 // The segment heights tried: low ones cost redundant rows (2 (kRowSteps - 1)
 // per segment), high ones leave too few tasks.
 constexpr int kRowChoices[] = {8, 12, 16, 24, 32};
+constexpr int kBatchRowChoices[] = {8, 12, 16, 20, 24, 28, 32};
 
 // k_step_rows' best split of one lattice and its estimate (rows = 0: the
 // lattice does not fit it)
