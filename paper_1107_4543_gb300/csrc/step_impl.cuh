@@ -86,7 +86,7 @@ __device__ __forceinline__ ParamPairs pairs_of(const DevParams &P) { return Para
 __device__ __forceinline__ const ConstPairs &pairs_of(const ConstPairs &P) { return P; }
 
 // P: the lattice's ParamsOf<T>::type, or (16-bit types) a ConstPairs
-template <typename T, typename PS>
+template <typename T, typename LD, typename PS>
 __device__ __forceinline__ void step_task(const T *__restrict__ src, T *__restrict__ dst,
                                           const Geom &g, const PS &P, long long task, int lane) {
   constexpr int V = Elem<T>::V;
@@ -100,12 +100,12 @@ __device__ __forceinline__ void step_task(const T *__restrict__ src, T *__restri
     p.active = false;
   if constexpr (sizeof(T) == 2) {
     uint32_t w[9][V / 2];
-    pull9_packed<T>(src, g, p, w);
+    pull9_packed<T, LD>(src, g, p, w);
     collide_packed<T>(w, pairs_of(P));
     store9_packed<T>(dst, g, p, w);
   } else if constexpr (std::is_same<T, double>::value) {
     double f[9][V];
-    pull9<T, false>(src, g, p, 1.0, f);
+    pull9<T, false, LD>(src, g, p, 1.0, f);
 #pragma unroll
     for (int e = 0; e < V; ++e)
       collide_dev64(f[0][e], f[1][e], f[2][e], f[3][e], f[4][e], f[5][e], f[6][e], f[7][e],
@@ -113,7 +113,7 @@ __device__ __forceinline__ void step_task(const T *__restrict__ src, T *__restri
     store9<T, false>(dst, g, p, 1.0, f);
   } else {
     float f[9][V];
-    pull9<T, false>(src, g, p, 1.0f, f);
+    pull9<T, false, LD>(src, g, p, 1.0f, f);
 #pragma unroll
     for (int e = 0; e < V; ++e)
       collide_dev<PRECISE, SCALED>(f[0][e], f[1][e], f[2][e], f[3][e], f[4][e], f[5][e], f[6][e],
@@ -136,7 +136,7 @@ k_step_dev(const T *__restrict__ src, T *__restrict__ dst, Geom g,
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   pdl_wait();
   for (long long task = warp0; task < ntasks; task += nwarps)
-    step_task<T>(src, dst, g, P, task, lane);
+    step_task<T, LoadOverlapped>(src, dst, g, P, task, lane);
 }
 
 // Whether lattice `lat` takes part in single step k of a ragged generation
@@ -193,12 +193,12 @@ __device__ __forceinline__ void batch_block(const BatchEntry *__restrict__ ents,
   const T *src = static_cast<const T *>(B.buf[from]);
   T *dst = static_cast<T *>(B.buf[from ^ 1]);
   if constexpr (CP && sizeof(T) == 2) {
-    step_task<T>(src, dst, B.g, ConstPairs{(pbase + B.lat) * PC_COUNT}, task, lane);
+    step_task<T, LoadReadOnly>(src, dst, B.g, ConstPairs{(pbase + B.lat) * PC_COUNT}, task, lane);
   } else if constexpr (CP) {
     static_assert(sizeof(T) == 4, "constant tables: FP32 and the 16-bit types");
-    step_task<T>(src, dst, B.g, c_dev[pbase + B.lat], task, lane);
+    step_task<T, LoadReadOnly>(src, dst, B.g, c_dev[pbase + B.lat], task, lane);
   } else {
-    step_task<T>(src, dst, B.g, ents[B.lat].dp, task, lane);
+    step_task<T, LoadReadOnly>(src, dst, B.g, ents[B.lat].dp, task, lane);
   }
 }
 
@@ -263,7 +263,7 @@ k_step_batch_stride(const BatchEntry *__restrict__ ents, const BlockRec *__restr
     if (task < B.g.tasks && bounds::ok(B.lat >= 0 && B.lat < nents, bounds::BATCH_REC) &&
         limit_takes(limits, B.lat, k, par)) {  // warp-uniform
       const int from = par ^ B.off;
-      step_task<T>(static_cast<const T *>(B.buf[from]), static_cast<T *>(B.buf[from ^ 1]), B.g,
+      step_task<T, LoadReadOnly>(static_cast<const T *>(B.buf[from]), static_cast<T *>(B.buf[from ^ 1]), B.g,
                    ents[B.lat].dp, task, lane);
     }
     if (nb >= nblocks) break;
