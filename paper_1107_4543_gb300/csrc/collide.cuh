@@ -505,6 +505,25 @@ struct F64Params {
   double s3, s4, s5, s6, s7, s8;
 };
 
+// 1 / b correctly rounded (Markstein, IBM J. Res. Dev. 34 (1990) 111): r (1 +
+// e + e^2), e = 1 - b r exact, takes the hardware's approximation (a relative
+// error of about 2^-20) to within 2^-60 before its rounding, so to the nearest
+// FP64 number or, next to a midpoint, the other one; one more step r + r (1 -
+// b r), its difference exact, then rounds correctly for every significand but
+// the one of all ones.  recip_rounds says that b is not that one and, like its
+// reciprocal, far from overflow and underflow.
+__device__ __forceinline__ bool recip_rounds(double b) {  // 2^-500 <= |b| < 2^500
+  const unsigned hi = (unsigned)__double2hiint(b), lo = (unsigned)__double2loint(b);
+  return ((hi >> 20) & 0x7ffu) - 523u < 1000u && ((hi | 0xfff00000u) & lo) != 0xffffffffu;
+}
+__device__ __forceinline__ double recip(double b) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+  const double e = fma(-b, r, 1.0);
+  r = fma(r, fma(e, e, e), r);
+  return fma(r, fma(-b, r, 1.0), r);
+}
+
 // a / b correctly rounded, for the three quotients of one collision by the
 // same b: with y = 1/b correctly rounded (two Newton-Raphson steps from the
 // hardware's approximation), q = a y and the exact remainder r = a - b q give

@@ -11,11 +11,11 @@
 // jx jy/rho - jx0 jy0/rho0: every term is of the size of the perturbation,
 // so nothing of order one is subtracted after rounding.  GB300's FP64 rate
 // (1/64 of FP32) bounded these kernels, not their 60 bytes per node (8192^2
-// FP32: init 8.1 ms, moments 4.6 ms, against 0.6 ms of HBM traffic), so only
+// FP32: init 6.1 ms, moments 4.6 ms, against 0.6 ms of HBM traffic), so only
 // what needs FP64 runs there: the init forms the six differences in FP64 and
-// their linear combinations as float-float sums, and the moments sum the
-// stored values as float-float (feq_rounded, moments_node): 1.7 and 2.4 ms,
-// the FP64 form's values in the init and within 2^-45 in the moments.
+// their linear combinations as float-float sums (feq_rounded), and the
+// moments sum the stored values as float-float where those sums are exact
+// (sums_exact): 1.4 and 2.5 ms, with the FP64 form's bits in both.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
@@ -131,7 +131,7 @@ __device__ __forceinline__ bool ff_split(double d, FF &o, float &lost) {
 // same operations, their combinations as float-float to ~2^-44 of the
 // largest term (in units of the diagonal weight 1/36: the other weights are
 // 4 and 16 times that).  A value whose rounding that error could change --
-// one in ~10^4 -- or a difference outside the split's range returns false,
+// one node in several thousand -- or a difference outside the split's range returns false,
 // and the caller takes the FP64 form.
 __device__ __forceinline__ bool feq_rounded(const RefState &R, double r, double u, double v,
                                             float d[9]) {
@@ -290,15 +290,22 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(mag << 29));
 }
 __device__ __forceinline__ double ff_value(FF s) { return widen(s.h) + widen(s.l); }
-// 1 / r within an ulp: the hardware's approximation and two Newton-Raphson
-// steps, the ordinary division where those could overflow
-__device__ __forceinline__ double reciprocal(double r) {
-  const unsigned e = ((unsigned)__double2hiint(r) >> 20) & 0x7ffu;
-  if (e - 523u >= 1000u) return 1.0 / r;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r));
-  y = fma(y, fma(-r, y, 1.0), y);
-  return fma(y, fma(-r, y, 1.0), y);
+// Whether the sums over nine FP32 values come out exact both in FP64 and as
+// float-float, so that the cheaper one gives the FP64 form's bits.  Values of
+// exponents e0 .. e1 (zeros apart) are multiples of 2^(e0 - 23), and partial
+// sums stay below 2^(e1 + 5): FP64 holds them for e1 - e0 <= 25, and the FP32
+// sum of the two_sum errors, each at most 2^(e1 - 20), for e1 - e0 <= 18.
+// Infinities, NaN and sums that FP32 could not hold fail the test too.
+__device__ __forceinline__ bool sums_exact(const float (&f)[9]) {
+  unsigned top = 0u, low = 0xffffffffu;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    const unsigned mag = __float_as_uint(f[i]) & 0x7fffffffu;
+    top = max(top, mag);
+    low = min(low, mag - 1u);  // a zero is no bound
+  }
+  top >>= 23;
+  return top - ((low + 1u) >> 23) <= 18u && top <= 248u;
 }
 
 // rho = rho0 + sum f', j = j0 + sum c f' of the pre-collision populations
@@ -322,8 +329,8 @@ __device__ __forceinline__ void moments_node(const AuxView &a, int x, int y, flo
     u = jx * inv;
     v = jy * inv;
   } else {
-    // the deviations' sums as float-float (~48 bits of the stored 24 or
-    // fewer), then two FP64 additions each and one reciprocal
+    // the FP64 sums from left to right; as float-float and one FP64 addition
+    // where that is known to give the same
     float f[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -331,14 +338,27 @@ __device__ __forceinline__ void moments_node(const AuxView &a, int x, int y, flo
       f[i] = decode_f32<T>(buf[(long long)i * a.g.plane + (long long)ys * a.g.rstride + xs],
                            inv_scale);
     }
-    FF s0{f[0], 0.0f}, s1{f[1], 0.0f}, s2{f[2], 0.0f};
+    double S0, S1, S2;
+    if (sums_exact(f)) {
+      FF s0{f[0], 0.0f}, s1{f[1], 0.0f}, s2{f[2], 0.0f};
 #pragma unroll
-    for (int i = 1; i < 9; ++i) ff_acc(s0, f[i]);
-    ff_acc(s1, -f[3]); ff_acc(s1, f[5]); ff_acc(s1, -f[6]); ff_acc(s1, -f[7]); ff_acc(s1, f[8]);
-    ff_acc(s2, -f[4]); ff_acc(s2, f[5]); ff_acc(s2, f[6]); ff_acc(s2, -f[7]); ff_acc(s2, -f[8]);
-    r = a.rho0 + ff_value(s0);
-    const double jx = a.jx0 + ff_value(s1), jy = a.jy0 + ff_value(s2);
-    const double inv = reciprocal(r);
+      for (int i = 1; i < 9; ++i) ff_acc(s0, f[i]);
+      ff_acc(s1, -f[3]); ff_acc(s1, f[5]); ff_acc(s1, -f[6]); ff_acc(s1, -f[7]); ff_acc(s1, f[8]);
+      ff_acc(s2, -f[4]); ff_acc(s2, f[5]); ff_acc(s2, f[6]); ff_acc(s2, -f[7]); ff_acc(s2, -f[8]);
+      S0 = ff_value(s0);
+      S1 = ff_value(s1);
+      S2 = ff_value(s2);
+    } else {
+      double d[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) d[i] = (double)f[i];
+      S0 = d[0] + d[1] + d[2] + d[3] + d[4] + d[5] + d[6] + d[7] + d[8];
+      S1 = d[1] - d[3] + d[5] - d[6] - d[7] + d[8];
+      S2 = d[2] - d[4] + d[5] + d[6] - d[7] - d[8];
+    }
+    r = a.rho0 + S0;
+    const double jx = a.jx0 + S1, jy = a.jy0 + S2;
+    const double inv = recip_rounds(r) ? recip(r) : 1.0 / r;
     u = jx * inv;
     v = jy * inv;
   }
