@@ -525,14 +525,15 @@ __device__ __forceinline__ double recip(double b) {
 }
 
 // a / b correctly rounded, for the three quotients of one collision by the
-// same b: with y = 1/b correctly rounded (two Newton-Raphson steps from the
-// hardware's approximation), q = a y and the exact remainder r = a - b q give
-// the correctly rounded quotient q + r y (Markstein, IBM J. Res. Dev. 34
-// (1990) 111).  The argument needs b, the a's and the quotients far from
-// overflow and underflow; `fast` says so from the exponents (a zero a is
-// fine), and anything else takes the ordinary division.  Three quotients
-// cost 4 + 3 x 3 FP64 operations instead of three times the compiler's
-// division sequence.
+// same b: with y = 1 / b correctly rounded (recip), q = a y and the exact
+// remainder r = a - b q give the correctly rounded quotient q + r y
+// (Markstein).  With y one unit off, as two Newton-Raphson steps from the
+// hardware's approximation may leave it, a / b next to a midpoint rounds
+// wrongly: 2^-8 / (1 - 2^-53) did.  The argument needs b, the a's and the
+// quotients far from overflow and underflow; `fast` says so from the
+// exponents (a zero a is fine), and anything else takes the ordinary
+// division.  Three quotients cost 5 + 3 x 3 FP64 operations instead of three
+// times the compiler's division sequence.
 struct Quotients {
   double b, y;
   bool fast;
@@ -542,11 +543,8 @@ struct Quotients {
   }
   __device__ __forceinline__ Quotients(double b_, double a0, double a1, double a2) : b(b_) {
     auto ok = [](double a) { return normal(a) || a_zero(a); };
-    fast = normal(b) && ok(a0) && ok(a1) && ok(a2);
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
-    r = fma(r, fma(-b, r, 1.0), r);
-    y = fma(r, fma(-b, r, 1.0), r);
+    fast = recip_rounds(b) && ok(a0) && ok(a1) && ok(a2);
+    y = recip(b);
   }
   static __device__ __forceinline__ bool a_zero(double a) {
     return (((unsigned)__double2hiint(a) << 1) | (unsigned)__double2loint(a)) == 0u;
@@ -566,7 +564,7 @@ struct Quotients {
 // a bit are saved: products by powers of two are exact, so they ride in
 // fused multiply-adds and are shared between rows that scale alike ((2 a) +
 // (2 b) rounds to 2 (a + b)); the three divisions share one reciprocal
-// (Quotients).  118 instead of ~185 FP64 instructions per node.  Compile
+// (Quotients).  119 instead of ~185 FP64 instructions per node.  Compile
 // without multiply-add contraction (-fmad=false).
 __device__ __forceinline__ void collide_f64(double (&f)[9], const F64Params &P) {
   const double rho = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];

@@ -4,7 +4,7 @@
 // section 2.1 (collide_f64), and this file is compiled with -fmad=false, so
 // the step is bit-identical to a straightforward FP64 CPU implementation of
 // the same definition.  Per node it moves 9 + 9 doubles (144 B) and performs
-// ~118 FP64 operations; on GB300 the FP64 units (two lanes per clock and SM),
+// ~119 FP64 operations; on GB300 the FP64 units (two lanes per clock and SM),
 // not HBM, bound it.
 #include "lbm_internal.h"
 #include "node_xy.cuh"
@@ -15,7 +15,7 @@ namespace lbm {
 // One node per thread and 32-thread blocks: whatever the size, the warps
 // spread evenly over the SMs' FP64 units.  (Warp tasks of 64 nodes with
 // 16-byte vectors, in 256-thread blocks, ran 64^2 on 16 of the 152 SMs, 19.9
-// against 5.2 us per step, and 2048^2 at 951 against 909 - 946 us.)  A warp
+// against 5.2 us per step, and 2048^2 at 951 against 917 - 946 us.)  A warp
 // instruction holds a scheduler's FP64 unit for 64 cycles however many lanes
 // are active, so blocks of fewer nodes gain nothing (8 per warp: 64^2 at
 // 5.9 us).
@@ -45,12 +45,12 @@ __device__ __forceinline__ double quotient(double a, double b) {
 }
 
 // The step of a small lattice: four warps, one per scheduler of an SM, share
-// the FP64 operations of 32 nodes, since one warp's 118 operations at 64
+// the FP64 operations of 32 nodes, since one warp's 119 operations at 64
 // cycles each are the time of a step while there are fewer warps than
-// schedulers.  Three phases, 16 + 15 + 9 operations on the longest warp,
+// schedulers.  Three phases, 16 + 16 + 9 operations on the longest warp,
 // exchange their sums, products and relaxed moments through shared memory;
 // every value is formed by collide_f64's own operations, so the bits are
-// the same.  160 operations in all: past two blocks per SM the plain form is
+// the same.  164 operations in all: past two blocks per SM the plain form is
 // the faster one.  us per step, plain / this: 64^2 5.1 / 3.1, 97 x 100 (304
 // blocks, two per SM) 5.2 / 4.3, 101^2 (319) 5.2 / 5.6, 200^2 11.8 / 14.6.
 __global__ void __launch_bounds__(128)
