@@ -47,6 +47,7 @@ static __constant__ float c_pairs[kPairTable * PC_COUNT];
 static __constant__ DevParams c_dev[kDevTable];
 
 struct ConstPairs {
+  static constexpr bool kTable = true;
   int base;  // first constant of the lattice: slot * PC_COUNT
   __device__ __forceinline__ F2x2 two(PairConst c) const {
     return {f2s(c_pairs[base + c]), f2s(c_pairs[base + c + 1])};

@@ -39,6 +39,7 @@ inline typename PairParams<T>::type pair_params(const DevParams &P) {
 
 // 16-bit constants as broadcast pairs in shared memory (PairConst order)
 struct SharedPairs {
+  static constexpr bool kTable = false;
   const float2 *c;  // 16-byte aligned
   __device__ __forceinline__ F2x2 two(PairConst k) const {
     const float4 v = *reinterpret_cast<const float4 *>(c + k);
