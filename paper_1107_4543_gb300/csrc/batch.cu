@@ -69,10 +69,12 @@ struct lbm_batch_ctx {
     long long nrows = 0;
     // entries held in shared memory for all the steps of a launch (small
     // lattices; k_batch_resident), which the block records leave out, largest
-    // first, and the bytes of the largest one's planes
+    // first: [0] those alone on their SM, [1] those of which two share one
+    // (resident_pairs), and the nodes of each kind's largest
     int nres = 0;
     int *res = nullptr;
-    size_t res_planes = 0;
+    int res_count[2] = {0, 0};
+    long long res_nodes[2] = {0, 0};
     // the group's slots in its type's constant table (-1: none) and the
     // device staging of their refresh (n x const_slot_bytes(dtype))
     int pbase = -1;
@@ -82,9 +84,10 @@ struct lbm_batch_ctx {
   std::vector<int> member_res;                  // member stepped as a resident entry
   bool spent = false;  // a ragged generation ran: members' parities differ
   std::vector<Group> groups;
-  bool resident = false;                 // some group has resident entries
-  cudaStream_t res_stream = nullptr;     // their launches, beside the batch stream
-  cudaEvent_t res_fork = nullptr, res_join = nullptr;
+  bool resident[2] = {false, false};     // some group has resident entries of the kind
+  // their launches, beside the batch stream and one another
+  cudaStream_t res_stream[2] = {nullptr, nullptr};
+  cudaEvent_t res_fork = nullptr, res_join[2] = {nullptr, nullptr};
   std::vector<int> offs;                 // member buffer index at creation
   std::vector<cudaStream_t> saved_streams;
   AuxView *views[2] = {nullptr, nullptr}; // drift views at batch parity 0 / 1
@@ -191,27 +194,30 @@ static int batch_upload_pairs(lbm_batch_ctx *b) {
 
 // Launch the resident entries of every group for `steps` steps from batch
 // parity `parity` (limits: per-entry step limits of a ragged generation, or
-// null) on the side stream, forked from the batch stream; resident_join
+// null) on the side streams, forked from the batch stream; resident_join
 // makes the batch stream wait for them.
 static int resident_fork(lbm_batch_ctx *b, int parity, long steps, bool ragged) {
-  if (!b->resident || steps < 1) return LBM_OK;
-  if (!b->res_stream) {
-    CK(cudaStreamCreateWithFlags(&b->res_stream, cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&b->res_fork, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&b->res_join, cudaEventDisableTiming));
-  }
+  if (!(b->resident[0] || b->resident[1]) || steps < 1) return LBM_OK;
+  if (!b->res_fork) CK(cudaEventCreateWithFlags(&b->res_fork, cudaEventDisableTiming));
   CK(cudaEventRecord(b->res_fork, b->stream));
-  CK(cudaStreamWaitEvent(b->res_stream, b->res_fork, 0));
-  for (auto &gr : b->groups)
-    if (gr.nres > 0)
-      CK(launch_batch_resident(gr.dtype, gr.ents, gr.res, gr.nres, gr.n, gr.res_planes, parity,
-                               steps, ragged ? gr.limits : nullptr, b->res_stream));
-  CK(cudaEventRecord(b->res_join, b->res_stream));
+  for (int c = 0; c < 2; ++c) {
+    if (!b->resident[c]) continue;
+    if (!b->res_stream[c]) CK(cudaStreamCreateWithFlags(&b->res_stream[c], cudaStreamNonBlocking));
+    if (!b->res_join[c]) CK(cudaEventCreateWithFlags(&b->res_join[c], cudaEventDisableTiming));
+    CK(cudaStreamWaitEvent(b->res_stream[c], b->res_fork, 0));
+    for (auto &gr : b->groups)
+      if (gr.res_count[c] > 0)
+        CK(launch_batch_resident(gr.dtype, gr.ents, gr.res + (c ? gr.res_count[0] : 0),
+                                 gr.res_count[c], gr.n, gr.res_nodes[c], parity, steps,
+                                 ragged ? gr.limits : nullptr, b->res_stream[c]));
+    CK(cudaEventRecord(b->res_join[c], b->res_stream[c]));
+  }
   return LBM_OK;
 }
 
 static int resident_join(lbm_batch_ctx *b) {
-  if (b->resident && b->res_join) CK(cudaStreamWaitEvent(b->stream, b->res_join, 0));
+  for (auto *ev : b->res_join)
+    if (ev) CK(cudaStreamWaitEvent(b->stream, ev, 0));
   return LBM_OK;
 }
 
@@ -424,12 +430,12 @@ long long batch_nodes(const lbm_batch_ctx *b) { return b->nodes; }
 
 static void batch_free(lbm_batch_ctx *b) {
   batch_drop_graphs(b);
-  for (auto *st : {b->up, b->down, b->res_stream})
+  for (auto *st : {b->up, b->down, b->res_stream[0], b->res_stream[1]})
     if (st) {
       cudaStreamSynchronize(st);
       cudaStreamDestroy(st);
     }
-  for (auto *ev : {b->res_fork, b->res_join})
+  for (auto *ev : {b->res_fork, b->res_join[0], b->res_join[1]})
     if (ev) cudaEventDestroy(ev);
   for (auto &r : b->ring)
     for (auto &e : r)
@@ -735,6 +741,8 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
   b->member_local.assign(b->members.size(), -1);
   b->member_res.assign(b->members.size(), 0);
   const size_t res_max = resident_limit(dev);
+  size_t sm_bytes = 0, sm_reserved = 0;
+  resident_sm(&sm_bytes, &sm_reserved);
   for (int dt : {LBM_F32DEV, LBM_F16DEV, LBM_BF16DEV}) {
     std::vector<BatchEntry> ents;
     std::vector<BlockRec> bl;  // the plain grid's blocks
@@ -779,6 +787,7 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
     }
     if (ents.empty()) continue;
     const std::vector<RowsRec> rl = rows_records(b, dt, sm_count());
+    const int e_size = dt == LBM_F32DEV ? 4 : 2;
     lbm_batch_ctx::Group gr;
     gr.dtype = dt;
     gr.n = (int)ents.size();
@@ -792,13 +801,13 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
     auto nodes_of = [&](int k) { return (long long)ents[k].g.nx * ents[k].g.ny; };
     std::stable_sort(res.begin(), res.end(),
                      [&](int p, int q) { return nodes_of(p) > nodes_of(q); });
-    if (!res.empty())
-      gr.res_planes = (size_t)9 * nodes_of(res[0]) * (dt == LBM_F32DEV ? 4 : 2);
     gr.nres = (int)res.size();
-    if (gr.nres > 0) {
-      gr.res = (int *)dev_alloc(sizeof(int) * res.size());
-      b->resident = true;
+    for (int k : res) {
+      const int c = resident_pairs(nodes_of(k), e_size, sm_bytes, sm_reserved);
+      if (gr.res_count[c]++ == 0) gr.res_nodes[c] = nodes_of(k);
+      b->resident[c] = true;
     }
+    if (gr.nres > 0) gr.res = (int *)dev_alloc(sizeof(int) * res.size());
     if (const_slots(dt) > 0) {
       gr.pbase = slots_reserve(b->device, dt, gr.n);
       if (gr.pbase >= 0) {

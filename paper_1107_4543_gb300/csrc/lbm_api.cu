@@ -80,6 +80,19 @@ size_t resident_limit(int device) {
   return lim;
 }
 
+void resident_sm(size_t *sm_bytes, size_t *reserved) {
+  int d = 0, sm = 0, blk = 0;
+  if (cudaGetDevice(&d) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, d) != cudaSuccess ||
+      cudaDeviceGetAttribute(&blk, cudaDevAttrReservedSharedMemoryPerBlock, d) != cudaSuccess) {
+    cudaGetLastError();
+    sm = 228 * 1024;
+    blk = 1024;
+  }
+  *sm_bytes = (size_t)sm;
+  *reserved = (size_t)blk;
+}
+
 int sm_count() {
   int d = 0, n = 0;
   if (cudaGetDevice(&d) != cudaSuccess ||

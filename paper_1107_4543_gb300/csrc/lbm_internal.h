@@ -205,32 +205,50 @@ inline cudaError_t launch_step_batch(int dtype, const BatchList &bl, int parity,
 
 // Batch members small enough to stay in shared memory for all the steps of
 // a launch (k_batch_resident, resident.cuh): those of which two fit one
-// block's shared memory, 2 x 9 compact planes, so that two share an SM.
-// resident_limit: the device's shared memory per block, lowered by the
-// environment variable LBM_RESIDENT_BYTES (0 turns resident members off).
+// block's shared memory, 2 x 9 compact planes.  resident_limit: the device's
+// shared memory per block, lowered by the environment variable
+// LBM_RESIDENT_BYTES (0 turns resident members off).
 inline size_t resident_bytes(int nx, int ny, int esize) {
   return (size_t)2 * 9 * (size_t)nx * (size_t)ny * (size_t)esize;
 }
+// Shared memory of a block for members of up to `nodes` nodes: the planes,
+// then the collision constants; and whether an SM with sm_bytes of shared
+// memory, of which each block reserves `reserved`, holds two such blocks.  All
+// blocks of a launch are of one size, so the few members that fill more than
+// half an SM with their constants (FP32 3209 - 3228 nodes, 16 bits 6422 -
+// 6456) take a launch of their own: in one launch with the others they would
+// leave every one of those alone on its SM.
+constexpr size_t resident_table(int esize) {
+  return esize == 4 ? sizeof(HlPairs) : sizeof(float2) * ((PC_COUNT + 1) / 2 * 2);
+}
+inline size_t resident_smem(long long nodes, int esize) {
+  return ((size_t)9 * (size_t)nodes * (size_t)esize + 15) / 16 * 16 + resident_table(esize);
+}
+inline bool resident_pairs(long long nodes, int esize, size_t sm_bytes, size_t reserved) {
+  return 2 * (resident_smem(nodes, esize) + reserved) <= sm_bytes;
+}
+// the current device's sm_bytes and reserved
+void resident_sm(size_t *sm_bytes, size_t *reserved);
 size_t resident_limit(int device);
 cudaError_t launch_batch_resident_f32(const BatchEntry *ents, const int *idx, int nres,
-                                      int nents, size_t planes, int parity, long steps,
+                                      int nents, long long nodes, int parity, long steps,
                                       const int *limits, cudaStream_t st);
 cudaError_t launch_batch_resident_f16(const BatchEntry *ents, const int *idx, int nres,
-                                      int nents, size_t planes, int parity, long steps,
+                                      int nents, long long nodes, int parity, long steps,
                                       const int *limits, cudaStream_t st);
 cudaError_t launch_batch_resident_bf16(const BatchEntry *ents, const int *idx, int nres,
-                                      int nents, size_t planes, int parity, long steps,
+                                      int nents, long long nodes, int parity, long steps,
                                       const int *limits, cudaStream_t st);
 inline cudaError_t launch_batch_resident(int dtype, const BatchEntry *ents, const int *idx,
-                                         int nres, int nents, size_t planes, int parity,
+                                         int nres, int nents, long long nodes, int parity,
                                          long steps, const int *limits, cudaStream_t st) {
   switch (dtype) {
     case LBM_F32DEV:
-      return launch_batch_resident_f32(ents, idx, nres, nents, planes, parity, steps, limits, st);
+      return launch_batch_resident_f32(ents, idx, nres, nents, nodes, parity, steps, limits, st);
     case LBM_F16DEV:
-      return launch_batch_resident_f16(ents, idx, nres, nents, planes, parity, steps, limits, st);
+      return launch_batch_resident_f16(ents, idx, nres, nents, nodes, parity, steps, limits, st);
     case LBM_BF16DEV:
-      return launch_batch_resident_bf16(ents, idx, nres, nents, planes, parity, steps, limits,
+      return launch_batch_resident_bf16(ents, idx, nres, nents, nodes, parity, steps, limits,
                                         st);
     default: return cudaErrorInvalidValue;
   }

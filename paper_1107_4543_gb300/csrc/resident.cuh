@@ -208,14 +208,15 @@ k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ id
   }
 }
 
-// planes: bytes of the largest member's nine planes
+// nodes: those of the largest member of the launch
 template <typename T>
 cudaError_t launch_resident_t(const BatchEntry *ents, const int *idx, int nres, int nents,
-                              size_t planes, int parity, long steps, const int *limits,
+                              long long nodes, int parity, long steps, const int *limits,
                               cudaStream_t st) {
   if (nres < 1 || steps < 1) return cudaSuccess;
-  const size_t at = (planes + 15) / 16 * 16;
-  const size_t smem = at + sizeof(typename ResidentConst<T>::Table);
+  constexpr size_t table = resident_table((int)sizeof(T));
+  static_assert(table == sizeof(typename ResidentConst<T>::Table) && table % 16 == 0, "table bytes");
+  const size_t smem = resident_smem(nodes, (int)sizeof(T)), at = smem - table;
   cudaError_t e = cudaFuncSetAttribute(
       k_batch_resident<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e != cudaSuccess) return e;

@@ -21,9 +21,9 @@ cudaError_t upload_batch_consts_f32(const BatchEntry *ents, int n, int pbase, vo
 }
 
 cudaError_t launch_batch_resident_f32(const BatchEntry *ents, const int *idx, int nres,
-                                      int nents, size_t planes, int parity, long steps,
+                                      int nents, long long nodes, int parity, long steps,
                                       const int *limits, cudaStream_t st) {
-  return launch_resident_t<float>(ents, idx, nres, nents, planes, parity, steps, limits, st);
+  return launch_resident_t<float>(ents, idx, nres, nents, nodes, parity, steps, limits, st);
 }
 
 cudaError_t launch_rows_f32(const Lattice &L, const void *src, void *dst, cudaStream_t st,
