@@ -69,12 +69,12 @@ struct lbm_batch_ctx {
     long long nrows = 0;
     // entries held in shared memory for all the steps of a launch (small
     // lattices; k_batch_resident), which the block records leave out, largest
-    // first: [0] those alone on their SM, [1] those of which two share one
-    // (resident_pairs), and the nodes of each kind's largest
+    // first and so kind by kind (ResidentKind), and the nodes of each kind's
+    // largest
     int nres = 0;
     int *res = nullptr;
-    int res_count[2] = {0, 0};
-    long long res_nodes[2] = {0, 0};
+    int res_count[RES_KINDS] = {};
+    long long res_nodes[RES_KINDS] = {};
     // the group's slots in its type's constant table (-1: none) and the
     // device staging of their refresh (n x const_slot_bytes(dtype))
     int pbase = -1;
@@ -84,10 +84,10 @@ struct lbm_batch_ctx {
   std::vector<int> member_res;                  // member stepped as a resident entry
   bool spent = false;  // a ragged generation ran: members' parities differ
   std::vector<Group> groups;
-  bool resident[2] = {false, false};     // some group has resident entries of the kind
+  bool resident[RES_KINDS] = {};         // some group has resident entries of the kind
   // their launches, beside the batch stream and one another
-  cudaStream_t res_stream[2] = {nullptr, nullptr};
-  cudaEvent_t res_fork = nullptr, res_join[2] = {nullptr, nullptr};
+  cudaStream_t res_stream[RES_KINDS] = {};
+  cudaEvent_t res_fork = nullptr, res_join[RES_KINDS] = {};
   std::vector<int> offs;                 // member buffer index at creation
   std::vector<cudaStream_t> saved_streams;
   AuxView *views[2] = {nullptr, nullptr}; // drift views at batch parity 0 / 1
@@ -197,19 +197,24 @@ static int batch_upload_pairs(lbm_batch_ctx *b) {
 // null) on the side streams, forked from the batch stream; resident_join
 // makes the batch stream wait for them.
 static int resident_fork(lbm_batch_ctx *b, int parity, long steps, bool ragged) {
-  if (!(b->resident[0] || b->resident[1]) || steps < 1) return LBM_OK;
+  bool any = false;
+  for (bool r : b->resident) any |= r;
+  if (!any || steps < 1) return LBM_OK;
   if (!b->res_fork) CK(cudaEventCreateWithFlags(&b->res_fork, cudaEventDisableTiming));
   CK(cudaEventRecord(b->res_fork, b->stream));
-  for (int c = 0; c < 2; ++c) {
+  for (int c = 0; c < RES_KINDS; ++c) {
     if (!b->resident[c]) continue;
     if (!b->res_stream[c]) CK(cudaStreamCreateWithFlags(&b->res_stream[c], cudaStreamNonBlocking));
     if (!b->res_join[c]) CK(cudaEventCreateWithFlags(&b->res_join[c], cudaEventDisableTiming));
     CK(cudaStreamWaitEvent(b->res_stream[c], b->res_fork, 0));
-    for (auto &gr : b->groups)
+    for (auto &gr : b->groups) {
+      int off = 0;
+      for (int k = 0; k < c; ++k) off += gr.res_count[k];
       if (gr.res_count[c] > 0)
-        CK(launch_batch_resident(gr.dtype, gr.ents, gr.res + (c ? gr.res_count[0] : 0),
-                                 gr.res_count[c], gr.n, gr.res_nodes[c], parity, steps,
-                                 ragged ? gr.limits : nullptr, b->res_stream[c]));
+        CK(launch_batch_resident(gr.dtype, gr.ents, gr.res + off, gr.res_count[c], gr.n,
+                                 gr.res_nodes[c], parity, steps, ragged ? gr.limits : nullptr,
+                                 b->res_stream[c]));
+    }
     CK(cudaEventRecord(b->res_join[c], b->res_stream[c]));
   }
   return LBM_OK;
@@ -430,12 +435,15 @@ long long batch_nodes(const lbm_batch_ctx *b) { return b->nodes; }
 
 static void batch_free(lbm_batch_ctx *b) {
   batch_drop_graphs(b);
-  for (auto *st : {b->up, b->down, b->res_stream[0], b->res_stream[1]})
+  std::vector<cudaStream_t> streams = {b->up, b->down};
+  streams.insert(streams.end(), b->res_stream, b->res_stream + RES_KINDS);
+  for (auto *st : streams)
     if (st) {
       cudaStreamSynchronize(st);
       cudaStreamDestroy(st);
     }
-  for (auto *ev : {b->res_fork, b->res_join[0], b->res_join[1]})
+  if (b->res_fork) cudaEventDestroy(b->res_fork);
+  for (auto *ev : b->res_join)
     if (ev) cudaEventDestroy(ev);
   for (auto &r : b->ring)
     for (auto &e : r)
@@ -803,7 +811,7 @@ int lbm_batch_create(int n, const lbm_handle *members, lbm_batch *out) {
                      [&](int p, int q) { return nodes_of(p) > nodes_of(q); });
     gr.nres = (int)res.size();
     for (int k : res) {
-      const int c = resident_pairs(nodes_of(k), e_size, sm_bytes, sm_reserved);
+      const ResidentKind c = resident_kind(nodes_of(k), e_size, sm_bytes, sm_reserved);
       if (gr.res_count[c]++ == 0) gr.res_nodes[c] = nodes_of(k);
       b->resident[c] = true;
     }

@@ -227,6 +227,17 @@ inline size_t resident_smem(long long nodes, int esize) {
 inline bool resident_pairs(long long nodes, int esize, size_t sm_bytes, size_t reserved) {
   return 2 * (resident_smem(nodes, esize) + reserved) <= sm_bytes;
 }
+// FP32 members of up to kResidentScalar nodes step one node per thread
+// (k_resident_tiny); larger ones have two nodes for each of the pair form's
+// threads.
+constexpr int kResidentScalar = 384;
+// The launches of a batch's resident members, from the largest members to the
+// smallest: alone on their SM, two to an SM, tiny
+enum ResidentKind { RES_ALONE, RES_PAIRS, RES_TINY, RES_KINDS };
+inline ResidentKind resident_kind(long long nodes, int esize, size_t sm_bytes, size_t reserved) {
+  if (esize == 4 && nodes <= kResidentScalar) return RES_TINY;
+  return resident_pairs(nodes, esize, sm_bytes, reserved) ? RES_PAIRS : RES_ALONE;
+}
 // the current device's sm_bytes and reserved
 void resident_sm(size_t *sm_bytes, size_t *reserved);
 size_t resident_limit(int device);

@@ -128,6 +128,30 @@ __device__ __forceinline__ void slot_store(T *A, int ia, int ib, bool two, F2 f)
   }
 }
 
+// the member's nine planes into shared memory, and back after n steps
+template <typename T>
+__device__ __forceinline__ void resident_load(T *A, const T *__restrict__ src, const Geom &g, int N) {
+  for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
+    const int i = q / N, r = q - i * N, y = r / g.nx;
+    A[q] = src[(long long)i * g.plane + (long long)y * g.rstride + (r - y * g.nx)];
+  }
+}
+template <typename T>
+__device__ __forceinline__ void resident_store(const T *A, T *__restrict__ dst, const Geom &g, int N,
+                                               int n) {
+  const int nx = g.nx, ny = g.ny;
+  for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
+    const int i = q / N, r = q - i * N, y = r / nx, x = r - y * nx;
+    int at = q;
+    if (n & 1) {  // post-collision population i of x is in slot (opposite i, x + c_i)
+      const int xs = x + CXd(i), ys = y + CYd(i);
+      at = opposite(i) * N + (ys < 0 ? ny - 1 : (ys == ny ? 0 : ys)) * nx +
+           (xs < 0 ? nx - 1 : (xs == nx ? 0 : xs));
+    }
+    dst[(long long)i * g.plane + (long long)y * g.rstride + x] = A[at];
+  }
+}
+
 // idx[b]: the entry block b steps.  Each member takes min(steps, limits[e])
 // steps (limits may be null) from buffer parity ^ off and leaves its state
 // in the buffer that parity of steps selects, as the per-step launches do.
@@ -160,10 +184,7 @@ k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ id
     const float v = RC::value(E.dp, threadIdx.x);
     table.c[threadIdx.x] = make_float2(v, v);
   }
-  for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
-    const int i = q / N, r = q - i * N, y = r / nx;
-    A[q] = src[(long long)i * E.g.plane + (long long)y * E.g.rstride + (r - y * nx)];
-  }
+  resident_load(A, src, E.g, N);
   __syncthreads();
   const int half = (N + 1) >> 1;
   for (int t = 0; t < n; ++t) {
@@ -196,16 +217,52 @@ k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ id
     }
     __syncthreads();
   }
-  for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
-    const int i = q / N, r = q - i * N, y = r / nx, x = r - y * nx;
-    int at = q;
-    if (n & 1) {  // post-collision population i of x is in slot (opposite i, x + c_i)
-      const int xs = x + CXd(i), ys = y + CYd(i);
-      at = opposite(i) * N + (ys < 0 ? ny - 1 : (ys == ny ? 0 : ys)) * nx +
-           (xs < 0 ? nx - 1 : (xs == nx ? 0 : xs));
+  resident_store(A, dst, E.g, N, n);
+}
+
+// FP32 members of at most kResidentScalar nodes, the same pattern with one
+// node per thread: so few nodes leave lanes idle in pairs, and a step is one
+// chain of shared-memory reads, collision and barrier, which the scalar
+// collision, its constants in registers, makes shorter; blocks as small as
+// the members let several share an SM.  us per step, in pairs by
+// k_batch_resident / here, 100 members: 3^2 0.41 / 0.22, 10^2 0.41 / 0.24, 16^2
+// 0.41 / 0.30, 18^2 0.55 / 0.40; 600 members: 16^2 1.02 / 0.84, 18^2 1.67 /
+// 1.26.  (Two step buffers, one node per thread, 512 threads for every size:
+// 0.28, 0.29, 0.40, 0.53; 1.28, 1.81.)
+static __global__ void __launch_bounds__(kResidentScalar)
+k_resident_tiny(const BatchEntry *__restrict__ ents, const int *__restrict__ idx, int nents,
+                int parity, int steps, const int *__restrict__ limits) {
+  __shared__ float A[9 * kResidentScalar];
+  const int e = idx[blockIdx.x];
+  if (!bounds::ok(e >= 0 && e < nents, bounds::BATCH_REC)) return;  // block-uniform
+  const BatchEntry &E = ents[e];
+  const int nx = E.g.nx, ny = E.g.ny, N = nx * ny;
+  if (!bounds::ok(N <= (int)blockDim.x, bounds::BATCH_REC)) return;
+  int n = steps;
+  if (limits != nullptr && limits[e] < n) n = limits[e];
+  if (n <= 0) return;  // block-uniform
+  const int from = parity ^ E.off, r = threadIdx.x;
+  resident_load(A, static_cast<const float *>(E.buf[from]), E.g, N);
+  const Nbr nb = nbr(r % nx, r / nx, nx, ny);
+  for (int t = 0; t < n; ++t) {
+    __syncthreads();
+    float f[9];
+    if (r < N && !(t & 1)) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) f[i] = A[i * N + nb.at(i)];
+      collide_dev<true, false>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7], f[8], E.dp);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) A[i * N + nb.at(i)] = f[opposite(i)];
+    } else if (r < N) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) f[opposite(i)] = A[i * N + r];
+      collide_dev<true, false>(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7], f[8], E.dp);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) A[i * N + r] = f[i];
     }
-    dst[(long long)i * E.g.plane + (long long)y * E.g.rstride + x] = A[at];
   }
+  __syncthreads();
+  resident_store(A, static_cast<float *>(E.buf[from ^ (n & 1)]), E.g, N, n);
 }
 
 // nodes: those of the largest member of the launch
@@ -224,8 +281,16 @@ cudaError_t launch_resident_t(const BatchEntry *ents, const int *idx, int nres, 
   const long chunk = 1L << 30;
   for (long done = 0; done < steps; done += chunk) {
     const long k = steps - done < chunk ? steps - done : chunk;
-    k_batch_resident<T><<<(unsigned)nres, kResidentThreads, smem, st>>>(
-        ents, idx, nents, parity ^ (int)(done & 1), (int)k, limits, (int)at);
+    bool tiny = false;
+    if constexpr (sizeof(T) == 4) {
+      tiny = nodes <= kResidentScalar;
+      if (tiny)
+        k_resident_tiny<<<(unsigned)nres, (unsigned)(nodes + 31) / 32 * 32, 0, st>>>(
+            ents, idx, nents, parity ^ (int)(done & 1), (int)k, limits);
+    }
+    if (!tiny)
+      k_batch_resident<T><<<(unsigned)nres, kResidentThreads, smem, st>>>(
+          ents, idx, nents, parity ^ (int)(done & 1), (int)k, limits, (int)at);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

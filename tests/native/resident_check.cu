@@ -25,6 +25,9 @@ int main() {
       if (resident) last_resident = n;
       if (resident && pair) last_pair = n;
       if (pair && last_pair != n && resident) ++failures;  // monotonic
+      const ResidentKind kind = resident_kind(n, esize, sm, reserved);
+      if (kind != (esize == 4 && n <= kResidentScalar ? RES_TINY : (pair ? RES_PAIRS : RES_ALONE)))
+        ++failures;
     }
     printf("esize %d: pairs to %lld, resident to %lld\n", esize, last_pair, last_resident);
     if (esize == 4 && (last_pair != 3208 || last_resident != 3228)) ++failures;

@@ -15,9 +15,12 @@ RATES = inp.s_ll(inp.rates("OPT"))
 PAIRS = [("f32", 8, 401), ("f32", 20, 20), ("f16", 6, 1070), ("bf16", 33, 31)]
 ALONE = [("f32", 46, 70), ("f32", 12, 269), ("f16", 92, 70), ("bf16", 12, 538)]
 OTHER = [("f32", 70, 60)]
+# FP32 members stepped one node per thread (up to 384 nodes), and the next size
+TINY = [("f32", 2, 2), ("f32", 3, 3), ("f32", 2, 31), ("f32", 33, 2), ("f32", 11, 11),
+        ("f32", 8, 16), ("f32", 43, 3), ("f32", 24, 16), ("f32", 35, 11)]
 
 
-@pytest.mark.parametrize("members", [PAIRS + ALONE + OTHER, ALONE, PAIRS])
+@pytest.mark.parametrize("members", [PAIRS + ALONE + OTHER, ALONE, PAIRS, TINY])
 def test_both_kinds_of_resident_members_equal_alone(members):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
