@@ -128,27 +128,38 @@ __device__ __forceinline__ void slot_store(T *A, int ia, int ib, bool two, F2 f)
   }
 }
 
-// the member's nine planes into shared memory, and back after n steps
+// The member's nine planes into shared memory, and back after n steps: a
+// node's nine elements at a time, so that nine loads are in flight and share
+// one address computation.  us per call of one step, one element of one plane
+// at a time (with its divisions) / nine: four FP16 members of 80^2 107 / 28, of
+// 2 x 3000 131 / 85, FP32 of 55 x 56 64 / 22.
 template <typename T>
 __device__ __forceinline__ void resident_load(T *A, const T *__restrict__ src, const Geom &g, int N) {
-  for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
-    const int i = q / N, r = q - i * N, y = r / g.nx;
-    A[q] = src[(long long)i * g.plane + (long long)y * g.rstride + (r - y * g.nx)];
+  Walk w(threadIdx.x, blockDim.x, g.nx);
+  for (int r = threadIdx.x; r < N; r += blockDim.x, w.next()) {
+    const T *p = src + (long long)w.y * g.rstride + w.x;
+    T v[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) v[i] = p[(long long)i * g.plane];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) A[i * N + r] = v[i];
   }
 }
 template <typename T>
 __device__ __forceinline__ void resident_store(const T *A, T *__restrict__ dst, const Geom &g, int N,
                                                int n) {
-  const int nx = g.nx, ny = g.ny;
-  for (int q = threadIdx.x; q < 9 * N; q += blockDim.x) {
-    const int i = q / N, r = q - i * N, y = r / nx, x = r - y * nx;
-    int at = q;
+  Walk w(threadIdx.x, blockDim.x, g.nx);
+  for (int r = threadIdx.x; r < N; r += blockDim.x, w.next()) {
+    T *p = dst + (long long)w.y * g.rstride + w.x;
     if (n & 1) {  // post-collision population i of x is in slot (opposite i, x + c_i)
-      const int xs = x + CXd(i), ys = y + CYd(i);
-      at = opposite(i) * N + (ys < 0 ? ny - 1 : (ys == ny ? 0 : ys)) * nx +
-           (xs < 0 ? nx - 1 : (xs == nx ? 0 : xs));
+      const Nbr b = nbr(w.x, w.y, g.nx, g.ny);
+#pragma unroll
+      for (int i = 0; i < 9; ++i)
+        p[(long long)i * g.plane] = A[opposite(i) * N + b.at(opposite(i))];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) p[(long long)i * g.plane] = A[i * N + r];
     }
-    dst[(long long)i * g.plane + (long long)y * g.rstride + x] = A[at];
   }
 }
 
@@ -180,11 +191,16 @@ k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ id
   T *A = reinterpret_cast<T *>(smem_raw);
   using RC = ResidentConst<T>;
   typename RC::Table &table = *reinterpret_cast<typename RC::Table *>(smem_raw + consts_at);
+  resident_load(A, src, E.g, N);
   if (threadIdx.x < RC::COUNT) {
-    const float v = RC::value(E.dp, threadIdx.x);
+    float v = 0.0f;  // thread k's constant, all of them read at once
+#pragma unroll
+    for (int k = 0; k < RC::COUNT; ++k) {
+      const float c = RC::value(E.dp, k);
+      if (threadIdx.x == k) v = c;
+    }
     table.c[threadIdx.x] = make_float2(v, v);
   }
-  resident_load(A, src, E.g, N);
   __syncthreads();
   const int half = (N + 1) >> 1;
   for (int t = 0; t < n; ++t) {
