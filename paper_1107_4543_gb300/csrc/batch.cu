@@ -657,8 +657,8 @@ static std::vector<size_t> packed_groups(const lbm_batch_ctx *b) {
 
 // Block records of the kRowSteps-per-launch grid of a batch's members of
 // storage type dt that are not resident; none where the grid does not take
-// some member or is not estimated to save at least 5% of the single-step
-// launches (plan.h; 16-bit batches of narrow or few lattices, whose
+// some member or is not estimated to save enough of the single-step
+// launches (plan.h, rows_batch_margin; 16-bit batches of narrow or few lattices, whose
 // populations fit in L2, step as fast one by one).  Tasks of most rows
 // first, so that the short ones fill the tail of the launch.
 static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms) {
@@ -674,13 +674,16 @@ static std::vector<RowsRec> rows_records(const lbm_batch_ctx *b, int dt, int sms
     nodes += (double)L.g.nx * L.g.ny;
     for (int k = 0; k < kChoices; ++k) work[k].add(rows_geom(L.g, kBatchRowChoices[k]));
   }
-  double us = 0.95 * single_us(nodes, esize);
+  const double single = single_us(nodes, esize);
+  double us = single;
   int rows = 0;
-  for (int k = 0; k < kChoices; ++k)
-    if (nodes > 0 && rows_batch_us(work[k], esize, sms) < us) {
-      us = rows_batch_us(work[k], esize, sms);
+  for (int k = 0; k < kChoices; ++k) {
+    const double t = rows_batch_us(work[k], esize, sms);
+    if (nodes > 0 && t < us && t < rows_batch_margin(work[k], dt == LBM_F16DEV, sms) * single) {
+      us = t;
       rows = kBatchRowChoices[k];
     }
+  }
   if (rows == 0) return recs;
   for (size_t mi = 0; mi < b->members.size(); ++mi) {
     const Lattice &L = b->members[mi]->L;

@@ -63,6 +63,17 @@ inline double rows_batch_us(const RowsWork &w, int esize, int sms) {
   return std::max(rows_us(w, esize, sms), 1.15 * rows_us(w, esize, sms, 0.1));
 }
 
+// What rows must be estimated to save of a batch's single steps.  5%, but 8%
+// in FP16 with fewer than 1.5 tasks per slot: the estimate does not see the
+// tail of the second wave there, and FP16's single steps are the fastest ones.
+// Measured rows / single steps at estimates of 0.93 and 0.92: 12 lattices of
+// 300^2 .. 1000^2 (1.0 tasks per slot) 30.4 / 29.0, 64 of 82^2 .. 1024^2 (1.25)
+// 57.0 / 56.4 us; at 0.91, 2000^2 (0.86) 23.3 / 24.5, 0.93, 400 of 85^2 ..
+// 300^2 (1.8) 86.9 / 93.8.
+inline double rows_batch_margin(const RowsWork &w, bool f16, int sms) {
+  return f16 && w.tasks < 1.5 * sms * kRowsWarps ? 0.92 : 0.95;
+}
+
 // Estimated us of one single-step launch over `nodes` nodes: its latency and
 // the L2's rate while both buffers fit there, HBM's beyond.  Measured: FP32
 // 1024^2 8.4, 1500 x 1111 16.4, 2048^2 45; 16 bits 1500 x 1111 9.4, 1732^2
