@@ -252,7 +252,7 @@ static cudaError_t launch_some(lbm_ctx *h, int from, int steps, cudaStream_t st,
                                const float *forced = nullptr) {
   const void *src = h->L.buf[from];
   void *dst = h->L.buf[from ^ 1];
-  if (h->L.plan == PLAN_TILE)
+  if (h->L.plan == PLAN_TILE && (forced || steps >= h->L.tile_least))
     return launch_tile(h->L, src, dst, st, steps, forced, h->sx, h->sy);
   return steps > 1 ? launch_rows(h->L, src, dst, st, steps) : launch_one(h, from, st);
 }
@@ -275,7 +275,7 @@ static int capture_graph(lbm_ctx *h, cudaGraphExec_t *out, int *steps, bool forc
   if (e == cudaSuccess) {
     const int launches = graph_launches(h);
     for (int k = 0; k < launches && e == cudaSuccess; ++k) {
-      const int n = next_steps(h->L, 1 << 20);
+      const int n = next_steps(h->L, 1 << 20, forced);
       e = launch_some(h, k & 1, n, cs, forced ? h->src_tab32 + 9 * done : nullptr);
       done += n;
     }
@@ -793,7 +793,7 @@ static int step_forced_tile(lbm_ctx *h, long n) {
       h->src_gy = h->sy;
     }
     const bool replay = h->src_graph && h->L.cur == 0 && n >= h->src_steps;
-    const int k = replay ? h->src_steps : next_steps(h->L, n);
+    const int k = replay ? h->src_steps : next_steps(h->L, n, true);
     float tab[9 * kMax];
     for (int q = 0; q < k; ++q) {
       double fs[9];

@@ -70,6 +70,7 @@ struct Lattice {
   StepPlan plan = PLAN_SINGLE;
   RowsGeom rows = {};
   TileGeom tile = {};
+  int tile_least = 0;  // a rest of fewer steps is faster in single-step launches
   int dtype;
   int V;             // nodes per vector (vec_nodes)
   int variant;       // launch variant of the step kernel (tuner)

@@ -107,11 +107,17 @@ inline RowsGeom plan_rows(const Geom &g, int esize, int sms, double *us) {
   return best;
 }
 
+// Estimated us of one k_step_tile launch of T steps on tiles of `by` rows: 1.2
+// + 0.05 per tile row loaded + (0.33 + 0.04 per row) for each step, fitted to
+// FP32 101^2 (2 .. 8 steps) and 512^2 (2 .. 6 steps) within 10%.
+inline double tile_us(int by, int T) {
+  double us = 1.2 + 0.05 * (by + 2 * T);
+  for (int s = 1; s <= T; ++s) us += 0.33 + 0.04 * (by + 2 * (T - s));
+  return us;
+}
+
 // k_step_tile: the split of least estimated time per step with all tiles
-// resident at once (one block per SM).  The estimate, in us per launch, is
-// 1.2 + 0.05 per tile row loaded + (0.33 + 0.04 per row) for each step, fitted
-// to FP32 101^2 (2 .. 8 steps) and 512^2 (2 .. 6 steps) within 10%.
-// steps = 0: no split fits.
+// resident at once (one block per SM); steps = 0: no split fits.
 inline TileGeom plan_tile(const Geom &g, int esize, int sms, double *us_per_step) {
   TileGeom best = {0, 0, 0, 0, 0};
   *us_per_step = 1e30;
@@ -126,14 +132,24 @@ inline TileGeom plan_tile(const Geom &g, int esize, int sms, double *us_per_step
     const int nty = std::min(g.ny, sms / ntx);
     const int by = (g.ny + nty - 1) / nty;
     if (tile_bytes(by, T, esize) > (size_t)kMaxSmem) continue;
-    double us = 1.2 + 0.05 * (by + 2 * T);
-    for (int s = 1; s <= T; ++s) us += 0.33 + 0.04 * (by + 2 * (T - s));
+    const double us = tile_us(by, T);
     if (us / T < *us_per_step) {
       *us_per_step = us / T;
       best = {bx, by, ntx, (g.ny + by - 1) / by, T};
     }
   }
   return best;
+}
+
+// The least steps that k_step_tile takes: a launch of few steps still pays for
+// loading the halo of tall tiles.  Single steps outside a graph cost a little
+// more than estimated, so they have to be estimated 25% faster.  us per call of
+// 1, 2, 3 steps, tiles / single steps: 700^2 FP16 7.3 / 4.5, 9.9 / 9.0, 12.7 /
+// 13.5; one step of 5 x 3000 FP32 4.4 / 2.6, of 512^2 FP32 5.5 / 3.5.
+inline int tile_least(const TileGeom &t, double single) {
+  int n = 1;
+  while (n < t.steps && tile_us(t.by, n) > 1.25 * n * single) ++n;
+  return n;
 }
 
 // The estimated fastest of tiles, rows and single steps for the 32- and
@@ -143,11 +159,13 @@ inline TileGeom plan_tile(const Geom &g, int esize, int sms, double *us_per_step
 inline void plan_lattice(Lattice &L, int sms) {
   L.plan = PLAN_SINGLE;
   if (L.esize == 8) return;
-  double best = 0.95 * single_us((double)L.g.nx * L.g.ny, L.esize), us = 0;
+  const double single = single_us((double)L.g.nx * L.g.ny, L.esize);
+  double best = 0.95 * single, us = 0;
   const TileGeom t = plan_tile(L.g, L.esize, sms, &us);
   if (t.steps > 1 && us < best) {
     L.plan = PLAN_TILE;
     L.tile = t;
+    L.tile_least = tile_least(t, single);
     best = us;
   }
   const RowsGeom r = plan_rows(L.g, L.esize, sms, &us);
@@ -158,9 +176,12 @@ inline void plan_lattice(Lattice &L, int sms) {
 }
 
 // Steps of the next launch of n remaining steps: as many as the plan takes,
-// without leaving a single step behind k_step_rows (4 = 2 + 2).
-inline int next_steps(const Lattice &L, long n) {
-  if (L.plan == PLAN_TILE) return (int)std::min<long>(n, L.tile.steps);
+// without leaving a single step behind k_step_rows (4 = 2 + 2); 1 is a
+// single-step launch where the plan's kernel takes no fewer than 2 (rows) or
+// tile_least.  Forced steps take tiles down to one step.
+inline int next_steps(const Lattice &L, long n, bool forced = false) {
+  if (L.plan == PLAN_TILE)
+    return n < L.tile_least && !forced ? 1 : (int)std::min<long>(n, L.tile.steps);
   if (L.plan == PLAN_ROWS) return n == 1 ? 1 : (n == 2 || n == 4 ? 2 : kRowSteps);
   return 1;
 }
