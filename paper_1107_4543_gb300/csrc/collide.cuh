@@ -38,6 +38,13 @@ __device__ __forceinline__ float mul_hl(float a, float h, float l) {
   return PRECISE ? fmaf(a, h, a * l) : a * h;
 }
 
+// 1 / d by the hardware reciprocal
+__device__ __forceinline__ float rcp_approx(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return r;
+}
+
 // Deviation form: f' = f - f^eq(rho0, j0); the base carries the moments
 // m^eq(rho0, j0), so rho = rho0 + rho', j = j0 + j' and the non-equilibrium
 // parts are n = m' - [m^eq(rho, j) - m^eq(rho0, j0)].  Written so that FP32
@@ -82,7 +89,7 @@ __device__ __forceinline__ void collide_dev(float &f0, float &f1, float &f2, flo
   // O(amplitude^2) quadratic terms below, and unlike an IEEE division it has
   // no slow path for non-finite operands, so a lattice that has gone
   // unstable costs no more per node than a healthy one
-  const float c = __fdividef(rho_phys, P.rho0 + rho_phys);
+  const float c = rho_phys * rcp_approx(P.rho0 + rho_phys);
   const float jxx = SCALED ? (jx_p * jx_p) * P.inv_scale : jx_p * jx_p;
   const float jyy = SCALED ? (jy_p * jy_p) * P.inv_scale : jy_p * jy_p;
   const float jxy = SCALED ? (jx_p * jy_p) * P.inv_scale : jx_p * jy_p;
@@ -100,7 +107,7 @@ __device__ __forceinline__ void collide_dev(float &f0, float &f1, float &f2, flo
   const float dpxy = fmaf(-nx, c, nx);  // jx jy / rho - jx0 jy0 / rho0
 
   // non-equilibrium parts, each straight from partial sums
-  const float n3 = fmaf(4.0f, diag, axis - 2.0f * f0) - 3.0f * djsq;  // e' + 2 rho' - 3 dJ
+  const float n3 = fmaf(-3.0f, djsq, fmaf(4.0f, diag, fmaf(-2.0f, f0, axis)));  // e' + 2 rho' - 3 dJ
   const float n4 = fmaf(3.0f, djsq, 3.0f * (f0 - axis));             // eps' - rho' + 3 dJ
   const float n5 = fmaf(2.0f, dxd, -d13);                            // qx' + jx'
   const float n6 = fmaf(2.0f, dyd, -d24);                            // qy' + jy'
@@ -166,13 +173,6 @@ __device__ __forceinline__ F2 operator*(F2 a, F2 b) {
 __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
   F2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
-
-// 1 / d by the hardware reciprocal
-__device__ __forceinline__ float rcp_approx(float d) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return r;
 }
 
@@ -370,10 +370,9 @@ inline HlPairs hl_pairs(const DevParams &P) {
 __device__ __forceinline__ F2 mul_hl2(F2 a, const F2x2 &k) { return fma2(a, k.a, a * k.b); }
 
 // collide_dev<true, false> (FP32 storage) for two nodes, one per lane: the
-// same operations in the same order, so each lane's result equals the scalar
-// form's bit for bit (its one product that the compiler contracts, the
-// -3 dJ of n3, is an explicit multiply-add here; products by powers of two
-// are exact either way).
+// same operations in the same order, multiply-adds written out in both, so
+// each lane's result equals the scalar form's bit for bit however the compiler
+// contracts the rest (products by powers of two, exact either way).
 template <typename K>
 __device__ __forceinline__ void collide_pair_hl(F2 &f0, F2 &f1, F2 &f2_, F2 &f3, F2 &f4, F2 &f5,
                                                 F2 &f6, F2 &f7, F2 &f8, const K &P) {
