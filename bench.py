@@ -12,10 +12,12 @@ reduction).
   e2e        MLUPS through the C ABI with host buffers: every step uploads
              the initial fields (rho, ux, uy) from pinned host memory
              (packed batch I/O), steps, and downloads rho, ux, uy
-  roofline   the batched step kernel: algorithmic 72 B per node and launch
-             (one read and one write of the populations for its three time
-             steps) over its average launch time against the measured HBM
-             copy bandwidth; its FP32 arithmetic is the nearer bound
+  roofline   the batched step kernel that the library's plan names
+             (lbm_batch_plan): algorithmic 72 B per node and launch (one read
+             and one write of the populations for its time steps) over its
+             average launch time against the measured HBM copy bandwidth,
+             and its FP32 operations against the FP32 units, which are the
+             nearer bound of launches of several steps
   fp64_plain the plain FP64 path on one 8192^2 lattice, for comparison
   cpu_baseline  the FP64 CPU oracle on a bounded sample of the workload
 
@@ -47,14 +49,45 @@ sys.path.insert(0, ROOT)
 import lbm_inputs as inp  # noqa: E402
 
 BYTES_PER_LU = {"f64": 144, "f64dev": 144, "f32": 72, "f16": 36, "bf16": 36}
-# time steps per launch on large lattices and batches of the 32- and 16-bit
-# types (kRowSteps in csrc/lbm_internal.h); the FP64 types take one
-STEPS_PER_LAUNCH = 3
+C_TYPES = {"f64": "double", "f64dev": "double", "f32": "float", "f16": "__half",
+           "bf16": "__nv_bfloat16"}
+# lane operations of one lattice update's collision (an add, multiply or
+# multiply-add each), and operations per clock and SM of the unit that runs
+# them on GB300 (152 SMs)
+OPS_PER_LU = {"f64": 119, "f64dev": 71, "f32": 97, "f16": 89, "bf16": 89}
+OPS_PER_CLOCK = {"f64": 2, "f64dev": 2, "f32": 128, "f16": 128, "bf16": 128}
 
 
-def hbm_bytes_per_update(dtype):
+def hbm_bytes_per_update(dtype, steps_per_launch):
     """HBM bytes of one lattice update: the populations cross once each way per launch."""
-    return BYTES_PER_LU[dtype] / (1 if dtype.startswith("f64") else STEPS_PER_LAUNCH)
+    return BYTES_PER_LU[dtype] / steps_per_launch
+
+
+def step_kernel(L, dtype, plan, batched=False):
+    """Name of the kernel that a plan (lbm_step_plan, lbm_batch_plan) launches."""
+    if dtype == "f64":
+        return "k_step_f64"
+    name = {L.LBM_PLAN_SINGLE: "k_step_batch" if batched else "k_step_dev",
+            L.LBM_PLAN_ROWS: "k_rows_batch" if batched else "k_step_rows",
+            L.LBM_PLAN_TILES: "k_step_tile"}[plan]
+    return "%s<%s>" % (name, C_TYPES[dtype])
+
+
+def resident_launches(specs, resident, dtype):
+    """Launches that a stepping call makes for its resident members: one for
+    each kind (ResidentKind in csrc/lbm_internal.h) among them, by their nodes on
+    GB300's 228 KB of shared memory per SM."""
+    tiny, pairs = (384, 3208) if dtype == "f32" else (0, 6421)
+    nodes = [s["nx"] * s["ny"] for s, r in zip(specs, resident) if r]
+    return len({0 if n <= tiny else 1 if n <= pairs else 2 for n in nodes})
+
+
+def alu_record(torch, dtype, mlups, mhz):
+    """The collision's operations against the vector units at a clock."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    peak = OPS_PER_CLOCK[dtype] * sms * mhz * 1e6
+    return {"ops_per_update": OPS_PER_LU[dtype], "sm_mhz": mhz,
+            "frac": round(OPS_PER_LU[dtype] * mlups * 1e6 / peak, 4)}
 
 
 KERNEL_SOURCES = ["csrc/step_impl.cuh", "csrc/d2q9_pull.cuh", "csrc/collide.cuh",
@@ -424,13 +457,18 @@ def bench_batched(args, L, torch, rank, ws):
     lu_per_step = nodes * lbm_steps
     lu_job = reduce_sum(lu_per_step * args.steps)  # every rank's lattice updates
     value = job_mlups(lu_job, total_ms * 1e-3)
-    # batched launches of STEPS_PER_LAUNCH time steps, single ones for the
-    # remainder
-    step_launches = lbm_steps // STEPS_PER_LAUNCH + lbm_steps % STEPS_PER_LAUNCH
-    launch_ms = float(np.mean(step_ms)) / (lbm_steps / STEPS_PER_LAUNCH)
-    # those, the resident launch, the constant-table refresh and one drift
+    # how the members outside shared memory step: launches of several steps and
+    # single ones for the remainder, or single steps (none: all are resident)
+    if resident.all():
+        plan, per, step_launches = None, lbm_steps, 0
+    else:
+        plan, per = L.lbm_batch_plan(b, L.DTYPES[bdt])
+        step_launches = lbm_steps // per + lbm_steps % per
+    launch_ms = float(np.mean(step_ms)) / (lbm_steps / per)
+    # those, the resident launches, the constant-table refresh and one drift
     # launch pair
-    launches = args.steps * (step_launches + 2 + int(resident.any()) + table_fills)
+    launches = args.steps * (step_launches + 2 + resident_launches(specs, resident, bdt)
+                             + table_fills)
 
     # e2e: host fields in, moments out, through the public API: one
     # lbm_batch_solve_packed call per benchmark step (upload of the fields
@@ -487,16 +525,23 @@ def bench_batched(args, L, torch, rank, ws):
         L.lbm_destroy(h)
 
     peak, peak_kind = peaks()
-    kname = {"f32": "float", "f16": "__half", "bf16": "__nv_bfloat16"}[bdt]
     sname = {"f32": "FP32", "f16": "FP16", "bf16": "BF16"}[bdt]
     achieved = BYTES_PER_LU[bdt] * step_nodes / (launch_ms * 1e-3) / 1e9
-    tr = traffic_record("k_rows_batch<%s>" % kname)
-    roofline = {"bound": "fma", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-                "frac": round(achieved / peak, 4),
-                # ncu DRAM bytes per lattice update of a smaller capture of the
-                # same kernel, scaled to this launch's lattice updates
+    kernel = ("k_batch_resident<%s>" % C_TYPES[bdt] if plan is None
+              else step_kernel(L, bdt, plan, batched=True))
+    tr = traffic_record(kernel)
+    # achieved, peak and frac: the populations' bytes, once each way per
+    # launch, against the measured HBM copy rate; fma: the collision's
+    # operations against the FP32 units at the clock seen under load
+    roofline = {"bound": "hbm" if per == 1 else "fma", "achieved": round(achieved, 1),
+                "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
+                "frac_of": "measured HBM copy rate",
+                "fma": alu_record(torch, bdt, step_nodes * lbm_steps / np.mean(step_ms) / 1e3,
+                                  clk["sm_mhz"] or clk["sm_max_mhz"] or 2070.0),
+                # ncu DRAM bytes per node and launch of a smaller capture of the
+                # same kernel, scaled to this launch's nodes
                 "traffic": (round(tr["dram_bytes_per_lu"] * step_nodes) if tr else None),
-                "kernel": "k_rows_batch<%s>" % kname, "steps_per_launch": STEPS_PER_LAUNCH,
+                "kernel": kernel, "steps_per_launch": per,
                 "peak_source": peak_kind,
                 "algorithmic_bytes_per_launch": BYTES_PER_LU[bdt] * step_nodes,
                 "avg_launch_ms": round(launch_ms, 4),
@@ -550,7 +595,7 @@ def large_one(L, torch, stream, n, dtype, lbm_steps, reps, warmup):
     """One n x n lattice (optimized rates, device-side Gaussian pulse A = 1e-3,
     b = 20) in one storage type: `reps` timed runs of lbm_steps steps after
     `warmup` untimed ones (CUDA events on the launching stream).  Returns
-    (MLUPS, ms per time step)."""
+    (MLUPS, ms per time step, lbm_step_plan)."""
     r = inp.rates("OPT")
     h = L.lbm_create(n, n, inp.s_ll(r), 1.0, (0.0, 0.0), L.DTYPES[dtype])
     try:
@@ -567,9 +612,23 @@ def large_one(L, torch, stream, n, dtype, lbm_steps, reps, warmup):
         e1.record()
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1)
+        plan = L.lbm_step_plan(h)
     finally:
         L.lbm_destroy(h)
-    return n * n * lbm_steps * reps / (ms * 1e-3) / 1e6, ms / (lbm_steps * reps)
+    return n * n * lbm_steps * reps / (ms * 1e-3) / 1e6, ms / (lbm_steps * reps), plan
+
+
+def roofline_one(L, torch, dtype, plan, per, mlups, achieved, peak, peak_kind):
+    """Roofline of one lattice's step kernel: the populations' bytes, once each
+    way per launch, against the measured HBM copy rate (achieved, peak, frac),
+    and the collision's operations against its vector unit at the maximum
+    clock."""
+    return {"bound": ("fp64-alu" if dtype.startswith("f64") else
+                      "hbm" if plan == L.LBM_PLAN_SINGLE else "fma"),
+            "kernel": step_kernel(L, dtype, plan), "steps_per_launch": per,
+            "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
+            "frac": round(achieved / peak, 4), "frac_of": "measured HBM copy rate",
+            "alu": alu_record(torch, dtype, mlups, 2070.0), "peak_source": peak_kind}
 
 
 def bench_large(args, L, torch, rank, ws):
@@ -580,17 +639,15 @@ def bench_large(args, L, torch, rank, ws):
     peak, peak_kind = peaks()
     for dtype in args.dtypes.split(","):
         lbm_steps = 50 if not dtype.startswith("f64") else 10
-        mlups, step_ms = large_one(L, torch, stream, n, dtype, lbm_steps, args.steps,
-                                   args.warmup)
-        achieved = hbm_bytes_per_update(dtype) * n * n / (step_ms * 1e-3) / 1e9
+        mlups, step_ms, (plan, per) = large_one(L, torch, stream, n, dtype, lbm_steps, args.steps,
+                                                args.warmup)
+        achieved = hbm_bytes_per_update(dtype, per) * n * n / (step_ms * 1e-3) / 1e9
         lines.append({"metric": "MLUPS, single %dx%d lattice" % (n, n), "value": round(mlups, 1),
                       "unit": "MLUPS", "dtype": dtype, "n_gpus": ws, "steps": args.steps,
                       "warmup": args.warmup, "higher_is_better": True,
                       "config": {"workload": "single-%dx%d-%s" % (n, n, dtype)},
-                      "roofline": {"bound": "fp64-alu" if dtype.startswith("f64") else "fma",
-                                   "achieved": round(achieved, 1), "peak": peak,
-                                   "unit": "GB/s", "frac": round(achieved / peak, 4),
-                                   "peak_source": peak_kind}})
+                      "roofline": roofline_one(L, torch, dtype, plan, per, mlups, achieved,
+                                               peak, peak_kind)})
     return lines
 
 
@@ -606,17 +663,12 @@ def config3_record(L, torch):
     n, steps = 8192, 1000
     out = {"workload": "single-8192x8192-1000-steps", "note": "one timed run of 1000 steps "
            "after 2 x 50 warm-up steps; 2.4-9.7 GB of populations per type (> L2)"}
-    kern = {"f32": "k_step_rows<float>", "f16": "k_step_rows<__half>",
-            "bf16": "k_step_rows<__nv_bfloat16>", "f64": "k_step_f64",
-            "f64dev": "k_step_dev<double>"}
     for dtype in ("f32", "f16", "bf16", "f64", "f64dev"):
-        mlups, ms = large_one(L, torch, stream, n, dtype, steps, 1, 2)
-        achieved = hbm_bytes_per_update(dtype) * n * n / (ms * 1e-3) / 1e9
+        mlups, ms, (plan, per) = large_one(L, torch, stream, n, dtype, steps, 1, 2)
+        achieved = hbm_bytes_per_update(dtype, per) * n * n / (ms * 1e-3) / 1e9
         out[dtype] = {"mlups": round(mlups, 1), "ms_per_lbm_step": round(ms, 4),
-                      "roofline": {"bound": "fma" if not dtype.startswith("f64") else "fp64-alu",
-                                   "kernel": kern[dtype], "achieved": round(achieved, 1),
-                                   "peak": peak, "unit": "GB/s",
-                                   "frac": round(achieved / peak, 4), "peak_source": peak_kind}}
+                      "roofline": roofline_one(L, torch, dtype, plan, per, mlups, achieved, peak,
+                                               peak_kind)}
     return out
 
 
@@ -692,7 +744,7 @@ def bench_slabs(args, L, torch):
     fields = inp.gaussian_pulse(n, n, 1e-3, 20.0)
     stream = torch.cuda.current_stream()
     out = {}
-    mlups, _ = large_one(L, torch, stream, n, "f32", steps, 1, 1)
+    mlups, _, _ = large_one(L, torch, stream, n, "f32", steps, 1, 1)
     out["unsplit"] = round(mlups, 1)
     for k in (1, 2, 4):
         s = L.lbm_slabs_create(n, n, inp.s_ll(r), 1.0, (0.0, 0.0), L.LBM_F32DEV, k)

@@ -158,6 +158,17 @@ int lbm_tune(lbm_handle h, double *times_ms, int *chosen);
 int lbm_set_variant(lbm_handle h, int variant);
 int lbm_get_variant(lbm_handle h, int *variant);
 
+/* lbm_step_plan -- (runtime; no counterpart in the paper) how long calls of
+ * lbm_step launch this lattice's steps, chosen from its size and storage type
+ * when it is made: *kind LBM_PLAN_SINGLE (one step per launch), LBM_PLAN_ROWS
+ * or LBM_PLAN_TILES (*steps steps per launch; fewer for a remainder).  Results
+ * are bit-identical either way.  A point source takes LBM_PLAN_ROWS lattices
+ * one step per launch.  steps may be NULL. */
+#define LBM_PLAN_SINGLE 0
+#define LBM_PLAN_ROWS 1
+#define LBM_PLAN_TILES 2
+int lbm_step_plan(lbm_handle h, int *kind, int *steps);
+
 /* lbm_moments -- rho, ux, uy (host, ny x nx) at the current time: the
  * moments of the pre-collision populations, u = j / rho.  Synchronizes. */
 int lbm_moments(lbm_handle h, double *rho, double *ux, double *uy);
@@ -468,6 +479,10 @@ int lbm_batch_get_variant(lbm_batch b, int *variant);
  * the member's populations in HBM once; results are bit-identical either
  * way. */
 int lbm_batch_resident(lbm_batch b, int *flags);
+/* lbm_batch_plan -- as lbm_step_plan for the batch's members of storage type
+ * `dtype` that are not resident (lbm_batch_resident): LBM_PLAN_SINGLE or
+ * LBM_PLAN_ROWS.  LBM_EINVAL when the batch has none. */
+int lbm_batch_plan(lbm_batch b, int dtype, int *kind, int *steps);
 /* (runtime; no counterpart in the paper) Which members' collision constants
  * the per-step launches read from a constant-memory table (flags: one int
  * per member, 1 for such a member).  Each storage type of a batch reserves

@@ -1344,6 +1344,18 @@ int lbm_batch_const_table(lbm_batch b, int *flags) {
   return LBM_OK;
 }
 
+int lbm_batch_plan(lbm_batch b, int dtype, int *kind, int *steps) {
+  REQUIRE(b != nullptr && kind != nullptr, "null argument");
+  for (auto &gr : b->groups) {
+    if (gr.dtype != dtype || gr.nblocks == 0) continue;
+    *kind = gr.nrows > 0 ? LBM_PLAN_ROWS : LBM_PLAN_SINGLE;
+    if (steps) *steps = gr.nrows > 0 ? kRowSteps : 1;
+    return LBM_OK;
+  }
+  set_error("no members of that storage type outside shared memory");
+  return LBM_EINVAL;
+}
+
 int lbm_batch_get_variant(lbm_batch b, int *variant) {
   REQUIRE(b != nullptr && variant != nullptr, "null argument");
   *variant = b->tuned ? b->variant : -1;

@@ -991,6 +991,14 @@ int lbm_set_source(lbm_handle h, int x, int y, double amplitude, double period) 
   return LBM_OK;
 }
 
+int lbm_step_plan(lbm_handle h, int *kind, int *steps) {
+  REQUIRE(h != nullptr && kind != nullptr, "null argument");
+  const StepPlan p = h->src_on && h->L.plan == PLAN_ROWS ? PLAN_SINGLE : h->L.plan;
+  *kind = p == PLAN_TILE ? LBM_PLAN_TILES : (p == PLAN_ROWS ? LBM_PLAN_ROWS : LBM_PLAN_SINGLE);
+  if (steps) *steps = p == PLAN_TILE ? h->L.tile.steps : (p == PLAN_ROWS ? kRowSteps : 1);
+  return LBM_OK;
+}
+
 int lbm_set_variant(lbm_handle h, int variant) {
   REQUIRE(h != nullptr, "null handle");
   REQUIRE(variant >= 0 && variant < kStepVariants, "no such launch variant");

@@ -77,6 +77,10 @@ _SIGS = {
     "lbm_set_variant": (ctypes.c_int, [_vp, ctypes.c_int]),
     "lbm_batch_set_variant": (ctypes.c_int, [_vp, ctypes.c_int]),
     "lbm_batch_get_variant": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int)]),
+    "lbm_step_plan": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int),
+                                     ctypes.POINTER(ctypes.c_int)]),
+    "lbm_batch_plan": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
+                                      ctypes.POINTER(ctypes.c_int)]),
     "lbm_batch_resident": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int)]),
     "lbm_batch_const_table": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int)]),
     "lbm_get_variant": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int)]),
@@ -295,6 +299,7 @@ def lbm_tune(h):
 
 
 LBM_BATCH_TUNE_VARIANTS = 6
+LBM_PLAN_SINGLE, LBM_PLAN_ROWS, LBM_PLAN_TILES = 0, 1, 2
 
 
 def lbm_set_variant(h, variant):
@@ -315,6 +320,22 @@ def lbm_batch_get_variant(b):
     v = ctypes.c_int()
     _ck(load().lbm_batch_get_variant(b, ctypes.byref(v)), "lbm_batch_get_variant")
     return v.value
+
+
+def lbm_step_plan(h):
+    """(kind, steps): how long calls of lbm_step launch this lattice's steps,
+    kind one of LBM_PLAN_*, steps time steps per launch."""
+    k, n = ctypes.c_int(), ctypes.c_int()
+    _ck(load().lbm_step_plan(h, ctypes.byref(k), ctypes.byref(n)), "lbm_step_plan")
+    return k.value, n.value
+
+
+def lbm_batch_plan(b, dtype):
+    """lbm_step_plan of a batch's members of one storage type that are not
+    resident."""
+    k, n = ctypes.c_int(), ctypes.c_int()
+    _ck(load().lbm_batch_plan(b, int(dtype), ctypes.byref(k), ctypes.byref(n)), "lbm_batch_plan")
+    return k.value, n.value
 
 
 def lbm_batch_resident(b):
