@@ -282,8 +282,9 @@ const char *lbm_last_error(void);
  * (compiled with -DLBM_DEBUG_BOUNDS: paper_1107_4543_gb300/build.py
  * build(debug=True) makes _build_debug/liblbm.so).  The von Neumann QR, the
  * optimizer's polynomial-matrix slots and tables, the batched step's block
- * records and lane positions and the batched init / moments blocks check
- * their indices; a failed check sets a bit of a device word and the access
+ * records and lane positions, the rows, tiles and resident members of the
+ * kernels with several steps per launch and the batched init / moments blocks
+ * check their indices; a failed check sets a bit of a device word and the access
  * goes to the array's first element instead (no trap, the context stays
  * usable).  lbm_debug_bounds ORs the words of every translation unit of the
  * current device into *word (bits: see csrc/bounds.cuh) and, if reset,

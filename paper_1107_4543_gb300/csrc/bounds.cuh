@@ -11,8 +11,9 @@
 // deflation bounds (vn.cu), the optimizer's polynomial-matrix slots, power
 // blocks, point-table and K_l-table offsets (optcost.cu), the batched
 // step's block records and lane positions (step_impl.cuh), the resident
-// batch members' entries (resident.cuh), and the batched init / moments
-// blocks (io_dev.cu).
+// batch members' entries, planes and nodes (resident.cuh), the chunks, rows and
+// tiles of the kernels with several steps per launch (step_multi.cuh), and the
+// batched init / moments blocks (io_dev.cu).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -30,6 +31,9 @@ enum Site : unsigned {
   BATCH_REC = 1u << 7,    // batched step: block record's lattice
   BATCH_LANE = 1u << 8,   // batched step: lane row / chunk inside the lattice
   IO_BLOCK = 1u << 9,     // batched init / moments block
+  ROWS_NODE = 1u << 10,   // k_step_rows, k_rows_batch: chunk and row
+  TILE_NODE = 1u << 11,   // k_step_tile: tile size, column and row
+  RES_NODE = 1u << 12,    // resident members: planes in shared memory, node
   SELFTEST = 1u << 31,    // lbm_debug_bounds_selftest
 };
 

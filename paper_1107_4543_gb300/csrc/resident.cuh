@@ -137,7 +137,7 @@ template <typename T>
 __device__ __forceinline__ void resident_load(T *A, const T *__restrict__ src, const Geom &g, int N) {
   Walk w(threadIdx.x, blockDim.x, g.nx);
   for (int r = threadIdx.x; r < N; r += blockDim.x, w.next()) {
-    const T *p = src + (long long)w.y * g.rstride + w.x;
+    const T *p = src + (long long)bounds::ck(w.y, g.ny, bounds::RES_NODE) * g.rstride + w.x;
     T v[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) v[i] = p[(long long)i * g.plane];
@@ -150,7 +150,7 @@ __device__ __forceinline__ void resident_store(const T *A, T *__restrict__ dst, 
                                                int n) {
   Walk w(threadIdx.x, blockDim.x, g.nx);
   for (int r = threadIdx.x; r < N; r += blockDim.x, w.next()) {
-    T *p = dst + (long long)w.y * g.rstride + w.x;
+    T *p = dst + (long long)bounds::ck(w.y, g.ny, bounds::RES_NODE) * g.rstride + w.x;
     if (n & 1) {  // post-collision population i of x is in slot (opposite i, x + c_i)
       const Nbr b = nbr(w.x, w.y, g.nx, g.ny);
 #pragma unroll
@@ -182,6 +182,7 @@ k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ id
   if (!bounds::ok(e >= 0 && e < nents, bounds::BATCH_REC)) return;  // block-uniform
   const BatchEntry &E = ents[e];
   const int nx = E.g.nx, ny = E.g.ny, N = nx * ny;
+  if (!bounds::ok(9 * N * (int)sizeof(T) <= consts_at, bounds::RES_NODE)) return;  // block-uniform
   int n = steps;
   if (limits != nullptr && limits[e] < n) n = limits[e];
   if (n <= 0) return;  // block-uniform
@@ -209,8 +210,8 @@ k_batch_resident(const BatchEntry *__restrict__ ents, const int *__restrict__ id
       for (int p = threadIdx.x; p < half; p += blockDim.x, wa.next(), wb.next()) {
         // an odd lattice's last pair is one node (taken twice, stored once)
         const bool two = p + half < N;
-        const Nbr a = nbr(wa.x, wa.y, nx, ny);
-        const Nbr b = two ? nbr(wb.x, wb.y, nx, ny) : a;
+        const Nbr a = nbr(wa.x, bounds::ck(wa.y, ny, bounds::RES_NODE), nx, ny);
+        const Nbr b = two ? nbr(wb.x, bounds::ck(wb.y, ny, bounds::RES_NODE), nx, ny) : a;
         F2 f[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i] = slot_load(A, i * N + a.at(i), i * N + b.at(i));
@@ -253,7 +254,7 @@ k_resident_tiny(const BatchEntry *__restrict__ ents, const int *__restrict__ idx
   if (!bounds::ok(e >= 0 && e < nents, bounds::BATCH_REC)) return;  // block-uniform
   const BatchEntry &E = ents[e];
   const int nx = E.g.nx, ny = E.g.ny, N = nx * ny;
-  if (!bounds::ok(N <= (int)blockDim.x, bounds::BATCH_REC)) return;
+  if (!bounds::ok(N <= (int)blockDim.x, bounds::RES_NODE)) return;
   int n = steps;
   if (limits != nullptr && limits[e] < n) n = limits[e];
   if (n <= 0) return;  // block-uniform

@@ -217,7 +217,8 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
   if (!in) seg = 0;
   const bool out = in && lane >= H && lane < 32 - H && vc >= 0 && vc < nchunks;
   const int y0 = (int)seg * rg.rows, y1 = min(y0 + rg.rows, g.ny);
-  const int c = vc < 0 ? vc + nchunks : (vc >= nchunks ? vc - nchunks : vc);
+  const int c = bounds::ck(vc < 0 ? vc + nchunks : (vc >= nchunks ? vc - nchunks : vc), nchunks,
+                           bounds::ROWS_NODE);
   const int x0 = c * V;
   Seam<W> S;
   S.el = (g.nx - 1) & (V - 1);
@@ -232,7 +233,7 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
   auto row_of = [&](int y) -> const T * {
     while (y < 0) y += g.ny;
     while (y >= g.ny) y -= g.ny;
-    return src + (long long)y * g.rstride;
+    return src + (long long)bounds::ck(y, g.ny, bounds::ROWS_NODE) * g.rstride;
   };
   Vec *raw = sm + lane, *dly = sm + 9 * 32 + lane;
   const T *pm = row_of(ya - 1) + x0, *pc = row_of(ya) + x0, *pp = row_of(ya + 1) + x0;
@@ -286,7 +287,9 @@ __device__ __forceinline__ void rows_task(const T *__restrict__ src, T *__restri
       collide_chunk<T, W>(w, par);
     }
     if (j >= 2 * (STEPS - 1)) {
-      if (out && y0 + j - 2 * (STEPS - 1) < y1) {
+      if (out && y0 + j - 2 * (STEPS - 1) < y1 &&
+          bounds::ok(y0 >= 0 && y1 <= g.ny && x0 + (1 + fill) * V <= g.pitch,
+                     bounds::ROWS_NODE)) {
 #pragma unroll
         for (int i = 0; i < 9; ++i)
           *reinterpret_cast<Vec *>(drow + (long long)i * g.plane) = get_words(w[i]);
@@ -486,19 +489,23 @@ k_step_tile(const T *__restrict__ src, T *__restrict__ dst, Geom g, TileGeom tg,
   const int bw = min(tg.bx, g.nx - X0), bh = min(tg.by, g.ny - Y0);
   const int hx = tile_halo_x(steps), H = bh + 2 * steps;
   const int plane = H * kTileCols;
+  // the shared memory is that of tg.by rows (block-uniform)
+  if (!bounds::ok(bw >= 1 && bh >= 1 && bh <= tg.by && bw + 2 * hx <= kTileCols, bounds::TILE_NODE))
+    return;
   T *A = reinterpret_cast<T *>(tile_smem), *B = A + 9 * plane;
   const int j = 2 * lane, x = X0 - hx + j;
   const bool need = j < bw + 2 * hx;
   auto wrap_y = [&](int y) {
     while (y < 0) y += g.ny;
     while (y >= g.ny) y -= g.ny;
-    return y;
+    return bounds::ck(y, g.ny, bounds::TILE_NODE);
   };
   // the pair's nodes, each taken periodically, and which of them the source
   // is (-1: none)
   int xa = x;
   while (xa < 0) xa += g.nx;
   while (xa >= g.nx) xa -= g.nx;
+  xa = bounds::ck(xa, g.nx, bounds::TILE_NODE);
   const int xb = xa + 1 == g.nx ? 0 : xa + 1;
   const bool vec = xa + 1 < g.nx && (xa & 1) == 0;
   const int at = FORCED ? (xa == sx ? 0 : (xb == sx ? 1 : -1)) : -1;
@@ -545,7 +552,10 @@ k_step_tile(const T *__restrict__ src, T *__restrict__ dst, Geom g, TileGeom tg,
       if (s < steps) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) tile_store<T>(B + i * plane + r * kTileCols + j, f[i]);
-      } else if (j >= hx && j < hx + bw) {
+      } else if (j >= hx && j < hx + bw &&
+                 bounds::ok(Y0 + r - steps >= 0 && Y0 + r - steps < g.ny && x >= 0 &&
+                                x + 2 <= g.pitch,
+                            bounds::TILE_NODE)) {
         // an odd row's last pair also writes its first padding column
         T *o = dst + (long long)(Y0 + r - steps) * g.rstride + x;
 #pragma unroll
