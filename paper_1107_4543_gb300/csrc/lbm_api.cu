@@ -247,6 +247,20 @@ static cudaError_t launch_one(lbm_ctx *h, int from, cudaStream_t st) {
   return launch_step_dev(h->L, src, dst, st, h->block, h->L.variant);
 }
 
+// Whether the stream's owner is capturing it into a graph of their own.
+// Lattices in tiles and rows take single steps there: every step then changes
+// the buffer, so a captured call of an even number of steps can be replayed
+// (one launch of 6 steps would start from the same buffer each time), and
+// nothing of a forced call is read from the host after it returns.
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return s != cudaStreamCaptureStatusNone;
+}
+
 // one launch of `steps` steps (next_steps) from buffer `from` into the other
 static cudaError_t launch_some(lbm_ctx *h, int from, int steps, cudaStream_t st,
                                const float *forced = nullptr) {
@@ -909,12 +923,14 @@ int lbm_step(lbm_handle h, long n) {
   REQUIRE(!h->slab || n <= 1, "a slab takes one step between halo exchanges");
   REQUIRE(h->batch == nullptr, "lattice is a batch member; step the batch");
   DevGuard g(h->device);
+  const bool singly = h->L.plan != PLAN_SINGLE && capturing(h->stream);
   // the launch variants belong to the single-step kernel
-  if (n > 0 && (h->L.plan == PLAN_SINGLE || n == 1 || (h->src_on && h->L.plan == PLAN_ROWS))) {
+  if (n > 0 && !singly &&
+      (h->L.plan == PLAN_SINGLE || n == 1 || (h->src_on && h->L.plan == PLAN_ROWS))) {
     int rc = maybe_autotune(h);
     if (rc != LBM_OK) return rc;
   }
-  if (h->src_on && h->L.plan == PLAN_TILE) return step_forced_tile(h, n);
+  if (h->src_on && h->L.plan == PLAN_TILE && !singly) return step_forced_tile(h, n);
   if (h->src_on) {
     // The forcing changes every step.  Runs of kSrcGraph steps from buffer 0
     // replay a captured graph after the host uploads that run's forcing
@@ -926,7 +942,7 @@ int lbm_step(lbm_handle h, long n) {
       host_feq_j(rho_t, 0.0, 0.0, fs);
     };
     while (n > 0) {
-      if (h->L.cur == 0 && n >= kSrcGraph) {
+      if (h->L.cur == 0 && n >= kSrcGraph && !singly) {
         if (!h->src_graph || h->src_gx != h->sx || h->src_gy != h->sy) {
           int rc = capture_src_graph(h);
           if (rc != LBM_OK) return rc;
@@ -952,7 +968,12 @@ int lbm_step(lbm_handle h, long n) {
   }
   while (n > 0) {
     const int G = h->graph ? h->graph_steps : 64;
-    if (h->L.cur == 0 && n >= G) {
+    if (singly) {
+      CK(launch_one(h, h->L.cur, h->stream));
+      h->L.cur ^= 1;
+      n -= 1;
+      h->t += 1;
+    } else if (h->L.cur == 0 && n >= G) {
       if (!h->graph) {
         int rc = capture_graph(h, &h->graph, &h->graph_steps, false);
         if (rc != LBM_OK) return rc;
