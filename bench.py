@@ -82,6 +82,13 @@ def resident_launches(specs, resident, dtype):
     return len({0 if n <= tiny else 1 if n <= pairs else 2 for n in nodes})
 
 
+def clock_mhz(clk):
+    """SM clock of a Clocks.stop() summary: the median under load, else the
+    maximum, else (no samples: a timed region of a few ms) the nominal one."""
+    clk = clk or {}
+    return clk.get("sm_mhz") or clk.get("sm_max_mhz") or 2070.0
+
+
 def alu_record(torch, dtype, mlups, mhz):
     """The collision's operations against the vector units at a clock."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
@@ -537,7 +544,7 @@ def bench_batched(args, L, torch, rank, ws):
                 "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
                 "frac_of": "measured HBM copy rate",
                 "fma": alu_record(torch, bdt, step_nodes * lbm_steps / np.mean(step_ms) / 1e3,
-                                  clk["sm_mhz"] or clk["sm_max_mhz"] or 2070.0),
+                                  clock_mhz(clk)),
                 # ncu DRAM bytes per node and launch of a smaller capture of the
                 # same kernel, scaled to this launch's nodes
                 "traffic": (round(tr["dram_bytes_per_lu"] * step_nodes) if tr else None),
