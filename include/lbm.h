@@ -114,19 +114,22 @@ int lbm_init_field_dev(lbm_handle h, const double *rho_dev,
 #define LBM_INIT_PLANE 2
 int lbm_init_analytic(lbm_handle h, int kind, const double params[8]);
 
-/* lbm_step -- enqueue n >= 0 time steps (one fused pull-stream + collide
- * kernel per step, replayed from a captured CUDA graph in chunks) on the
- * handle's stream and return without waiting.  Errors: LBM_EINVAL (n < 0),
- * LBM_ECUDA (launch failure). */
+/* lbm_step -- enqueue n >= 0 time steps (fused pull-stream + collide kernels
+ * of one or several steps each, lbm_step_plan, replayed from a captured CUDA
+ * graph in chunks) on the handle's stream and return without waiting.
+ * Errors: LBM_EINVAL (n < 0), LBM_ECUDA (launch failure). */
 int lbm_step(lbm_handle h, long n);
 
 /* lbm_set_source -- the acoustic point source of section 5.1: before the
  * collision of every later lbm_step, node (x, y) is set to the equilibrium
  * at rest with density rho0 + amplitude * sin(2 pi t / period), t the
  * lattice time at the start of that step (0 after init).  amplitude = 0
- * removes the source.  Runs of 64 steps from an even step replay a captured
- * graph of (forced node, step) pairs after the host uploads that run's 64
- * forcing values; other steps are launched one by one (same results).  FP16
+ * removes the source.  Lattices in tiles (lbm_step_plan) force the node
+ * inside the kernel, several steps per launch, from values that the host
+ * uploads for each launch or captured graph of about 64 steps.  Elsewhere
+ * runs of 64 steps from an even step replay a captured graph of (forced node,
+ * step) pairs after the host uploads that run's 64 forcing values; other
+ * steps are launched one by one (same results in every form).  FP16
  * storage: a source set before lbm_init_field / lbm_set_populations enters
  * the choice of the storage scale (its node deviates by up to 4/9 of the
  * amplitude).  Errors: LBM_EINVAL (node outside the lattice, period <= 0,
@@ -366,13 +369,13 @@ int lbm_opt_minimize(const lbm_cost_spec *spec, const double sigmas_in[4],
 
 /* ------------------------------------------------------------- batches */
 /* Many independent lattices advanced together (runtime around the step of
- * section 2.1, which the paper states for one lattice): every time step is ONE
- * kernel launch per storage type over a work list of all members (each
- * lattice starts on a block boundary; one record per block gives its
- * lattice, geometry and buffers), and chunks of 64 steps are replayed from a
- * captured CUDA graph; members small enough for one block's shared memory
- * are instead held there for all the steps of a call (lbm_batch_resident),
- * with the same arithmetic.  Members must be deviation-storage lattices
+ * section 2.1, which the paper states for one lattice): ONE kernel launch per
+ * storage type over a work list of all members takes one time step, or three
+ * where that is faster (lbm_batch_plan; one record per block gives its
+ * lattice, geometry and buffers), and chunks of 66 steps are replayed from a
+ * captured CUDA graph; members small enough for shared memory are instead
+ * held there for all the steps of a call (lbm_batch_resident), with the same
+ * arithmetic.  Members must be deviation-storage lattices
  * (LBM_F32DEV, LBM_F16DEV or LBM_BF16DEV) created on the current device,
  * none of them in another batch; they keep their own memory, rates and
  * reference state, and each advances with exactly the arithmetic of
@@ -470,15 +473,15 @@ int lbm_batch_set_variant(lbm_batch b, int variant);
 int lbm_batch_get_variant(lbm_batch b, int *variant);
 /* (runtime; no counterpart in the paper) Which members the batch keeps in
  * shared memory for all the steps of a launch (flags: one int per member, 1
- * for such a member): lattices whose two step buffers of 9 compact planes,
- * 2 x 9 x nx x ny x element bytes, fit one block's shared memory (227 KB on
- * GB300: up to 56 x 56 nodes in FP32, 80 x 80 in FP16 / BF16), unless the
- * environment variable LBM_RESIDENT_BYTES, read when the batch is made,
- * caps that size (0: none).  One thread block per such member runs all the
- * steps of an lbm_batch_step call (or of a server generation) in one launch
- * beside the per-step launches of the other members, reading and writing
- * the member's populations in HBM once; results are bit-identical either
- * way. */
+ * for such a member): lattices whose nine compact planes, nx x ny elements
+ * each, fit one block's shared memory twice (227 KB on GB300: up to 56 x 56
+ * nodes in FP32, 80 x 80 in FP16 / BF16), unless the environment variable
+ * LBM_RESIDENT_BYTES, read when the batch is made, caps those 2 x 9 x nx x ny x
+ * element bytes (0: none).  One thread block per such member runs all the
+ * steps of an lbm_batch_step call (or of a server generation) in place, in
+ * one launch for members of about one size beside the launches of the other
+ * members, reading and writing the member's populations in HBM once; results
+ * are bit-identical either way. */
 int lbm_batch_resident(lbm_batch b, int *flags);
 /* lbm_batch_plan -- as lbm_step_plan for the batch's members of storage type
  * `dtype` that are not resident (lbm_batch_resident): LBM_PLAN_SINGLE or

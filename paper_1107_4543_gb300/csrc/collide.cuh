@@ -7,7 +7,9 @@
 // Eq. eq_noconservative); back-transform f <- f - M^-1 S (m - m^eq) with
 // M^-1 = M^T D^-1, D = diag(9,6,6,36,36,12,12,4,4) (M has orthogonal rows).
 // The 9x9 transforms are unrolled by hand over the nonzero entries
-// (0, +-1, +-2, +-4): no tensor cores, the step is bound by HBM traffic.
+// (0, +-1, +-2, +-4) and need no tensor cores.  Single steps of the 32- and
+// 16-bit types are bound by HBM, several steps per launch by the FMA pipe, the
+// FP64 types by the FP64 pipe.
 #pragma once
 
 namespace lbm {

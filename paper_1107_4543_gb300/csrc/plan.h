@@ -29,7 +29,8 @@ inline bool rows_fit(const Geom &g) {
   return (g.nx % kRowsV == 0 || rows_chunks(g) >= 3) && (double)g.ny * (rows_chunks(g) + 4) < 4e9;
 }
 
-// resident warps per SM of k_step_rows
+// resident warps per SM of k_step_rows; k_rows_batch's FP32 form holds 12 (136
+// registers), which its fitted rate contains
 constexpr int kRowsWarps = 16;
 
 // Work of k_step_rows over a lattice, or summed over a batch's: its tasks and
@@ -56,9 +57,10 @@ inline double rows_us(const RowsWork &w, int esize, int sms, double half = 0.25)
 // The same for a batch (k_rows_batch): its constants come from shared memory,
 // and where it has more than a task or two per slot, short segments fill the
 // tail.
-// Measured / estimated, 128 lattices of 32^2 .. 1024^2: FP32 in segments of 8,
-// 16, 28, 32 rows 91 / 83, 85 / 79, 81 / 77, 81 / 77 us, FP16 83 / 79, 80 /
-// 74, 78 / 73, 79 / 73.
+// The factors were fitted on one batch (rows_batch_margin has others): measured
+// / estimated, 128 lattices of 32^2 .. 1024^2: FP32 in segments of 8, 16, 28, 32
+// rows 91 / 83, 85 / 79, 81 / 77, 81 / 77 us, FP16 83 / 79, 80 / 74, 78 / 73,
+// 79 / 73.
 inline double rows_batch_us(const RowsWork &w, int esize, int sms) {
   return std::max(rows_us(w, esize, sms), 1.15 * rows_us(w, esize, sms, 0.1));
 }

@@ -29,7 +29,7 @@
 namespace lbm {
 
 // 384 threads (12 warps) per member, two blocks per SM at the 80-register
-// cap, no FP32 spills: 1,024 lattices of 32^2 - 56^2 take 4.9 ms for 500 steps
+// cap (4 bytes of FP32 spills): 1,024 lattices of 32^2 - 56^2 take 4.9 ms for 500 steps
 // (512 threads at 64 registers, 100 bytes of spills: 6.5; 320: 5.2; two step
 // buffers, one node per thread, 512 threads: 7.65)
 constexpr int kResidentThreads = 384;
