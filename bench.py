@@ -251,7 +251,7 @@ NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal
 
 
 def traffic_record(kernel):
-    """DRAM bytes per lattice update from the committed ncu summary, or None
+    """DRAM bytes per node and launch from the committed ncu summary, or None
     when the kernel sources changed since it was captured."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
